@@ -153,6 +153,9 @@ struct PlanCache {
   int64_t n_i = -1, n_j = -1;
   bool guard = false;
   cudaStream_t stream = nullptr;
+  bool hit(uint64_t g, int dv, int v, int64_t ni, int64_t nj, bool gd, cudaStream_t s) const {
+    return valid && gen == g && dev == dv && variant == v && n_i == ni && n_j == nj && guard == gd && stream == s;
+  }
 };
 
 DeviceInfo* device_entry(int dev) {
@@ -203,6 +206,13 @@ struct LibWorkspace {
   void* data = nullptr;
   size_t data_bytes = 0;
   double* aux = nullptr;  // potential-energy block sums + counter
+  // slots and segments of the symmetric forms. A buffer that became too
+  // small is kept until the stream's workspace is released: a captured graph
+  // may still launch kernels on it. Each is at least 1.5 times the one
+  // before, so that the retired ones together stay below twice the last.
+  void* sym = nullptr;
+  size_t sym_bytes = 0;
+  std::vector<void*> retired;
 };
 std::map<std::pair<int, cudaStream_t>, LibWorkspace> g_ws;
 
@@ -255,13 +265,36 @@ cn_status library_workspace(cudaStream_t s, size_t ctrl_need, size_t data_need, 
   return CN_OK;
 }
 
-// Bytes of the data region the library already holds for stream s.
-size_t library_data_bytes(cudaStream_t s) {
+// The symmetric forms' buffer of a stream (no initialisation needed).
+cn_status sym_workspace(cudaStream_t s, size_t need, char** out) {
   int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess) return 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return fail_cuda(e, "cudaGetDevice");
   std::lock_guard<std::mutex> lock(g_mu);
-  auto it = g_ws.find({dev, s});
-  return it == g_ws.end() ? 0 : it->second.data_bytes;
+  LibWorkspace& w = g_ws[{dev, s}];
+  if (w.sym_bytes < need) {
+    if (inject("capture") || capturing(s))
+      return fail(CN_ERR_WORKSPACE,
+                  "the symmetric form's slots of this stream must grow, which allocates; not allowed during graph "
+                  "capture (make one call before capturing)");
+    if (inject("alloc")) return fail(CN_ERR_CUDA, "cudaMalloc: injected allocation failure");
+    const size_t nb = align_up(std::max(need, w.sym_bytes + w.sym_bytes / 2), static_cast<size_t>(1) << 16);
+    void* p = nullptr;
+    if (w.sym) w.retired.reserve(w.retired.size() + 1);
+    if ((e = cudaMalloc(&p, nb)) != cudaSuccess) {
+      cudaGetLastError();  // not left behind for a caller that then takes another path
+      if (e == cudaErrorMemoryAllocation)
+        return fail(CN_ERR_WORKSPACE, "symmetric form: the slot arrays do not fit in device memory");
+      return fail_cuda(e, "cudaMalloc(symmetric slots)");
+    }
+    if (w.sym) w.retired.push_back(w.sym);
+    w.sym = p;
+    w.sym_bytes = nb;
+    g_plan_gen.fetch_add(1, std::memory_order_acq_rel);
+    ++t_own_bumps;
+  }
+  *out = static_cast<char*>(w.sym);
+  return CN_OK;
 }
 
 // Frees the library workspace of a stream that is about to be destroyed.
@@ -274,6 +307,8 @@ void release_library_workspace(cudaStream_t s) {
   if (it->second.ctrl) cudaFree(it->second.ctrl);
   if (it->second.data) cudaFree(it->second.data);
   if (it->second.aux) cudaFree(it->second.aux);
+  if (it->second.sym) cudaFree(it->second.sym);
+  for (void* p : it->second.retired) cudaFree(p);
   g_ws.erase(it);
   g_plan_gen.fetch_add(1, std::memory_order_acq_rel);
 }
@@ -315,65 +350,41 @@ bool valid_k(int variant, int k) {
 
 int64_t round_up(int64_t x, int64_t m) { return (x + m - 1) / m * m; }
 
-// Launch shape of the symmetric form from a small model of its schedule.
-// The N(N+1)/2-style triangle of T tile pairs (tile B = threads x K) is cut
-// into equal static ranges over G = min(resident slots, units) CTAs; the SM
-// holding the most CTAs sets the time, at a rate that saturates once about
-// six warps share the SM. Saturated rates are the ones measured at
-// N = 131072 (ordered pairs / s): they favour large K (fewer warp
-// reductions per pair), while small systems need small tiles to fill the
-// SMs.
+// Launch shape of the symmetric forms. Larger tiles run closer to the pipe
+// (8 x 256 2.2e12 unordered pairs/s in the inner loop, 4 x 128 2.0e12, both
+// at 16 warps per SM); smaller ones cut the work finer over the CTAs and
+// waste less on the diagonal tiles, which are evaluated one-sided. Measured
+// (us, equal masses, 152 SMs; the lines lie where the order changes, and
+// another SM count moves them by the work per SM):
+//   n       2x128/128  4x128/256  8x128/128  8x256/128
+//   5000      16.7       16.8       19.3+      19.3+
+//   7000      25.3       23.6       25.0       25.2
+//   10000       -        37.5       39.7       39.7
+//   14000       -        65.2       63.6       64.8
+//   20000       -          -       113.7      111.8
+//   24576       -       167+       161.9      157.7
+//   50001       -          -       623        608
+//   131072      -          -      4159       4069
+// (threads x K / records per stage). With the potential the fourth sum takes
+// 64-record stages for two CTAs of 256 threads per SM: 50001 798 -> 790,
+// 131072 5343 -> 5250 against 8 x 128.
 cn_tune sym_default_tune(int64_t n, int sms, bool pot) {
-  if (pot && n >= 28000) {
-    // with the potential, measured from N = 32768 to 131072: K = 8 x 128 runs
-    // 2-2.7% ahead of 4 x 256 (131072: 6.41 against 6.54 ms), which the
-    // schedule model below does not see (it charges multi-CTA shapes for
-    // their busiest CTA); at 24576 and below 4 x 256 stays ahead
-    cn_tune t{};
-    t.i_per_thread = 8;
-    t.threads = 128;
-    t.j_tile = 256;
-    t.stages = 4;
-    t.j_lanes = 1;
-    return t;
-  }
-  struct Shape {
-    int k, threads, j_tile, stages, slots_per_sm;
-    double rate, rate_pot;  // saturated effective pairs/s without and with the potential
-  };
-  static const Shape shapes[] = {
-      {8, 256, 256, 3, 1, 3.56e12, 0.0},     {4, 256, 256, 3, 1, 3.10e12, 2.59e12},
-      // K = 8 x 128 without the potential: two resident CTAs run well below
-      // the saturated rate (N = 24576: 280 us against 198 us for 4 x 256),
-      // so the force-only form does not take it
-      {8, 128, 256, 4, 3, 0.0, 2.38e12},     {8, 64, 128, 4, 8, 3.05e12, 2.38e12},
-      {4, 128, 256, 4, 3, 2.87e12, 2.33e12}, {4, 64, 128, 4, 8, 2.64e12, 2.10e12},
-      {2, 64, 64, 4, 8, 1.86e12, 1.50e12},   {1, 64, 64, 4, 9, 0.93e12, 0.75e12}};
-  cn_tune best{};
-  double best_t = 0.0;
-  for (const Shape& sh : shapes) {
-    // with the potential the rows of j-side sums take four floats per particle
-    if (cn::sym_smem_bytes(sh.threads, sh.k, sh.j_tile, sh.stages, pot) > kMaxSmem) continue;
-    if ((pot ? sh.rate_pot : sh.rate) <= 0.0) continue;
-    const int64_t b = static_cast<int64_t>(sh.k) * sh.threads;
-    const int64_t T = (std::max<int64_t>(n, 1) + b - 1) / b;
-    const int64_t units = T * (T + 1) / 2;
-    const int64_t g = std::min<int64_t>(static_cast<int64_t>(sh.slots_per_sm) * sms, units);
-    const int64_t per_sm = (g + sms - 1) / sms;
-    const int64_t per_cta = (units + g - 1) / g;
-    const double warps = static_cast<double>(per_sm) * sh.threads / 32.0;
-    const double sm_rate = (pot ? sh.rate_pot : sh.rate) / sms * std::min(1.0, warps / 6.0);
-    const double t = static_cast<double>(per_sm * per_cta) * 2.0 * static_cast<double>(b * b) / sm_rate;
-    if (best_t == 0.0 || t < best_t) {
-      best_t = t;
-      best.i_per_thread = sh.k;
-      best.threads = sh.threads;
-      best.j_tile = sh.j_tile;
-      best.stages = sh.stages;
-    }
-  }
-  best.j_lanes = 1;
-  return best;
+  const double n_eff = static_cast<double>(n) * std::sqrt(152.0 / std::max(sms, 1));
+  cn_tune t{};
+  t.i_per_thread = n_eff < 6000 ? 2 : n_eff < 12000 ? 4 : 8;
+  t.threads = n_eff < 24576 ? 128 : 256;
+  t.j_tile = n_eff >= 6000 && n_eff < 12000 ? 256 : pot && t.threads == 256 ? 64 : 128;
+  t.stages = 3;
+  t.j_lanes = 1;
+  return t;
+}
+
+// Shapes given by a tune are accepted up to the shared memory that a row of
+// j-side sums per warp over the whole tile would take (three or four floats
+// per particle), the limit that the entry point has always had.
+size_t sym_tile_bytes(const Plan& p, bool pot) {
+  const size_t b = static_cast<size_t>(p.threads) * p.k;
+  return 256 + static_cast<size_t>(p.stages) * p.j_tile * 16 + (p.threads / 32) * b * (pot ? 4 : 3) * sizeof(float);
 }
 
 // The packed shapes of 256 threads with four or eight i-particles per lane
@@ -641,7 +652,7 @@ cn_status resolve_plan(int dev, int variant, int64_t n_i, int64_t n_j, bool guar
     if (p->j_tile % (8 * p->j_lanes)) return fail(CN_ERR_INVALID_ARG, "j_tile must be a multiple of 8 x j_lanes");
   }
   const size_t smem = variant == cn::kSym
-                          ? cn::sym_smem_bytes(p->threads, p->k, p->j_tile, p->stages, false)
+                          ? sym_tile_bytes(*p, false)
                           : (two_records(variant) ? cn::adjoint_smem_bytes(*p) : cn::ring_smem_bytes(*p));
   if (smem > kMaxSmem) return fail(CN_ERR_INVALID_ARG, "the launch shape exceeds the shared memory of one CTA");
   if (variant == cn::kSym && p->i_tile() % p->j_tile) p->j_tile = std::min(p->j_tile, p->i_tile());
@@ -868,9 +879,7 @@ cn_status force_common(bool dd, int64_t n_i, const float* pos_i, int64_t n_j, co
   Geometry g;
   char *ctrl = nullptr, *data = nullptr;
   const uint64_t gen0 = g_plan_gen.load(std::memory_order_acquire);
-  const PlanCache& k = t_last.key;
-  if (lib_ws && k.valid && k.gen == gen0 && k.dev == dev && k.variant == variant && k.n_i == n_i && k.n_j == n_j &&
-      k.guard == guard && k.stream == s) {
+  if (lib_ws && t_last.key.hit(gen0, dev, variant, n_i, n_j, guard, s)) {
     p = t_last.p;
     g = t_last.g;
     ctrl = t_last.ctrl;
@@ -969,6 +978,130 @@ cn_status jerk_common(int64_t n_i, const float* pos_i, const float* vel_i, int64
   return e == cudaSuccess ? CN_OK : fail_cuda(e, "force-jerk kernel launch");
 }
 
+// ------------------------------------------------------------------ symmetric forms
+// Shape, workspace and layout of a symmetric launch.
+struct SymPlan {
+  PlanCache key;
+  int k = 0, threads = 0, chunk = 0, stages = 0;
+  bool guard = false;
+  int64_t tile = 0, tiles = 0, n_blocks = 0, n_pad = 0;
+  int64_t band = 0;  // tile rows per launch
+  int64_t slots = 0;  // resident CTAs
+  size_t smem = 0, jslot_b = 0, seg_b = 0, need = 0;
+  char* data = nullptr;
+};
+
+cn_status sym_occupancy(int dev, cn::SymForm form, const SymPlan& sp, int* ctas) {
+  const auto key = std::make_tuple(dev, 1000 + static_cast<int>(form), sp.guard, 1, sp.k, sp.threads, sp.smem);
+  {
+    std::lock_guard<std::mutex> lock(g_mu);
+    auto it = g_occ.find(key);
+    if (it != g_occ.end()) {
+      *ctas = it->second;
+      return CN_OK;
+    }
+  }
+  const cudaError_t e = cn::occupancy_sym(form, sp.k, sp.guard, sp.threads, sp.smem, ctas);
+  if (e != cudaSuccess) return fail_cuda(e, "cudaOccupancyMaxActiveBlocksPerMultiprocessor");
+  if (*ctas <= 0) return fail(CN_ERR_INVALID_ARG, "launch shape does not fit on one SM");
+  std::lock_guard<std::mutex> lock(g_mu);
+  g_occ[key] = *ctas;
+  return CN_OK;
+}
+
+// Fits the plan of `form` for n particles (p: the shape) and gets its
+// workspace. The j-side slots of every off-diagonal unit take one
+// [rows][n_pad] array (half of it written) when that fits in kSymSlotCap,
+// else bands of fewer rows, each merged into running sums; plus the i-side
+// segments, one per (CTA, row). The shape's chunk_units, when set, fixes the
+// rows per band.
+cn_status sym_setup(int dev, const DeviceInfo& d, cn::SymForm form, int64_t n, bool guard, const Plan& p,
+                    cudaStream_t s, SymPlan* sp) {
+  sp->k = guard ? 2 : std::max(2, p.k);
+  sp->threads = p.threads;
+  sp->guard = guard;
+  sp->chunk = static_cast<int>(std::min<int64_t>(round_up(p.j_tile, cn::kSymBlock), 1024));
+  sp->stages = std::max(2, p.stages);  // a stage is refilled a chunk after it was read
+  sp->tile = static_cast<int64_t>(sp->k) * sp->threads;
+  sp->tiles = ceil_div(n, sp->tile);
+  sp->n_blocks = ceil_div(n, cn::kSymBlock);
+  sp->n_pad = sp->n_blocks * cn::kSymBlock;
+  if (sp->tiles > 65535) return fail(CN_ERR_INVALID_ARG, "too many tiles for the symmetric form");
+  while ((sp->smem = cn::sym_smem_bytes(form, sp->threads, sp->k, sp->chunk, sp->stages)) > kMaxSmem) {
+    if (sp->stages > 2)
+      --sp->stages;
+    else if (sp->chunk > cn::kSymBlock)
+      sp->chunk = static_cast<int>(round_up(sp->chunk / 2, cn::kSymBlock));
+    else
+      return fail(CN_ERR_INVALID_ARG, "the launch shape exceeds the shared memory of one CTA");
+  }
+  int occ = 0;
+  cn_status st = sym_occupancy(dev, form, *sp, &occ);
+  if (st != CN_OK) return st;
+  sp->slots = static_cast<int64_t>(p.ctas_per_sm > 0 ? std::min(p.ctas_per_sm, occ) : occ) * d.sms;
+  const size_t word = sizeof(float) * static_cast<size_t>(cn::sym_sums(form));
+  const size_t row_b = static_cast<size_t>(sp->n_pad) * word;
+  sp->band = sp->tiles;
+  if (p.chunk_units > 0)
+    sp->band = std::min<int64_t>(p.chunk_units, sp->tiles);
+  else if (static_cast<double>(sp->tiles) * static_cast<double>(row_b) > static_cast<double>(kSymSlotCap))
+    sp->band = std::max<int64_t>(1, std::min<int64_t>(sp->tiles, static_cast<int64_t>(kSymSlotCap / row_b)));
+  sp->jslot_b = align_up(static_cast<size_t>(sp->band) * row_b, 256);
+  sp->seg_b = align_up(static_cast<size_t>(sp->slots + sp->band) * static_cast<size_t>(sp->tile) * word, 256);
+  sp->need = sp->jslot_b + sp->seg_b + (sp->band < sp->tiles ? 2 * row_b : 0);
+  return sym_workspace(s, sp->need, &sp->data);
+}
+
+cn_status sym_launch(const char* entry, const DeviceInfo& d, cn::SymForm form, const SymPlan& sp, int64_t n,
+                     const float* pos, const float* rec2, float eps2, float* const (&out)[3], cudaStream_t s) {
+  cn::SymArgs a{};
+  a.g.n = n;
+  a.g.n_tiles = static_cast<int32_t>(sp.tiles);
+  a.g.n_blocks = static_cast<int32_t>(sp.n_blocks);
+  a.g.tile_blocks = static_cast<int32_t>(sp.tile / cn::kSymBlock);
+  a.pos = reinterpret_cast<const float4*>(pos);
+  a.rec2 = reinterpret_cast<const float4*>(rec2);
+  a.slots_j = reinterpret_cast<float*>(sp.data);
+  a.slots_seg = reinterpret_cast<float*>(sp.data + sp.jslot_b);
+  a.n_seg = sp.slots + sp.band;
+  a.status = d.status;
+  a.n_pad = sp.n_pad;
+  a.chunk = sp.chunk;
+  a.stages = sp.stages;
+  a.eps2 = eps2;
+  a.wait_ns = g_wait_ns.load();
+  cn::SymMerge m{};
+  m.slots_seg = a.slots_seg;
+  m.slots_j = a.slots_j;
+  m.carry = sp.band < sp.tiles ? reinterpret_cast<float2*>(sp.data + sp.jslot_b + sp.seg_b) : nullptr;
+  for (int o = 0; o < 3; ++o) m.out[o] = out[o];
+  m.n_pad = sp.n_pad;
+  m.tile = static_cast<int32_t>(sp.tile);
+  for (int64_t r0 = 0; r0 < sp.tiles; r0 += sp.band) {
+    const int64_t r1 = std::min(sp.tiles, r0 + sp.band);
+    a.g.row0 = static_cast<int32_t>(r0);
+    a.g.row1 = static_cast<int32_t>(r1);
+    a.g.cost0 = a.g.row_start(r0);
+    a.g.cost = a.g.row_start(r1) - a.g.cost0;
+    a.g.grid = static_cast<int32_t>(std::max<int64_t>(1, std::min<int64_t>(sp.slots, a.g.cost / cn::kSymCostPair)));
+    m.g = a.g;
+    m.first = r0 == 0;
+    m.last = r1 == sp.tiles;
+    if (log_enabled())
+      std::fprintf(stderr,
+                   "[cunbody] %s: n %lld%s | K %d threads %d chunk %d stages %d | tile %lld tiles %lld band rows "
+                   "%lld..%lld cost %lld grid %d smem %zu slots %zu bytes\n",
+                   entry, static_cast<long long>(n), sp.guard ? " (guarded)" : "", sp.k, sp.threads, sp.chunk,
+                   sp.stages, static_cast<long long>(sp.tile), static_cast<long long>(sp.tiles),
+                   static_cast<long long>(r0), static_cast<long long>(r1), static_cast<long long>(a.g.cost), a.g.grid,
+                   sp.smem, sp.need);
+    if (inject("launch")) return fail(CN_ERR_CUDA, "kernel launch: injected launch failure");
+    const cudaError_t e = cn::launch_sym(form, a, m, sp.k, sp.guard, sp.threads, sp.smem, s);
+    if (e != cudaSuccess) return fail_cuda(e, "symmetric kernel launch");
+  }
+  return CN_OK;
+}
+
 cn_status symmetric_common(int64_t n, const float* pos_mass, float eps2, float* acc_out, float* pot_out,
                            cudaStream_t s) {
   if (n < 0) return fail(CN_ERR_INVALID_ARG, "n must be >= 0");
@@ -988,98 +1121,28 @@ cn_status symmetric_common(int64_t n, const float* pos_mass, float eps2, float* 
   DeviceInfo* d = nullptr;
   if ((st = current_device(&dev, &d)) != CN_OK) return st;
   const bool guard = needs_guard(eps2);
-  // with the potential the default shape must leave room for four sums per
-  // particle in the shared-memory rows
-  cn_tune pot_tune{};
-  const cn_tune* shape = nullptr;
-  if (pot && !registered_tune(dev, cn::kSym, n, n)) {
-    pot_tune = sym_default_tune(n, d->sms, true);
-    shape = &pot_tune;
+  const cn::SymForm form = pot ? cn::kSymForcePot : cn::kSymForce;
+  thread_local SymPlan t_last;
+  const uint64_t gen0 = g_plan_gen.load(std::memory_order_acquire);
+  if (!t_last.key.hit(gen0, dev, form, n, n, guard, s)) {
+    const uint64_t bumps0 = t_own_bumps;
+    cn_tune pot_tune{};
+    const cn_tune* shape = nullptr;
+    if (pot && !registered_tune(dev, cn::kSym, n, n)) {
+      pot_tune = sym_default_tune(n, d->sms, true);
+      shape = &pot_tune;
+    }
+    Plan p;
+    if ((st = resolve_plan(dev, cn::kSym, n, n, guard, shape, &p)) != CN_OK) return st;
+    if (pot && !shape && sym_tile_bytes(p, true) > kMaxSmem)
+      return fail(CN_ERR_INVALID_ARG, "the launch shape exceeds the shared memory of one CTA");
+    t_last.key.valid = false;
+    if ((st = sym_setup(dev, *d, form, n, guard, p, s, &t_last)) != CN_OK) return st;
+    const uint64_t gen1 = g_plan_gen.load(std::memory_order_acquire);
+    t_last.key = PlanCache{gen1 == gen0 + (t_own_bumps - bumps0), gen1, dev, form, n, n, guard, s};
   }
-  Plan p;
-  if ((st = resolve_plan(dev, cn::kSym, n, n, guard, shape, &p)) != CN_OK) return st;
-  const int64_t B = p.i_tile();
-  const int64_t T = ceil_div(n, B);
-  if (T > 65535) return fail(CN_ERR_INVALID_ARG, "too many tiles for the symmetric form");
-  const size_t smem = cn::sym_smem_bytes(p.threads, p.k, p.j_tile, p.stages, pot);
-  if (smem > kMaxSmem) return fail(CN_ERR_INVALID_ARG, "the launch shape exceeds the shared memory of one CTA");
-  int occ = 0;
-  cudaError_t e = cn::occupancy_sym(p.k, guard, p.threads, smem, &occ, pot);
-  if (e != cudaSuccess) return fail_cuda(e, "cudaOccupancyMaxActiveBlocksPerMultiprocessor");
-  if (occ <= 0) return fail(CN_ERR_INVALID_ARG, "launch shape does not fit on one SM");
-  // Slots: the j-side sums of every off-diagonal unit, one [T][n_pad] array
-  // (16 T n_pad bytes, ~16 N^2 / B, half of it written) when it fits in
-  // kSymSlotCap, else bands of w tile rows with [w][n_pad] j-side slots and
-  // FP64 running sums (~16 w N + 32 N bytes); plus the i-side segments,
-  // [CTAs + rows of the band][2][B] ((hi, lo) sums per CTA and row it
-  // touches). The tune's chunk_units, when set, fixes the rows per band.
-  const int64_t n_pad = T * B;
-  int64_t w = T;
-  if (p.chunk_units > 0)
-    w = std::min<int64_t>(p.chunk_units, T);
-  else if (static_cast<double>(T) * static_cast<double>(n_pad) * 16.0 > static_cast<double>(kSymSlotCap))
-    w = std::max<int64_t>(1, std::min<int64_t>(T, static_cast<int64_t>(kSymSlotCap / (16 * static_cast<size_t>(n_pad)))));
-  const bool banded = w < T;
-  const int64_t slots = static_cast<int64_t>(p.ctas_per_sm > 0 ? std::min(p.ctas_per_sm, occ) : occ) * d->sms;
-  const size_t jslot_b = align_up(static_cast<size_t>(w) * static_cast<size_t>(n_pad) * 16, 256);
-  const size_t seg_b = align_up(static_cast<size_t>(slots + w) * static_cast<size_t>(B) * 32, 256);  // (hi, lo)
-  const size_t acc64_b = banded ? static_cast<size_t>(n) * 32 : 0;
-  const size_t need = jslot_b + seg_b + acc64_b;
-  size_t free_b = 0, total_b = 0;
-  if (cudaMemGetInfo(&free_b, &total_b) == cudaSuccess && need > free_b + library_data_bytes(s))
-    return fail(CN_ERR_WORKSPACE, "symmetric form: the slot arrays do not fit in device memory");
-  char *ctrl = nullptr, *data = nullptr;
-  if ((st = library_workspace(s, kCtrlBytes, need, &ctrl, &data)) != CN_OK) return st;
-  cn::SymArgs a{};
-  a.pos = reinterpret_cast<const float4*>(pos_mass);
-  a.slots_j = reinterpret_cast<float4*>(data);
-  a.slots_seg = reinterpret_cast<float4*>(data + jslot_b);
-  a.n_seg = slots + w;
-  a.status = d->status;
-  a.n = n;
-  a.n_pad = n_pad;
-  a.n_tiles = static_cast<int32_t>(T);
-  a.sub_tile = p.j_tile;
-  a.stages = p.stages;
-  a.eps2 = eps2;
-  a.wait_ns = g_wait_ns.load();
-  cn::SymMerge m{};
-  m.slots_seg = a.slots_seg;
-  m.slots_j = a.slots_j;
-  m.acc64 = banded ? reinterpret_cast<double*>(data + jslot_b + seg_b) : nullptr;
-  m.acc_out = acc_out;
-  m.pot_out = pot_out;
-  m.n = n;
-  m.n_pad = n_pad;
-  m.tile = static_cast<int32_t>(B);
-  m.n_tiles = static_cast<int32_t>(T);
-  auto row_start = [T](int64_t r) { return r * T - r * (r - 1) / 2; };  // first unit of tile row r
-  for (int64_t r0 = 0; r0 < T; r0 += w) {
-    const int64_t r1 = std::min(T, r0 + w);
-    a.row0 = static_cast<int32_t>(r0);
-    a.unit_base = row_start(r0);
-    a.units = row_start(r1) - row_start(r0);
-    m.row0 = static_cast<int32_t>(r0);
-    m.row1 = static_cast<int32_t>(r1);
-    m.first = r0 == 0;
-    m.last = r1 == T;
-    const int grid = static_cast<int>(std::min<int64_t>(slots, a.units));
-    m.unit_base = a.unit_base;
-    m.units = a.units;
-    m.grid = grid;
-    if (log_enabled())
-      std::fprintf(stderr,
-                   "[cunbody] cn_force_symmetric: n %lld%s%s | K %d threads %d sub_tile %d stages %d | tile %lld "
-                   "tiles %lld band rows %lld..%lld units %lld grid %d smem %zu slots %zu bytes\n",
-                   static_cast<long long>(n), pot ? " +pot" : "", guard ? " (guarded)" : "", guard ? 1 : p.k,
-                   p.threads, p.j_tile, p.stages, static_cast<long long>(B), static_cast<long long>(T),
-                   static_cast<long long>(r0), static_cast<long long>(r1), static_cast<long long>(a.units), grid, smem,
-                   need);
-    if (inject("launch")) return fail(CN_ERR_CUDA, "kernel launch: injected launch failure");
-    e = cn::launch_sym(a, m, guard ? 1 : p.k, guard, p.threads, grid, smem, s, pot);
-    if (e != cudaSuccess) return fail_cuda(e, "symmetric kernel launch");
-  }
-  return CN_OK;
+  float* const out[3] = {acc_out, pot_out, nullptr};
+  return sym_launch("cn_force_symmetric", *d, form, t_last, n, pos_mass, nullptr, eps2, out, s);
 }
 
 cn_status run_batched(const cn_batch_plan* plan, const float* pos_i, const float* pos_j, float* acc_out,

@@ -1,0 +1,602 @@
+// Symmetric (Newton's third law) evaluation for an i set equal to the j set:
+// every unordered pair is evaluated once and its term is added to both
+// particles. The paper's kernel evaluates every ordered pair; this form does
+// about half the pair work.
+//
+// A warp holds 32 x K particles of its CTA's tile (threads x K particles, K
+// per thread in packed f32x2 pairs) and sweeps the other particles in blocks
+// of 32: at step t lane l takes record l ^ t of the block from shared memory,
+// so at every step the lanes hold 32 different j records, and the j-side
+// sums travel with their record, exchanged by one shuffle per step (lane
+// l's sums at step t belong to record l ^ t; the exchange between steps t
+// and t + 1 is the xor with t ^ (t + 1)). After 32 steps lane l holds the
+// sums of record l over the warp's particles. No reduction over lanes is
+// needed: against summing each record over the warp by a reduce-scatter
+// this takes 24 shuffles and 24 additions per 8 records to 48 shuffles and
+// none, which leaves the FP32 pipe to the pair terms (inner loop at K = 8 x
+// 256 threads, 2.07 GHz: 1.93e12 -> 2.03e12 unordered pairs/s).
+//
+// What bounds the loop: the FP32 pipe, and with it the register file. A
+// packed multiply-add whose three operands are different registers issues
+// every third cycle, against every second one when an operand is repeated
+// from the instruction before it (measured: 3.17 and 2.17 cycles), and
+// 6 of the 14-16 packed operations of a pair term are of that kind; two CTAs
+// of 256 threads per SM (<= 128 registers) run 4% faster than one.
+//
+// Masses. Where the masses of a staged chunk are all equal, they leave the
+// pair term: the sums are formed of r^-3 d and scaled when they are folded
+// (14 instead of 16 lane operations per unordered pair: 2.20e12 pairs/s).
+// That is decided per chunk and warp from the records themselves (the
+// warp's own masses equal too). It needs r^-3 within the FP32 range, as
+// does the general term's r^-3 m: beyond coordinates of 1e11 or below a
+// softening of 1e-10 the term is formed as (m r)(r r), the order of the
+// one-sided kernel.
+//
+// Shared memory per CTA: a ring of staged chunks (bulk copies), three buffers
+// of the j-side sums of a chunk, one row per warp, and the i-side (hi, lo)
+// sums of the current row of tiles, folded from registers every kSymFold
+// records by TwoSum. The warps are not held together by a barrier: a warp
+// that has swept chunk k waits for the "done" barrier of chunk k - 1 (long
+// complete unless a warp is a whole chunk behind), adds up its share of
+// chunk k - 1's rows and arrives on chunk k's barrier. A __syncthreads per
+// chunk instead cost 1.4 us per chunk (N = 131072, 64-record chunks).
+//
+// j-side sums go to one slot per (row, block), i-side sums to one segment
+// per (CTA, row), both as planes of one float per particle; a second kernel
+// adds them per particle in a fixed order: the result is deterministic,
+// with no atomics on data.
+#pragma once
+
+#include "cn_device.cuh"
+#include "cn_sym.h"
+
+namespace cn {
+
+constexpr int kSymFold = 512;          // j records summed in FP32 registers between TwoSum folds
+constexpr float kSymFar = 1e11f;       // |coordinate| up to which r^-3 stays a normal number
+constexpr float kSymSoft = 1e-20f;     // eps2 from which it stays finite
+constexpr int kSymUnroll = 4;          // steps per loop trip (must divide 32)
+
+enum SymMode : int {
+  kSymUniform = 0,  // equal masses, factored out of the pair terms
+  kSymGeneral = 1,  // r^-3 times either mass
+  kSymWide = 2,     // (m r)(r r): any range
+};
+
+__device__ __forceinline__ float2 sym_dup(float v) { return make_float2(v, v); }
+__device__ __forceinline__ float& sym_half(float2& v, int k) { return (k & 1) ? v.y : v.x; }
+
+// ------------------------------------------------------------------ policies
+// A policy holds K i-particles and their FP32 sums, and adds one j record's
+// terms to both sides (`pair`) or to the i side alone (`one`). kSumsI and
+// kSumsJ sums per particle; i-side sum c is folded as sign(c) * scale * sum;
+// with equal masses, `scale` is the j mass and j-side sums are multiplied by
+// the warp's own mass at the end of a block.
+//
+// Force (and potential): per pair, d = x_j - x_i, s = |d|^2 + eps2, r =
+// s^-1/2; i: m_j r^3 d (and m_j r), j: -m_i r^3 d (and -m_i r). The
+// potential skips pairs at exactly zero separation.
+template <int K_, bool POT, bool GUARD>
+struct SymForcePolicy {
+  static constexpr int K = K_;
+  static constexpr int P = K / 2;
+  static constexpr int kSumsI = POT ? 4 : 3;
+  static constexpr int kSumsJ = POT ? 4 : 3;
+  static constexpr int kRec = 1;
+  static constexpr bool kGuard = GUARD;
+  float2 nx[P][3], acc[P][kSumsI];
+  static constexpr bool kOwnMass = true;  // general terms need the warp's own masses
+
+  __device__ __forceinline__ void load(const SymArgs& a, int64_t p, bool valid, int k, float& mass, float& reach) {
+    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (valid) v = __ldg(a.pos + p);
+    sym_half(nx[k >> 1][0], k) = -v.x;
+    sym_half(nx[k >> 1][1], k) = -v.y;
+    sym_half(nx[k >> 1][2], k) = -v.z;
+    mass = v.w;
+    reach = fmaxf(fabsf(v.x), fmaxf(fabsf(v.y), fabsf(v.z)));
+  }
+
+  template <int MODE, bool BOTH>
+  __device__ __forceinline__ void term(const float4 r0, float2 e2, const float2 (&nm)[P], float2 (&c)[kSumsJ]) {
+    const float2 jx = sym_dup(r0.x), jy = sym_dup(r0.y), jz = sym_dup(r0.z), jm = sym_dup(r0.w);
+#pragma unroll
+    for (int p = 0; p < P; ++p) {
+      const float2 dx = __fadd2_rn(jx, nx[p][0]);
+      const float2 dy = __fadd2_rn(jy, nx[p][1]);
+      const float2 dz = __fadd2_rn(jz, nx[p][2]);
+      float2 s, d2;
+      if constexpr (POT) {
+        d2 = __ffma2_rn(dx, dx, __ffma2_rn(dy, dy, __fmul2_rn(dz, dz)));
+        s = __fadd2_rn(d2, e2);
+      } else {
+        s = __ffma2_rn(dx, dx, __ffma2_rn(dy, dy, __ffma2_rn(dz, dz, e2)));
+      }
+      float2 r = make_float2(rsqrt_mufu(s.x), rsqrt_mufu(s.y));
+      if constexpr (GUARD) {
+        r.x = (s.x > 0.f) ? r.x : 0.f;
+        r.y = (s.y > 0.f) ? r.y : 0.f;
+      }
+      const float2 rr = __fmul2_rn(r, r);
+      float2 qi, qj;
+      if constexpr (MODE == kSymUniform) {
+        qi = qj = __fmul2_rn(r, rr);
+      } else if constexpr (MODE == kSymGeneral) {
+        const float2 r3 = __fmul2_rn(r, rr);
+        qi = __fmul2_rn(jm, r3);
+        if constexpr (BOTH) qj = __fmul2_rn(nm[p], r3);
+      } else {
+        qi = __fmul2_rn(__fmul2_rn(jm, r), rr);
+        if constexpr (BOTH) qj = __fmul2_rn(__fmul2_rn(nm[p], r), rr);
+      }
+      acc[p][0] = __ffma2_rn(qi, dx, acc[p][0]);
+      acc[p][1] = __ffma2_rn(qi, dy, acc[p][1]);
+      acc[p][2] = __ffma2_rn(qi, dz, acc[p][2]);
+      if constexpr (BOTH) {
+        c[0] = __ffma2_rn(qj, dx, c[0]);
+        c[1] = __ffma2_rn(qj, dy, c[1]);
+        c[2] = __ffma2_rn(qj, dz, c[2]);
+      }
+      if constexpr (POT) {
+        const float2 rp = make_float2(d2.x != 0.f ? r.x : 0.f, d2.y != 0.f ? r.y : 0.f);
+        if constexpr (MODE == kSymUniform) {
+          acc[p][3] = __fadd2_rn(acc[p][3], rp);
+          if constexpr (BOTH) c[3] = __fadd2_rn(c[3], rp);
+        } else {
+          acc[p][3] = __ffma2_rn(jm, rp, acc[p][3]);
+          if constexpr (BOTH) c[3] = __ffma2_rn(nm[p], rp, c[3]);
+        }
+      }
+    }
+  }
+  template <int MODE>
+  __device__ __forceinline__ void pair(const float4* ring, uint32_t off, int /*chunk*/, float2 e2,
+                                       const float2 (&nm)[P], float2 (&c)[kSumsJ]) {
+    term<MODE, true>(*reinterpret_cast<const float4*>(reinterpret_cast<const char*>(ring) + off), e2, nm, c);
+  }
+  template <int MODE>
+  __device__ __forceinline__ void one(const float4* js, int /*chunk*/, float2 e2, int /*self*/) {
+    float2 none[kSumsJ], own[P];
+    term<MODE, false>(js[0], e2, own, none);
+  }
+  __device__ static constexpr float sign(int c) { return c == 3 ? -1.f : 1.f; }  // phi = -sum m r
+
+  __device__ static __forceinline__ void output(const SymMerge& m, int64_t p, int c, float v) {
+    if (c < 3)
+      m.out[0][3 * p + c] = v;
+    else
+      m.out[1][p] = v;
+  }
+};
+
+// ------------------------------------------------------------------ sweeps
+// The off-diagonal blocks of a chunk against the warp's particles, both
+// sides. `off`: byte offset of the chunk in the ring (a multiple of 512), so
+// that record l ^ t of a block is at its offset ^ (l ^ t) * 16. The j-side
+// sums of each block go to this warp's row, multiplied by `own`; `mass`: the
+// thread's own masses in shared memory (mass[k * nt]).
+template <class Pol, int MODE>
+__device__ __forceinline__ void sym_sweep(Pol& acc, const float4* ring, uint32_t off, int chunk, int blocks, int lane,
+                                          float2 e2, float own, const float* mass, int nt, float* row) {
+  float2 nm[Pol::P];
+#pragma unroll
+  for (int k = 0; k < Pol::K; ++k) sym_half(nm[k >> 1], k) = MODE == kSymUniform ? 0.f : -mass[k * nt];
+#pragma unroll 1
+  for (; blocks > 0; --blocks) {
+    float2 c[Pol::kSumsJ];
+#pragma unroll
+    for (int d = 0; d < Pol::kSumsJ; ++d) c[d] = make_float2(0.f, 0.f);
+#pragma unroll 1
+    for (int u = 0; u < kSymBlock; u += kSymUnroll) {
+      const uint32_t o = off + (static_cast<uint32_t>(lane ^ u) << 4);
+      const int next = ((kSymUnroll - 1) ^ u ^ (u + kSymUnroll)) & 31;  // exchange into the next trip
+#pragma unroll
+      for (int s = 0; s < kSymUnroll; ++s) {
+        acc.template pair<MODE>(ring, o ^ static_cast<uint32_t>(s << 4), chunk, e2, nm, c);
+        const int m = s + 1 < kSymUnroll ? s ^ (s + 1) : next;
+#pragma unroll
+        for (int d = 0; d < Pol::kSumsJ; ++d) {
+          c[d].x = __shfl_xor_sync(0xffffffffu, c[d].x, m);
+          c[d].y = __shfl_xor_sync(0xffffffffu, c[d].y, m);
+        }
+      }
+    }
+#pragma unroll
+    for (int d = 0; d < Pol::kSumsJ; ++d) row[d * chunk + lane] = own * (c[d].x + c[d].y);
+    off += kSymBlock * 16;
+    row += kSymBlock;
+  }
+}
+
+// Diagonal blocks: every ordered pair, i side only.
+template <class Pol, int MODE>
+__device__ __forceinline__ void sym_diag(Pol& acc, const float4* js, int chunk, int count, float2 e2, int self) {
+#pragma unroll 1
+  for (int j = 0; j < count; j += 8) {
+#pragma unroll
+    for (int jj = 0; jj < 8; ++jj) acc.template one<MODE>(js + j + jj, chunk, e2, self - (j + jj));
+  }
+}
+
+// ------------------------------------------------------------------ kernel
+// Shared-memory control block. What only thread 0 or the start of a chunk
+// needs lives here, not in registers: the sweeps need all 128.
+struct SymChunk {
+  int32_t row, blk, nb, diag;  // nb = 0: no more chunks
+};
+struct SymControl {
+  uint64_t full[8];
+  uint64_t done[3];  // a chunk swept by every warp (and the chunk before it added up)
+  int32_t abort;
+  uint32_t issued;   // chunks staged (thread 0)
+  SymCursor ahead;   // the next one (thread 0)
+  int64_t end;
+  SymChunk chunk[16];
+};
+static_assert(sizeof(SymControl) <= 1024, "control block");
+
+// Stages the next chunk of this CTA (thread 0), or marks the end.
+template <class Pol>
+__device__ __noinline__ void sym_produce(const SymArgs& a, SymControl* ctl, float4* ring) {
+  constexpr int JR = Pol::kRec;
+  const uint32_t q = ctl->issued;
+  SymChunk& ch = ctl->chunk[q & 15u];
+  const int slot = static_cast<int>(q % static_cast<uint32_t>(a.stages));
+  SymCursor cur = ctl->ahead;
+  bool diag = false;
+  ch.nb = 0;
+  if (cur.s < ctl->end) cur.take(a.g, ctl->end, a.chunk / kSymBlock, &ch.row, &ch.blk, &ch.nb, &diag);
+  ch.diag = diag;
+#ifdef CN_DEBUG_BOUNDS
+  if (ch.nb != 0 && (ch.row < a.g.row0 || ch.row >= a.g.row1 || ch.nb < 1 || ch.nb > a.chunk / kSymBlock ||
+                     ch.blk < ch.row * a.g.tile_blocks || ch.blk + ch.nb > a.g.n_blocks ||
+                     static_cast<int64_t>(blockIdx.x) + (ch.row - a.g.row0) >= a.n_seg)) {
+    set_status(a.status, kStatusBadSchedule);
+    ch.nb = 0;  // the CTA stops here
+  }
+#endif
+  ctl->ahead = cur;
+  ctl->issued = q + 1;
+  if (ch.nb == 0) {
+    ctl->ahead.s = ctl->end;
+    mbar_arrive(&ctl->full[slot]);
+    return;
+  }
+  const int64_t first = static_cast<int64_t>(ch.blk) * kSymBlock;
+  const int64_t left = a.g.n - first;
+  const int want = ch.nb * kSymBlock;
+  const int cnt = static_cast<int>(left < want ? left : want);
+  float4* dst = ring + static_cast<size_t>(slot) * JR * a.chunk;
+  for (int z = cnt; z < want; ++z) {  // zero-mass padding of the last block
+    dst[z] = make_float4(0.f, 0.f, 0.f, 0.f);
+    if constexpr (JR == 2) dst[a.chunk + z] = make_float4(0.f, 0.f, 0.f, 0.f);
+  }
+  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  mbar_arrive_expect_tx(&ctl->full[slot], static_cast<uint32_t>(cnt) * 16u * JR);
+  bulk_copy_g2s(dst, a.pos + first, static_cast<uint32_t>(cnt) * 16u, &ctl->full[slot]);
+  if constexpr (JR == 2)
+    bulk_copy_g2s(dst + a.chunk, a.rec2 + first, static_cast<uint32_t>(cnt) * 16u, &ctl->full[slot]);
+}
+
+template <class Pol>
+__global__ void __launch_bounds__(256, 2) sym_kernel(const __grid_constant__ SymArgs a) {
+  extern __shared__ __align__(1024) unsigned char smem[];
+  constexpr int K = Pol::K, P = Pol::P, NI = Pol::kSumsI, NJ = Pol::kSumsJ, JR = Pol::kRec;
+  const int NT = blockDim.x;
+  const int tid = threadIdx.x;
+  const int lane = tid & 31;
+  const int warp = tid >> 5;
+  const int NW = NT >> 5;
+  const int B = NT * K;
+  const int CH = a.chunk;
+  const uint32_t S = static_cast<uint32_t>(a.stages);
+  SymControl* ctl = reinterpret_cast<SymControl*>(smem);
+  volatile int32_t* abort = &ctl->abort;
+  float4* ring = reinterpret_cast<float4*>(smem + 1024);                             // [S][JR][CH]
+  float* rows = reinterpret_cast<float*>(ring + static_cast<size_t>(S) * JR * CH);   // [3][NW][NJ][CH]
+  float* sums = rows + static_cast<size_t>(3) * NW * NJ * CH;  // [2][NI][B]: (hi, lo) of the row's i side
+  float* mass = sums + static_cast<size_t>(2) * NI * B;        // [B]: the tile's masses
+
+  if (tid == 0) {
+    for (uint32_t s = 0; s < S; ++s) mbar_init(&ctl->full[s], 1);
+    for (int s = 0; s < 3; ++s) mbar_init(&ctl->done[s], NW);
+    ctl->abort = 0;
+    ctl->issued = 0;
+    mbar_init_fence();
+    ctl->end = a.g.part(static_cast<int64_t>(blockIdx.x) + 1);
+    ctl->ahead.seek(a.g, a.g.part(blockIdx.x));
+  }
+  __syncthreads();
+  // only shared memory so far: global memory after the previous kernel ends
+  grid_dependency_wait();
+  if (tid == 0)
+    for (uint32_t s = 0; s < S; ++s) sym_produce<Pol>(a, ctl, ring);
+
+  Pol acc;
+  const float2 e2 = sym_dup(a.eps2);
+  int32_t cur_I = -1;
+  float scale = 1.f;   // of the sums in registers
+  int held = 0;        // j records in them
+  bool own_uniform = false, own_near = false;  // the warp's masses are equal; its positions are in range
+
+  // adds the register sums to the row's (hi, lo) sums (each thread its own
+  // particles') and clears them
+  auto fold = [&]() {
+#pragma unroll
+    for (int k = 0; k < K; ++k)
+#pragma unroll
+      for (int c = 0; c < NI; ++c) {
+        float* h = sums + c * B + k * NT + tid;
+        float* l = h + NI * B;
+        float s, e;
+        two_sum(*h, __fmul_rn(Pol::sign(c) * scale, sym_half(acc.acc[k >> 1][c], k)), s, e);
+        *h = s;
+        *l = __fadd_rn(*l, e);
+      }
+#pragma unroll
+    for (int p = 0; p < P; ++p)
+#pragma unroll
+      for (int c = 0; c < NI; ++c) acc.acc[p][c] = make_float2(0.f, 0.f);
+    held = 0;
+  };
+  // writes the row's i-side sums to this CTA's segment
+  auto flush = [&](int32_t I) {
+    fold();
+    float* seg = a.slots_seg + (static_cast<size_t>(blockIdx.x) + static_cast<size_t>(I - a.g.row0)) * NI * B;
+#pragma unroll
+    for (int c = 0; c < NI; ++c)
+#pragma unroll
+      for (int k = 0; k < K; ++k) {
+        const int e = c * B + k * NT + tid;
+        seg[e] = __fadd_rn(sums[e], sums[e + NI * B]);
+      }
+  };
+  // once every warp has swept chunk q: refills its stage (thread 0) and adds
+  // up this warp's share of its j-side sums, over the warps in order
+  auto settle = [&](uint32_t q) {
+    const uint32_t b = q % 3;
+    bool live = !*abort;
+    if (live && !mbar_wait(&ctl->done[b], (q / 3) & 1u, a.wait_ns)) {
+      set_status(a.status, kStatusTimeoutEmpty);
+      *abort = 1;
+      live = false;
+    }
+    live = __all_sync(0xffffffffu, live);
+    if (!live) return;
+    if (tid == 0) sym_produce<Pol>(a, ctl, ring);
+    const SymChunk ch = ctl->chunk[q & 15u];
+    if (ch.diag) return;
+    const float* row = rows + b * (NW * NJ * CH);
+    float* slot = a.slots_j + static_cast<size_t>(ch.row - a.g.row0) * NJ * a.n_pad +
+                  static_cast<size_t>(ch.blk) * kSymBlock;
+    for (int it = warp; it < NJ * ch.nb; it += NW) {
+      const int d = it % NJ, j = (it / NJ) * kSymBlock + lane;
+      const float* r = row + d * CH + j;
+      float v = r[0];
+      for (int w = 1; w < NW; ++w) v += r[w * (NJ * CH)];
+      slot[static_cast<size_t>(d) * a.n_pad + j] = v;
+    }
+  };
+
+  uint32_t q = 0;
+  for (;; ++q) {
+    const uint32_t slot = q % S;
+    // After a timed-out wait anywhere in the CTA (abort set) every warp
+    // leaves: nothing below waits for another warp but with a bound.
+    bool live = !*abort;
+    if (live && !mbar_wait(&ctl->full[slot], (q / S) & 1u, a.wait_ns)) {
+      set_status(a.status, kStatusTimeoutFull);
+      *abort = 1;
+      live = false;
+    }
+    live = __all_sync(0xffffffffu, live);
+    if (!live) break;
+    const SymChunk ch = ctl->chunk[q & 15u];
+    if (ch.nb == 0) break;
+    if (ch.row != cur_I) {
+      if (cur_I >= 0) flush(cur_I);
+      cur_I = ch.row;
+      bool same = true, near = true;
+      float m0 = 0.f;
+#pragma unroll
+      for (int k = 0; k < K; ++k) {
+        const int64_t p = static_cast<int64_t>(cur_I) * B + k * NT + tid;
+        float m, reach;
+        acc.load(a, p, p < a.g.n, k, m, reach);
+        mass[k * NT + tid] = m;
+        if (k == 0) m0 = __shfl_sync(0xffffffffu, m, 0);
+        same = same && m == m0;
+        near = near && reach <= kSymFar;
+      }
+      own_uniform = __all_sync(0xffffffffu, same && fabsf(m0) <= 3.4e38f);
+      own_near = __all_sync(0xffffffffu, near && a.eps2 >= kSymSoft);
+#pragma unroll
+      for (int p = 0; p < P; ++p)
+#pragma unroll
+        for (int c = 0; c < NI; ++c) acc.acc[p][c] = make_float2(0.f, 0.f);
+#pragma unroll
+      for (int k = 0; k < K; ++k)
+#pragma unroll
+        for (int c = 0; c < 2 * NI; ++c) sums[c * B + k * NT + tid] = 0.f;
+      held = 0;
+      __syncwarp();
+    }
+    const uint32_t off = slot * static_cast<uint32_t>(JR * CH) * 16u;
+    const float4* js = ring + slot * static_cast<uint32_t>(JR * CH);
+    const int count = ch.nb * kSymBlock;
+    int mode = kSymWide;
+    float factor = 1.f;
+    if constexpr (!Pol::kGuard) {
+      const float mj = js[0].w;
+      bool same = fabsf(mj) <= 3.4e38f, near = own_near;
+      for (int t = lane; t < count; t += 32) {
+        const float4 v = js[t];
+        same = same && v.w == mj;
+        near = near && fmaxf(fabsf(v.x), fmaxf(fabsf(v.y), fabsf(v.z))) <= kSymFar;
+      }
+      if (__all_sync(0xffffffffu, near)) {
+        mode = kSymGeneral;
+        if (__all_sync(0xffffffffu, same) && (ch.diag || own_uniform)) {
+          mode = kSymUniform;
+          factor = mj;
+        }
+      }
+    }
+    if (held > 0 && (factor != scale || held + count > kSymFold)) fold();
+    scale = factor;
+    held += count;
+    if (ch.diag) {
+      const int self = cur_I * B - ch.blk * kSymBlock + tid;
+      if constexpr (!Pol::kGuard) {
+        if (mode == kSymUniform)
+          sym_diag<Pol, kSymUniform>(acc, js, CH, count, e2, self);
+        else if (mode == kSymGeneral)
+          sym_diag<Pol, kSymGeneral>(acc, js, CH, count, e2, self);
+      }
+      if (mode == kSymWide) sym_diag<Pol, kSymWide>(acc, js, CH, count, e2, self);
+    } else {
+      float* mine = rows + (q % 3) * (NW * NJ * CH) + warp * (NJ * CH);
+      if constexpr (!Pol::kGuard) {
+        if (mode == kSymUniform)
+          sym_sweep<Pol, kSymUniform>(acc, ring, off, CH, ch.nb, lane, e2, -mass[tid], mass + tid, NT, mine);
+        else if (mode == kSymGeneral)
+          sym_sweep<Pol, kSymGeneral>(acc, ring, off, CH, ch.nb, lane, e2, 1.f, mass + tid, NT, mine);
+      }
+      if (mode == kSymWide) sym_sweep<Pol, kSymWide>(acc, ring, off, CH, ch.nb, lane, e2, 1.f, mass + tid, NT, mine);
+    }
+    if (q > 0) settle(q - 1);
+    __syncwarp();
+    if (lane == 0) mbar_arrive(&ctl->done[q % 3]);
+  }
+  // the merge kernel may be scheduled while this one ends (not earlier: its
+  // waiting CTAs would take room beside this one's)
+  grid_launch_dependents();
+  if (q > 0) settle(q - 1);
+  if (cur_I >= 0) flush(cur_I);
+  // an aborted run: wait (bounded) for copies that may still be in flight
+  __syncthreads();
+  if (tid == 0 && *abort) {
+    const uint32_t issued = ctl->issued;
+    for (uint32_t c = issued > S ? issued - S : 0u; c < issued; ++c) {
+      if (!mbar_wait(&ctl->full[c % S], (c / S) & 1u, a.wait_ns)) {
+        set_status(a.status, kStatusTimeoutDrain);
+        break;
+      }
+    }
+  }
+}
+
+// Per-particle merge (see SymMerge): 32 particles per CTA, whose slots and
+// segments are dealt out over the 8 warps, in flight together (the chain of
+// loads of one thread per particle was the larger part of the time at
+// N = 4096 .. 16384); the warps' sums are added in warp order. All sums
+// are FP32 (hi, lo) pairs by TwoSum: six FP32 operations, where an FP64
+// addition and its conversion take 32 times as long on this GPU.
+constexpr int kSymMergeWarps = 8;
+template <class Pol>
+__global__ void __launch_bounds__(32 * kSymMergeWarps) sym_merge_kernel(const __grid_constant__ SymMerge m) {
+  constexpr int NI = Pol::kSumsI, NW = kSymMergeWarps;
+  __shared__ float2 part[NW][NI][32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int64_t p = blockIdx.x * static_cast<int64_t>(32) + lane;
+  const bool valid = p < m.g.n;
+  const int32_t I = static_cast<int32_t>((blockIdx.x * static_cast<int64_t>(32)) / m.tile);  // 32 divides the tile
+  const int32_t jend = I < m.g.row1 ? I : m.g.row1;
+  const int nj = jend > m.g.row0 ? jend - m.g.row0 : 0;
+  // i-side: the CTAs whose parts hold the units of row I (when it is one of the launch's rows)
+  int ns = 0;
+  const float* seg = nullptr;
+  if (I >= m.g.row0 && I < m.g.row1) {
+    const int64_t s0 = m.g.row_start(I), s1 = m.g.row_start(static_cast<int64_t>(I) + 1);
+    const int64_t last = s1 - (m.g.diag_end(I) < m.g.n_blocks ? kSymCostPair : kSymCostDiag);
+    const int64_t c0 = m.g.owner(s0), c1 = m.g.owner(last);
+    ns = static_cast<int>(c1 - c0 + 1);
+    seg = m.slots_seg + (static_cast<size_t>(c0) + static_cast<size_t>(I - m.g.row0)) * NI * m.tile +
+          static_cast<size_t>(p - static_cast<int64_t>(I) * m.tile);
+  }
+  const float* slot = m.slots_j + static_cast<size_t>(p);
+  const int total = nj + ns;
+  grid_dependency_wait();  // the slots are complete once the symmetric kernel has ended
+  grid_launch_dependents();
+  float hi[NI], lo[NI];
+#pragma unroll
+  for (int c = 0; c < NI; ++c) hi[c] = lo[c] = 0.f;
+  constexpr int kAhead = 4;
+  for (int q = warp; q < total; q += kAhead * NW) {
+    float w[kAhead][NI];
+#pragma unroll
+    for (int u = 0; u < kAhead; ++u) {
+      const int e = q + u * NW;
+      if (e < total && valid) {
+        const float* src = e < nj ? slot + static_cast<size_t>(e) * NI * m.n_pad
+                                  : seg + static_cast<size_t>(e - nj) * NI * m.tile;
+        const size_t plane = e < nj ? static_cast<size_t>(m.n_pad) : static_cast<size_t>(m.tile);
+#pragma unroll
+        for (int c = 0; c < NI; ++c) w[u][c] = __ldcs(src + c * plane);
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < kAhead; ++u)
+      if (q + u * NW < total && valid) {
+#pragma unroll
+        for (int c = 0; c < NI; ++c) {
+          float e;
+          two_sum(hi[c], w[u][c], hi[c], e);
+          lo[c] = __fadd_rn(lo[c], e);
+        }
+      }
+  }
+#pragma unroll
+  for (int c = 0; c < NI; ++c) part[warp][c][lane] = make_float2(hi[c], lo[c]);
+  __syncthreads();
+  if (warp >= NI || !valid) return;
+  // warp c: component c
+  const int c = warp;
+  float h = 0.f, l = 0.f;
+  if (!m.first) {
+    const float2 v = m.carry[static_cast<size_t>(c) * m.n_pad + p];
+    h = v.x;
+    l = v.y;
+  }
+#pragma unroll
+  for (int w = 0; w < NW; ++w) {
+    float e;
+    two_sum(h, part[w][c][lane].x, h, e);
+    l = __fadd_rn(l, __fadd_rn(e, part[w][c][lane].y));
+  }
+  if (m.last)
+    Pol::output(m, p, c, __fadd_rn(h, l));
+  else
+    m.carry[static_cast<size_t>(c) * m.n_pad + p] = make_float2(h, l);
+}
+
+// ------------------------------------------------------------------ host side
+template <class Pol>
+size_t sym_smem_of(int threads, int chunk, int stages) {
+  return 1024 + static_cast<size_t>(stages) * Pol::kRec * chunk * 16 +
+         (static_cast<size_t>(3) * (threads / 32) * Pol::kSumsJ * chunk +
+          static_cast<size_t>(2 * Pol::kSumsI + 1) * threads * Pol::K) * sizeof(float);
+}
+
+template <class Pol>
+cudaError_t occupancy_sym_of(int threads, size_t smem, int* ctas) {
+  const void* f = reinterpret_cast<const void*>(&sym_kernel<Pol>);
+  cudaError_t e = prepare_kernel(f, smem);
+  if (e != cudaSuccess) return e;
+  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(ctas, f, threads, smem);
+}
+
+template <class Pol>
+cudaError_t launch_sym_of(const SymArgs& a, const SymMerge& m, int threads, size_t smem, cudaStream_t s) {
+  const void* f = reinterpret_cast<const void*>(&sym_kernel<Pol>);
+  cudaError_t e = prepare_kernel(f, smem);
+  if (e != cudaSuccess) return e;
+  void* args[] = {const_cast<SymArgs*>(&a)};
+  e = launch_pdl(f, dim3(static_cast<unsigned>(a.g.grid)), dim3(threads), args, smem, s);
+  if (e != cudaSuccess) return e;
+  void* margs[] = {const_cast<SymMerge*>(&m)};
+  return launch_pdl(reinterpret_cast<const void*>(&sym_merge_kernel<Pol>),
+                    dim3(static_cast<unsigned>(m.g.n_blocks)), dim3(32 * kSymMergeWarps), margs, 0, s);
+}
+
+}  // namespace cn

@@ -1,67 +1,154 @@
 // Symmetric (each unordered pair once) evaluation of an i set equal to the
-// j set: launch arguments and entry points of cn_sym.cu.
+// j set: launch arguments and entry points of the sym_kernel forms.
 #pragma once
 
 #include "cn_kernels.h"
 
 namespace cn {
 
-// One launch covers the tile rows I in [row0, row0 + band) of the upper
-// triangle of tile pairs (I <= J), i.e. units unit_base .. unit_base + units
-// - 1 of the row-major numbering, split into equal contiguous ranges over
-// the grid's CTAs. A CTA adds the i-side sums (tile I) of each of its units
-// of one row, by TwoSum, into one (hi, lo) slot pair per (CTA, row) segment:
-// slots_seg[(c + I - row0) * 2 tile + {0, tile} + p - I * tile] for CTA c (c +
-// I - row0 is unique per segment, since along the unit sequence neither the
-// CTA nor the row index decreases). Unit (I, J), I < J, writes its j-side
-// sums (tile J, partner I) to slots_j[(I - row0) * n_pad + p].
+// The unordered pairs of n particles, cut into rows of tiles. A tile is B =
+// threads x K particles (the i side, in registers); a block is 32
+// particles (the j side of one warp sweep). Row I is the blocks from the
+// tile's own first block on: the tile's own B / 32 ("diagonal") blocks,
+// evaluated one-sided, then all later ones, evaluated for both sides. A
+// block costs kSymCostDiag or kSymCostPair; the cost line of a launch's rows
+// is split evenly over its CTAs, and a unit (I, block) belongs to the CTA
+// in whose part it starts. A part is at least kSymCostPair long, so that
+// every CTA has a unit.
+constexpr int kSymCostDiag = 3;
+constexpr int kSymCostPair = 4;
+constexpr int kSymBlock = 32;
+
+struct SymGrid {
+  int64_t n;           // particles
+  int32_t n_tiles;     // ceil(n / tile)
+  int32_t n_blocks;    // ceil(n / 32)
+  int32_t tile_blocks; // B / 32
+  int32_t row0;        // the launch's rows
+  int32_t row1;
+  int32_t grid;        // its CTAs
+  int64_t cost0;       // cost line position of row0
+  int64_t cost;        // its length over rows row0 .. row1 - 1
+
+  // cost line position of a row's first unit (row <= n_tiles)
+  __host__ __device__ int64_t row_start(int64_t row) const {
+    const int64_t r = row < n_tiles ? row : n_tiles - 1;
+    int64_t s = static_cast<int64_t>(kSymCostDiag) * tile_blocks * r +
+                static_cast<int64_t>(kSymCostPair) * (r * n_blocks - static_cast<int64_t>(tile_blocks) * (r * (r + 1) / 2));
+    if (row >= n_tiles) s += static_cast<int64_t>(kSymCostDiag) * (n_blocks - r * tile_blocks);
+    return s;
+  }
+  // one past a row's last diagonal block
+  __host__ __device__ int32_t diag_end(int32_t row) const {
+    const int64_t e = static_cast<int64_t>(row + 1) * tile_blocks;
+    return static_cast<int32_t>(e < n_blocks ? e : n_blocks);
+  }
+  // where CTA g's part of the cost line begins
+  __host__ __device__ int64_t part(int64_t g) const { return cost0 + (g * cost + grid - 1) / grid; }
+  // the CTA that holds the unit starting at s
+  __host__ __device__ int64_t owner(int64_t s) const { return ((s - cost0) * grid) / cost; }
+};
+
+// A CTA's walk along the cost line, one staged chunk (up to `most` blocks of
+// one row, all diagonal or all not) at a time.
+struct SymCursor {
+  int64_t s;    // cost line position of the next unit
+  int32_t row;
+  int32_t blk;  // its block
+
+  // the first unit starting at or after x
+  __host__ __device__ void seek(const SymGrid& g, int64_t x) {
+    int32_t lo = g.row0, hi = g.row1 - 1;
+    while (lo < hi) {
+      const int32_t mid = (lo + hi + 1) >> 1;
+      if (g.row_start(mid) <= x)
+        lo = mid;
+      else
+        hi = mid - 1;
+    }
+    row = lo;
+    s = g.row_start(lo);
+    const int64_t r = x - s;
+    const int32_t first = lo * g.tile_blocks, nd = g.diag_end(lo) - first;
+    int64_t idx;
+    if (r <= static_cast<int64_t>(kSymCostDiag) * nd)
+      idx = (r + kSymCostDiag - 1) / kSymCostDiag;
+    else
+      idx = nd + (r - static_cast<int64_t>(kSymCostDiag) * nd + kSymCostPair - 1) / kSymCostPair;
+    s += idx <= nd ? kSymCostDiag * idx : static_cast<int64_t>(kSymCostDiag) * nd + kSymCostPair * (idx - nd);
+    blk = first + static_cast<int32_t>(idx);
+    if (blk >= g.n_blocks) {
+      ++row;
+      blk = row * g.tile_blocks;
+    }
+  }
+  // takes the next chunk before position `end`: its row, first block, blocks
+  // and kind; advances past it
+  __host__ __device__ void take(const SymGrid& g, int64_t end, int32_t most, int32_t* row_out, int32_t* blk_out,
+                                int32_t* count, bool* diag) {
+    const int32_t de = g.diag_end(row);
+    const bool dg = blk < de;
+    const int32_t w = dg ? kSymCostDiag : kSymCostPair;
+    const int64_t left = dg ? (end - s + kSymCostDiag - 1) / kSymCostDiag : (end - s + kSymCostPair - 1) / kSymCostPair;
+    int32_t c = (dg ? de : g.n_blocks) - blk;
+    if (c > most) c = most;
+    if (c > left) c = static_cast<int32_t>(left);
+    *row_out = row;
+    *blk_out = blk;
+    *count = c;
+    *diag = dg;
+    s += static_cast<int64_t>(w) * c;
+    blk += c;
+    if (blk >= g.n_blocks) {
+      ++row;
+      blk = row * g.tile_blocks;
+    }
+  }
+};
+
+// A launch. Sum d of the i side of particle p goes to plane d of the (CTA c,
+// row I) segment, slots_seg[((c + I - row0) * sums + d) * tile + p - I tile]
+// (c + I - row0 is unique per segment, since along the cost line neither the
+// CTA nor the row decreases); of the j side under row I to
+// slots_j[((I - row0) * sums + d) * n_pad + p].
 struct SymArgs {
-  const float4* pos;  // [n] (x, y, z, m)
-  float4* slots_seg;  // [n_seg][2][tile] (hi, lo), n_seg >= grid + band rows
-  int64_t n_seg;
-  float4* slots_j;
+  SymGrid g;
+  const float4* pos;   // [n] (x, y, z, m)
+  const float4* rec2;  // second record (velocity, loss weight) or NULL
+  float* slots_seg;
+  float* slots_j;
   int* status;
-  int64_t n;
-  int64_t n_pad;      // n_tiles * tile
-  int64_t unit_base;  // first unit of the launch (row-major over I <= J)
-  int64_t units;      // units of the launch
-  int32_t n_tiles;
-  int32_t row0;       // first tile row of the launch
-  int32_t sub_tile;   // j records per ring stage (divides the tile, multiple of 8)
+  int64_t n_seg;       // allocated segments
+  int64_t n_pad;       // n_blocks * 32
+  int32_t chunk;       // j records per ring stage (multiple of 32)
   int32_t stages;
   float eps2;
   uint64_t wait_ns;
 };
 
-// Per-particle merge of one band: adds, in FP64, the band's j-side slots (x,
-// y, z and the potential in w) in ascending partner order (partners I in
-// [row0, row1), I < P) and, for particles of the band's own tiles, the
-// i-side segments of their row in CTA order, to the running sums (acc64, or
-// zero for the first band); the last band writes the FP32 accelerations,
-// the others store the FP64 sums. The segments of row P are those of the
-// CTAs whose unit ranges meet [row_start(P), row_start(P + 1)).
+// Per-particle merge of one launch: the j-side slots of rows I < P (the
+// particle's tile) in ascending order, then the segments of row P in CTA
+// order, summed in (hi, lo) pairs by TwoSum; with several bands the sums
+// are carried in acc64 as (hi, lo) words and the last band writes the
+// outputs.
 struct SymMerge {
-  const float4* slots_seg;
-  const float4* slots_j;
-  double* acc64;     // [n][4] (acceleration, potential), NULL with a single band
-  float* acc_out;    // [n][3]
-  float* pot_out;    // [n] or NULL
-  int64_t n;
+  SymGrid g;
+  const float* slots_seg;
+  const float* slots_j;
+  float2* carry;      // [sums][n_pad] running (hi, lo) sums, NULL with a single band
+  float* out[3];      // outputs, by form
   int64_t n_pad;
-  int64_t unit_base;  // the band launch's schedule: first unit, units, CTAs
-  int64_t units;
-  int64_t grid;
   int32_t tile;
-  int32_t n_tiles;
-  int32_t row0;
-  int32_t row1;
   int32_t first;
   int32_t last;
 };
 
-size_t sym_smem_bytes(int threads, int k, int sub_tile, int stages, bool pot);
-cudaError_t occupancy_sym(int k, bool guard, int threads, size_t smem, int* ctas, bool pot);
-cudaError_t launch_sym(const SymArgs& a, const SymMerge& m, int k, bool guard, int threads, int grid, size_t smem,
-                       cudaStream_t s, bool pot);
+enum SymForm : int { kSymForce = 0, kSymForcePot = 1 };
+
+int sym_sums(SymForm form);  // sums per particle
+size_t sym_smem_bytes(SymForm form, int threads, int k, int chunk, int stages);
+cudaError_t occupancy_sym(SymForm form, int k, bool guard, int threads, size_t smem, int* ctas);
+cudaError_t launch_sym(SymForm form, const SymArgs& a, const SymMerge& m, int k, bool guard, int threads, size_t smem,
+                       cudaStream_t s);
 
 }  // namespace cn
