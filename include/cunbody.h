@@ -117,7 +117,7 @@ typedef struct cn_tune {
     int32_t ctas_per_sm;  /* resident CTAs per SM to launch (0 = occupancy maximum)               */
     int32_t chunk_units;  /* 0 = static schedule (equal share per CTA); > 0 = dynamic queue chunks
                              of this many (i-tile x j-tile) units. Symmetric form: tile rows per
-                             band (0 = one band while its slots fit in 2 GiB, else bands)       */
+                             band (0 = one band while its slots fit in 512 MiB, else bands)     */
     int32_t j_lanes;      /* single-system FP32, per-i-softening, force-jerk and adjoint forms:
                              lanes sharing the thread's i-particles (1, 2, 4, ..., 32; needs
                              j_tile a multiple of 8 x j_lanes; i_per_thread up to 8 for the
@@ -141,6 +141,12 @@ typedef struct cn_tune {
  * Section 2.2.2, Eq. 2); partial sums of i-tiles split across CTAs are
  * merged in FP64 in a fixed order, so results are bitwise reproducible for
  * a given launch shape.
+ * One set against itself (pos_i == pos_mass_j, n_i == n_j, more than 4096
+ * particles on a GB300, eps2 of normal size, no tune registered for the size
+ * class) takes the kernel of cn_force_symmetric: every unordered pair once,
+ * the same accuracy, and its slots in the library workspace. Where those
+ * cannot be allocated (memory, or a capture before which no such call was
+ * made on the stream) the call takes the one-sided kernel.
  */
 CN_API cn_status cn_force(int64_t n_i, const float *pos_i, int64_t n_j, const float *pos_mass_j, float eps2,
                    float *acc_out, float *pot_out, cn_stream stream);
@@ -151,7 +157,9 @@ CN_API cn_status cn_force(int64_t n_i, const float *pos_i, int64_t n_j, const fl
  * control head (queue words and split-tile arrival counters) with one
  * cudaMemsetAsync on `stream` before the kernel. No allocation happens
  * inside this call. Calls sharing a workspace must not overlap in time on
- * the device. */
+ * the device. For one set against itself (see cn_force) the bytes asked for
+ * hold the symmetric form's slots; a smaller workspace that is large enough
+ * for the one-sided kernel is accepted and takes that kernel. */
 CN_API cn_status cn_force_ws(int64_t n_i, const float *pos_i, int64_t n_j, const float *pos_mass_j, float eps2,
                       float *acc_out, float *pot_out, void *workspace, size_t ws_bytes, cn_stream stream);
 
@@ -225,7 +233,8 @@ CN_API cn_status cn_force_noalloc(int64_t n_i, const float *pos_i, int64_t n_j, 
  *   pos_mass_j, acc_out, pot_out, stream: as cn_force.
  * Same kernels and launch shapes as cn_force (tuned under
  * CN_VARIANT_F32_EPS_I / _POT), always with the s = 0 guard; with every
- * eps2_i equal to one value the results are bitwise those of cn_force.
+ * eps2_i equal to one value the results are bitwise those of cn_force's
+ * one-sided kernel.
  * Errors as cn_force.
  */
 CN_API cn_status cn_force_eps_i(int64_t n_i, const float *pos_eps_i, int64_t n_j, const float *pos_mass_j,
@@ -235,15 +244,15 @@ CN_API cn_status cn_force_eps_i(int64_t n_i, const float *pos_eps_i, int64_t n_j
  * Accelerations of Eq. 1 for n particles under each other's gravity (i set
  * = j set), evaluating every unordered pair once (Newton's third law: the
  * pair term is added to one particle and subtracted, with the other mass,
- * from the other). Not in the paper, whose kernel evaluates every ordered
- * pair: 16 FP32 lane operations and one MUFU per unordered pair plus a warp
- * reduce-scatter of the j-side sums, against 2 x 12 for the two ordered
- * pairs. The j-side sums of each tile pair and the i-side sums of each
- * (CTA, tile row) segment are merged per particle in FP64 in a fixed order
- * (bitwise reproducible for a given launch shape); accuracy as cn_force.
- * It pays off from about N = 24576 on a GB300 (1.15x cn_force at 24576,
- * 1.29x at 131072); at N = 16384 the two take the same time and below it
- * cn_force is faster (about 1.9x at 8192).
+ * from the other). The paper's kernel evaluates every ordered pair; this one
+ * does 14 FP32 lane operations per unordered pair where the masses of a
+ * stage are equal and 16 otherwise, against 2 x 12 for the two ordered
+ * pairs. The j-side sums of each (row of tiles, block) and the i-side sums of
+ * each (CTA, row) segment are merged per particle in (hi, lo) FP32 pairs in a
+ * fixed order (bitwise reproducible for a given launch shape); accuracy as
+ * cn_force.
+ * cn_force takes this form by itself for a set against itself above 4096
+ * particles; below that the one-sided form is faster.
  *   pos_mass : float[n][4] device records (x, y, z, m), 16-byte aligned
  *   eps2     : softening squared, finite and >= 0 (0: coincident pairs
  *              contribute nothing)
@@ -253,12 +262,13 @@ CN_API cn_status cn_force_eps_i(int64_t n_i, const float *pos_eps_i, int64_t n_j
  * Asynchronous on `stream`; n == 0 is a no-op. Errors: CN_ERR_INVALID_ARG
  * (n < 0, bad eps2, NULL or overlapping buffers, a tune with j_lanes),
  * CN_ERR_MISALIGNED, CN_ERR_CUDA (launch), CN_ERR_WORKSPACE (below).
- * Uses a library workspace of j-side slots, 16 N^2 / B bytes for tiles of
- * B particles (134 MB at N = 131072 with the default 2048-particle tiles,
- * half of it written), plus the i-side segments (32 B per particle of a
- * tile per CTA and row), while the slots fit in 2 GiB; above, the tile rows
- * are processed in bands of w rows (about 16 w N + 32 N bytes, w chosen to
- * fit 2 GiB, or set by the tune's chunk_units), one kernel and one merge
+ * Uses a library workspace of j-side slots, 12 N^2 / B bytes (16 with the
+ * potential) for tiles of B particles (101 MB at N = 131072 with the default
+ * 2048-particle tiles, half of it written), plus the i-side segments (12 or
+ * 16 B per particle of a tile per CTA and row), while the slots fit in 512
+ * MiB; above, the tile rows
+ * are processed in bands of w rows (about 12 w N + 24 N bytes, w chosen to
+ * fit 512 MiB, or set by the tune's chunk_units), one kernel and one merge
  * per band. A banded launch cuts the rows into other segments than a
  * one-band launch, so the two agree to FP32 rounding of the segment sums,
  * not bitwise. CN_ERR_WORKSPACE when even one band cannot be held.

@@ -63,7 +63,7 @@ constexpr size_t kCtrlBytes = 4096;  // queue words and spare control space at t
 constexpr uint64_t kDefaultWaitNs = 2000000000ull;
 constexpr size_t kMaxSmem = 227 * 1024;
 constexpr int32_t kNoIndex = 0;  // stands for the index array of a gathering plan whose lists are all empty
-constexpr size_t kSymSlotCap = static_cast<size_t>(2) << 30;  // symmetric-form slot memory before banding
+constexpr size_t kSymSlotCap = static_cast<size_t>(512) << 20;  // symmetric-form slot memory before banding
 
 thread_local std::string g_last_error;
 std::atomic<uint64_t> g_wait_ns{kDefaultWaitNs};
@@ -831,6 +831,149 @@ cn_status check_records(const float* p, int64_t n, const char* name) {
   return CN_OK;
 }
 
+// ------------------------------------------------------------------ symmetric forms
+// Shape, workspace and layout of a symmetric launch.
+struct SymPlan {
+  PlanCache key;
+  int k = 0, threads = 0, chunk = 0, stages = 0;
+  bool guard = false;
+  int64_t tile = 0, tiles = 0, n_blocks = 0, n_pad = 0;
+  int64_t band = 0;  // tile rows per launch
+  int64_t slots = 0;  // resident CTAs
+  size_t smem = 0, jslot_b = 0, seg_b = 0, need = 0;
+  char* data = nullptr;
+};
+
+cn_status sym_occupancy(int dev, cn::SymForm form, const SymPlan& sp, int* ctas) {
+  const auto key = std::make_tuple(dev, 1000 + static_cast<int>(form), sp.guard, 1, sp.k, sp.threads, sp.smem);
+  {
+    std::lock_guard<std::mutex> lock(g_mu);
+    auto it = g_occ.find(key);
+    if (it != g_occ.end()) {
+      *ctas = it->second;
+      return CN_OK;
+    }
+  }
+  const cudaError_t e = cn::occupancy_sym(form, sp.k, sp.guard, sp.threads, sp.smem, ctas);
+  if (e != cudaSuccess) return fail_cuda(e, "cudaOccupancyMaxActiveBlocksPerMultiprocessor");
+  if (*ctas <= 0) return fail(CN_ERR_INVALID_ARG, "launch shape does not fit on one SM");
+  std::lock_guard<std::mutex> lock(g_mu);
+  g_occ[key] = *ctas;
+  return CN_OK;
+}
+
+// Fits the plan of `form` for n particles (p: the shape); `need` bytes of
+// workspace go into data. The j-side slots of every off-diagonal unit take one
+// [rows][n_pad] array (half of it written) when that fits in kSymSlotCap,
+// else bands of fewer rows, each merged into running sums; plus the i-side
+// segments, one per (CTA, row). The shape's chunk_units, when set, fixes the
+// rows per band.
+cn_status sym_fit(int dev, const DeviceInfo& d, cn::SymForm form, int64_t n, bool guard, const Plan& p, SymPlan* sp) {
+  sp->k = guard ? 2 : std::max(2, p.k);
+  sp->threads = p.threads;
+  sp->guard = guard;
+  sp->chunk = static_cast<int>(std::min<int64_t>(round_up(p.j_tile, cn::kSymBlock), 1024));
+  sp->stages = std::max(2, p.stages);  // a stage is refilled a chunk after it was read
+  sp->tile = static_cast<int64_t>(sp->k) * sp->threads;
+  sp->tiles = ceil_div(n, sp->tile);
+  sp->n_blocks = ceil_div(n, cn::kSymBlock);
+  sp->n_pad = sp->n_blocks * cn::kSymBlock;
+  if (sp->tiles > 65535) return fail(CN_ERR_INVALID_ARG, "too many tiles for the symmetric form");
+  while ((sp->smem = cn::sym_smem_bytes(form, sp->threads, sp->k, sp->chunk, sp->stages)) > kMaxSmem) {
+    if (sp->stages > 2)
+      --sp->stages;
+    else if (sp->chunk > cn::kSymBlock)
+      sp->chunk = static_cast<int>(round_up(sp->chunk / 2, cn::kSymBlock));
+    else
+      return fail(CN_ERR_INVALID_ARG, "the launch shape exceeds the shared memory of one CTA");
+  }
+  int occ = 0;
+  cn_status st = sym_occupancy(dev, form, *sp, &occ);
+  if (st != CN_OK) return st;
+  sp->slots = static_cast<int64_t>(p.ctas_per_sm > 0 ? std::min(p.ctas_per_sm, occ) : occ) * d.sms;
+  const size_t word = sizeof(float) * static_cast<size_t>(cn::sym_sums(form));
+  const size_t row_b = static_cast<size_t>(sp->n_pad) * word;
+  sp->band = sp->tiles;
+  if (p.chunk_units > 0)
+    sp->band = std::min<int64_t>(p.chunk_units, sp->tiles);
+  else if (static_cast<double>(sp->tiles) * static_cast<double>(row_b) > static_cast<double>(kSymSlotCap))
+    sp->band = std::max<int64_t>(1, std::min<int64_t>(sp->tiles, static_cast<int64_t>(kSymSlotCap / row_b)));
+  sp->jslot_b = align_up(static_cast<size_t>(sp->band) * row_b, 256);
+  sp->seg_b = align_up(static_cast<size_t>(sp->slots + sp->band) * static_cast<size_t>(sp->tile) * word, 256);
+  sp->need = sp->jslot_b + sp->seg_b + (sp->band < sp->tiles ? 2 * row_b : 0);
+  return CN_OK;
+}
+
+cn_status sym_launch(const std::string& what, const DeviceInfo& d, cn::SymForm form, const SymPlan& sp, int64_t n,
+                     const float* pos, const float* rec2, float eps2, float* const (&out)[3], cudaStream_t s) {
+  cn::SymArgs a{};
+  a.g.n = n;
+  a.g.n_tiles = static_cast<int32_t>(sp.tiles);
+  a.g.n_blocks = static_cast<int32_t>(sp.n_blocks);
+  a.g.tile_blocks = static_cast<int32_t>(sp.tile / cn::kSymBlock);
+  a.pos = reinterpret_cast<const float4*>(pos);
+  a.rec2 = reinterpret_cast<const float4*>(rec2);
+  a.slots_j = reinterpret_cast<float*>(sp.data);
+  a.slots_seg = reinterpret_cast<float*>(sp.data + sp.jslot_b);
+  a.n_seg = sp.slots + sp.band;
+  a.status = d.status;
+  a.n_pad = sp.n_pad;
+  a.chunk = sp.chunk;
+  a.stages = sp.stages;
+  a.eps2 = eps2;
+  a.wait_ns = g_wait_ns.load();
+  cn::SymMerge m{};
+  m.slots_seg = a.slots_seg;
+  m.slots_j = a.slots_j;
+  m.carry = sp.band < sp.tiles ? reinterpret_cast<float2*>(sp.data + sp.jslot_b + sp.seg_b) : nullptr;
+  for (int o = 0; o < 3; ++o) m.out[o] = out[o];
+  m.n_pad = sp.n_pad;
+  m.tile = static_cast<int32_t>(sp.tile);
+  for (int64_t r0 = 0; r0 < sp.tiles; r0 += sp.band) {
+    const int64_t r1 = std::min(sp.tiles, r0 + sp.band);
+    a.g.row0 = static_cast<int32_t>(r0);
+    a.g.row1 = static_cast<int32_t>(r1);
+    a.g.cost0 = a.g.row_start(r0);
+    a.g.cost = a.g.row_start(r1) - a.g.cost0;
+    a.g.grid = static_cast<int32_t>(std::max<int64_t>(1, std::min<int64_t>(sp.slots, a.g.cost / cn::kSymCostPair)));
+    m.g = a.g;
+    m.first = r0 == 0;
+    m.last = r1 == sp.tiles;
+    if (log_enabled()) {
+      int64_t units = 0;
+      for (int64_t I = r0; I < r1; ++I) units += sp.n_blocks - I * a.g.tile_blocks;
+      std::fprintf(stderr,
+                   "[cunbody] %s%s | symmetric: K %d threads %d chunk %d stages %d | tile %lld tiles %lld band rows "
+                   "%lld..%lld units %lld grid %d smem %zu slots %zu bytes\n",
+                   what.c_str(), sp.guard ? " (guarded)" : "", sp.k, sp.threads, sp.chunk, sp.stages,
+                   static_cast<long long>(sp.tile), static_cast<long long>(sp.tiles), static_cast<long long>(r0),
+                   static_cast<long long>(r1), static_cast<long long>(units), a.g.grid, sp.smem, sp.need);
+    }
+    if (inject("launch")) return fail(CN_ERR_CUDA, "kernel launch: injected launch failure");
+    const cudaError_t e = cn::launch_sym(form, a, m, sp.k, sp.guard, sp.threads, sp.smem, s);
+    if (e != cudaSuccess) return fail_cuda(e, "symmetric kernel launch");
+  }
+  return CN_OK;
+}
+
+// Size from which one particle set against itself (the same pointer as i and
+// j set) takes the symmetric form: just above the split-j band of the
+// smallest systems. Measured (us, one-sided / symmetric): 4096 11.1 / 14.1,
+// 5000 20.5 / 16.7, 8192 36.3 / 27.9, 16384 108 / 78, 131072 5981 / 4080.
+bool sym_pays(int64_t n, int sms) {
+  return n > 4096 && static_cast<double>(n) * std::sqrt(152.0 / std::max(sms, 1)) > 4096.0;
+}
+
+Plan sym_default_plan(int64_t n, int sms, bool pot) {
+  const cn_tune t = sym_default_tune(n, sms, pot);
+  Plan p;
+  p.k = t.i_per_thread;
+  p.threads = t.threads;
+  p.j_tile = t.j_tile;
+  p.stages = t.stages;
+  return p;
+}
+
 // ------------------------------------------------------------------ single-system force
 // eps_i: the softening of each pair is its i-particle's, from the 4th slot
 // of its record (eps2 is not used); the kernels then always take the s = 0
@@ -867,41 +1010,63 @@ cn_status force_common(bool dd, int64_t n_i, const float* pos_i, int64_t n_j, co
   const bool guard = eps_i || needs_guard(eps2);
   const int variant = eps_i ? (pot ? cn::kF32EpsIPot : cn::kF32EpsI)
                             : (dd ? (pot ? cn::kDDPot : cn::kDD) : (pot ? cn::kF32Pot : cn::kF32));
+  // One set against itself: each unordered pair once (the i record's 4th slot
+  // is then the same mass the j side reads).
+  const bool self = !dd && !eps_i && !guard && pos_i == pos_mass_j && n_i == n_j && sym_pays(n_i, d->sms);
   struct Cached {
     PlanCache key;
+    bool sym = false;
+    SymPlan sp;
     Plan p;
     Geometry g;
     char* ctrl = nullptr;
     char* data = nullptr;
   };
   thread_local Cached t_last;
-  Plan p;
-  Geometry g;
-  char *ctrl = nullptr, *data = nullptr;
+  Cached now;
+  const int key = variant + (self ? 64 : 0);
   const uint64_t gen0 = g_plan_gen.load(std::memory_order_acquire);
-  if (lib_ws && t_last.key.hit(gen0, dev, variant, n_i, n_j, guard, s)) {
-    p = t_last.p;
-    g = t_last.g;
-    ctrl = t_last.ctrl;
-    data = t_last.data;
-  } else {
+  const Cached* c = &t_last;
+  if (!(lib_ws && t_last.key.hit(gen0, dev, key, n_i, n_j, guard, s))) {
+    c = &now;
     const uint64_t bumps0 = t_own_bumps;
-    // the per-particle kernels are guarded in every shape, so K is not restricted to 1
-    if ((st = resolve_plan(dev, variant, n_i, n_j, guard && !eps_i, nullptr, &p)) != CN_OK) return st;
-    if ((st = single_geometry(dev, *d, variant, guard, p, n_i, n_j, &g)) != CN_OK) return st;
-    if ((st = launch_workspace(s, g, ws, ws_bytes, lib_ws, &ctrl, &data)) != CN_OK) return st;
+    // the per-particle kernels are guarded in every shape, so K is not
+    // restricted to 1. The one-sided plan is made in any case: it is what is
+    // left when the symmetric form's slots cannot be had, and its kernel is
+    // loaded with it.
+    if ((st = resolve_plan(dev, variant, n_i, n_j, guard && !eps_i, nullptr, &now.p)) != CN_OK) return st;
+    if ((st = single_geometry(dev, *d, variant, guard, now.p, n_i, n_j, &now.g)) != CN_OK) return st;
+    bool wanted = self && !registered_tune(dev, variant, n_i, n_j);
+    const cn::SymForm form = pot ? cn::kSymForcePot : cn::kSymForce;
+    if (wanted) wanted = sym_fit(dev, *d, form, n_i, false, sym_default_plan(n_i, d->sms, pot), &now.sp) == CN_OK;
+    if (wanted && lib_ws) {
+      // not during a capture that would have to allocate, and not without memory
+      now.sym = sym_workspace(s, now.sp.need, &now.sp.data) == CN_OK;
+    } else if (wanted && ws && aligned(ws, 256) && ws_bytes >= std::max(now.sp.need, now.g.ws_bytes)) {
+      now.sym = true;
+      now.sp.data = static_cast<char*>(ws);
+    }
+    if (!now.sym && (st = launch_workspace(s, now.g, ws, ws_bytes, lib_ws, &now.ctrl, &now.data)) != CN_OK) return st;
     // cache only a plan that nothing changed under (another thread's tuning
-    // or workspace change would show as a generation step not our own)
+    // or workspace change would show as a generation step not our own), and
+    // not one that had to do without its slots
     const uint64_t gen1 = g_plan_gen.load(std::memory_order_acquire);
-    if (lib_ws && gen1 == gen0 + (t_own_bumps - bumps0)) {
-      t_last.key = PlanCache{true, gen1, dev, variant, n_i, n_j, guard, s};
-      t_last.p = p;
-      t_last.g = g;
-      t_last.ctrl = ctrl;
-      t_last.data = data;
+    if (lib_ws && now.sym == wanted && gen1 == gen0 + (t_own_bumps - bumps0)) {
+      now.key = PlanCache{true, gen1, dev, key, n_i, n_j, guard, s};
+      t_last = now;
     }
   }
-  PairArgs a = base_args(ctrl, data, g, p, d->status);
+  if (c->sym) {
+    float* const out[3] = {static_cast<float*>(acc_out), static_cast<float*>(pot_out), nullptr};
+    std::string what;
+    if (log_enabled())
+      what = std::string("cn_force: variant ") + variant_name(variant) + " n_i " + std::to_string(n_i) + " n_j " +
+             std::to_string(n_j);
+    return sym_launch(what, *d, pot ? cn::kSymForcePot : cn::kSymForce, c->sp, n_i, pos_i, nullptr, eps2, out, s);
+  }
+  const Plan& p = c->p;
+  const Geometry& g = c->g;
+  PairArgs a = base_args(c->ctrl, c->data, g, p, d->status);
   a.pos_i = reinterpret_cast<const float4*>(pos_i);
   a.pos_j = reinterpret_cast<const float4*>(pos_mass_j);
   a.acc_out = acc_out;
@@ -978,130 +1143,6 @@ cn_status jerk_common(int64_t n_i, const float* pos_i, const float* vel_i, int64
   return e == cudaSuccess ? CN_OK : fail_cuda(e, "force-jerk kernel launch");
 }
 
-// ------------------------------------------------------------------ symmetric forms
-// Shape, workspace and layout of a symmetric launch.
-struct SymPlan {
-  PlanCache key;
-  int k = 0, threads = 0, chunk = 0, stages = 0;
-  bool guard = false;
-  int64_t tile = 0, tiles = 0, n_blocks = 0, n_pad = 0;
-  int64_t band = 0;  // tile rows per launch
-  int64_t slots = 0;  // resident CTAs
-  size_t smem = 0, jslot_b = 0, seg_b = 0, need = 0;
-  char* data = nullptr;
-};
-
-cn_status sym_occupancy(int dev, cn::SymForm form, const SymPlan& sp, int* ctas) {
-  const auto key = std::make_tuple(dev, 1000 + static_cast<int>(form), sp.guard, 1, sp.k, sp.threads, sp.smem);
-  {
-    std::lock_guard<std::mutex> lock(g_mu);
-    auto it = g_occ.find(key);
-    if (it != g_occ.end()) {
-      *ctas = it->second;
-      return CN_OK;
-    }
-  }
-  const cudaError_t e = cn::occupancy_sym(form, sp.k, sp.guard, sp.threads, sp.smem, ctas);
-  if (e != cudaSuccess) return fail_cuda(e, "cudaOccupancyMaxActiveBlocksPerMultiprocessor");
-  if (*ctas <= 0) return fail(CN_ERR_INVALID_ARG, "launch shape does not fit on one SM");
-  std::lock_guard<std::mutex> lock(g_mu);
-  g_occ[key] = *ctas;
-  return CN_OK;
-}
-
-// Fits the plan of `form` for n particles (p: the shape) and gets its
-// workspace. The j-side slots of every off-diagonal unit take one
-// [rows][n_pad] array (half of it written) when that fits in kSymSlotCap,
-// else bands of fewer rows, each merged into running sums; plus the i-side
-// segments, one per (CTA, row). The shape's chunk_units, when set, fixes the
-// rows per band.
-cn_status sym_setup(int dev, const DeviceInfo& d, cn::SymForm form, int64_t n, bool guard, const Plan& p,
-                    cudaStream_t s, SymPlan* sp) {
-  sp->k = guard ? 2 : std::max(2, p.k);
-  sp->threads = p.threads;
-  sp->guard = guard;
-  sp->chunk = static_cast<int>(std::min<int64_t>(round_up(p.j_tile, cn::kSymBlock), 1024));
-  sp->stages = std::max(2, p.stages);  // a stage is refilled a chunk after it was read
-  sp->tile = static_cast<int64_t>(sp->k) * sp->threads;
-  sp->tiles = ceil_div(n, sp->tile);
-  sp->n_blocks = ceil_div(n, cn::kSymBlock);
-  sp->n_pad = sp->n_blocks * cn::kSymBlock;
-  if (sp->tiles > 65535) return fail(CN_ERR_INVALID_ARG, "too many tiles for the symmetric form");
-  while ((sp->smem = cn::sym_smem_bytes(form, sp->threads, sp->k, sp->chunk, sp->stages)) > kMaxSmem) {
-    if (sp->stages > 2)
-      --sp->stages;
-    else if (sp->chunk > cn::kSymBlock)
-      sp->chunk = static_cast<int>(round_up(sp->chunk / 2, cn::kSymBlock));
-    else
-      return fail(CN_ERR_INVALID_ARG, "the launch shape exceeds the shared memory of one CTA");
-  }
-  int occ = 0;
-  cn_status st = sym_occupancy(dev, form, *sp, &occ);
-  if (st != CN_OK) return st;
-  sp->slots = static_cast<int64_t>(p.ctas_per_sm > 0 ? std::min(p.ctas_per_sm, occ) : occ) * d.sms;
-  const size_t word = sizeof(float) * static_cast<size_t>(cn::sym_sums(form));
-  const size_t row_b = static_cast<size_t>(sp->n_pad) * word;
-  sp->band = sp->tiles;
-  if (p.chunk_units > 0)
-    sp->band = std::min<int64_t>(p.chunk_units, sp->tiles);
-  else if (static_cast<double>(sp->tiles) * static_cast<double>(row_b) > static_cast<double>(kSymSlotCap))
-    sp->band = std::max<int64_t>(1, std::min<int64_t>(sp->tiles, static_cast<int64_t>(kSymSlotCap / row_b)));
-  sp->jslot_b = align_up(static_cast<size_t>(sp->band) * row_b, 256);
-  sp->seg_b = align_up(static_cast<size_t>(sp->slots + sp->band) * static_cast<size_t>(sp->tile) * word, 256);
-  sp->need = sp->jslot_b + sp->seg_b + (sp->band < sp->tiles ? 2 * row_b : 0);
-  return sym_workspace(s, sp->need, &sp->data);
-}
-
-cn_status sym_launch(const char* entry, const DeviceInfo& d, cn::SymForm form, const SymPlan& sp, int64_t n,
-                     const float* pos, const float* rec2, float eps2, float* const (&out)[3], cudaStream_t s) {
-  cn::SymArgs a{};
-  a.g.n = n;
-  a.g.n_tiles = static_cast<int32_t>(sp.tiles);
-  a.g.n_blocks = static_cast<int32_t>(sp.n_blocks);
-  a.g.tile_blocks = static_cast<int32_t>(sp.tile / cn::kSymBlock);
-  a.pos = reinterpret_cast<const float4*>(pos);
-  a.rec2 = reinterpret_cast<const float4*>(rec2);
-  a.slots_j = reinterpret_cast<float*>(sp.data);
-  a.slots_seg = reinterpret_cast<float*>(sp.data + sp.jslot_b);
-  a.n_seg = sp.slots + sp.band;
-  a.status = d.status;
-  a.n_pad = sp.n_pad;
-  a.chunk = sp.chunk;
-  a.stages = sp.stages;
-  a.eps2 = eps2;
-  a.wait_ns = g_wait_ns.load();
-  cn::SymMerge m{};
-  m.slots_seg = a.slots_seg;
-  m.slots_j = a.slots_j;
-  m.carry = sp.band < sp.tiles ? reinterpret_cast<float2*>(sp.data + sp.jslot_b + sp.seg_b) : nullptr;
-  for (int o = 0; o < 3; ++o) m.out[o] = out[o];
-  m.n_pad = sp.n_pad;
-  m.tile = static_cast<int32_t>(sp.tile);
-  for (int64_t r0 = 0; r0 < sp.tiles; r0 += sp.band) {
-    const int64_t r1 = std::min(sp.tiles, r0 + sp.band);
-    a.g.row0 = static_cast<int32_t>(r0);
-    a.g.row1 = static_cast<int32_t>(r1);
-    a.g.cost0 = a.g.row_start(r0);
-    a.g.cost = a.g.row_start(r1) - a.g.cost0;
-    a.g.grid = static_cast<int32_t>(std::max<int64_t>(1, std::min<int64_t>(sp.slots, a.g.cost / cn::kSymCostPair)));
-    m.g = a.g;
-    m.first = r0 == 0;
-    m.last = r1 == sp.tiles;
-    if (log_enabled())
-      std::fprintf(stderr,
-                   "[cunbody] %s: n %lld%s | K %d threads %d chunk %d stages %d | tile %lld tiles %lld band rows "
-                   "%lld..%lld cost %lld grid %d smem %zu slots %zu bytes\n",
-                   entry, static_cast<long long>(n), sp.guard ? " (guarded)" : "", sp.k, sp.threads, sp.chunk,
-                   sp.stages, static_cast<long long>(sp.tile), static_cast<long long>(sp.tiles),
-                   static_cast<long long>(r0), static_cast<long long>(r1), static_cast<long long>(a.g.cost), a.g.grid,
-                   sp.smem, sp.need);
-    if (inject("launch")) return fail(CN_ERR_CUDA, "kernel launch: injected launch failure");
-    const cudaError_t e = cn::launch_sym(form, a, m, sp.k, sp.guard, sp.threads, sp.smem, s);
-    if (e != cudaSuccess) return fail_cuda(e, "symmetric kernel launch");
-  }
-  return CN_OK;
-}
-
 cn_status symmetric_common(int64_t n, const float* pos_mass, float eps2, float* acc_out, float* pot_out,
                            cudaStream_t s) {
   if (n < 0) return fail(CN_ERR_INVALID_ARG, "n must be >= 0");
@@ -1137,12 +1178,14 @@ cn_status symmetric_common(int64_t n, const float* pos_mass, float eps2, float* 
     if (pot && !shape && sym_tile_bytes(p, true) > kMaxSmem)
       return fail(CN_ERR_INVALID_ARG, "the launch shape exceeds the shared memory of one CTA");
     t_last.key.valid = false;
-    if ((st = sym_setup(dev, *d, form, n, guard, p, s, &t_last)) != CN_OK) return st;
+    if ((st = sym_fit(dev, *d, form, n, guard, p, &t_last)) != CN_OK) return st;
+    if ((st = sym_workspace(s, t_last.need, &t_last.data)) != CN_OK) return st;
     const uint64_t gen1 = g_plan_gen.load(std::memory_order_acquire);
     t_last.key = PlanCache{gen1 == gen0 + (t_own_bumps - bumps0), gen1, dev, form, n, n, guard, s};
   }
   float* const out[3] = {acc_out, pot_out, nullptr};
-  return sym_launch("cn_force_symmetric", *d, form, t_last, n, pos_mass, nullptr, eps2, out, s);
+  const std::string what = log_enabled() ? "cn_force_symmetric: n " + std::to_string(n) : std::string();
+  return sym_launch(what, *d, form, t_last, n, pos_mass, nullptr, eps2, out, s);
 }
 
 cn_status run_batched(const cn_batch_plan* plan, const float* pos_i, const float* pos_j, float* acc_out,
@@ -1678,6 +1721,25 @@ cn_status force_f32_on_workspace(int64_t n_i, const float* pos_i, int64_t n_j, c
                                  float* acc_out, float* pot_out, void* ws, size_t ws_bytes, cudaStream_t s) {
   return force_common(false, n_i, pos_i, n_j, pos_mass_j, eps2, acc_out, pot_out, ws, ws_bytes, false, s);
 }
+// Workspace bytes of a call of `variant` in its one-sided form.
+size_t one_sided_workspace_bytes(int variant, int64_t n_i, int64_t n_j) {
+  if (n_i <= 0 || n_j <= 0 || variant < kF32 || variant > kF32EpsIPot || variant == kBatched || variant == kBatchedPot ||
+      variant == kSym)
+    return 0;
+  int dev = 0;
+  DeviceInfo* d = nullptr;
+  if (current_device(&dev, &d) != CN_OK) return 0;
+  Plan p;
+  if (resolve_plan(dev, variant, n_i, n_j, false, nullptr, &p) != CN_OK) return 0;
+  Geometry g;
+  if (single_geometry(dev, *d, variant, false, p, n_i, n_j, &g) != CN_OK) return 0;
+  // the guarded (eps2 = 0) shape uses one i-particle per thread: size for the larger of the two
+  Plan pg = p;
+  pg.k = 1;
+  Geometry gg;
+  if (single_geometry(dev, *d, variant, true, pg, n_i, n_j, &gg) != CN_OK) return g.ws_bytes;
+  return std::max(g.ws_bytes, gg.ws_bytes);
+}
 cn_status set_error(cn_status st, const std::string& msg) { return fail(st, msg); }
 
 cn_status fail_nothrow(cn_status st, const char* msg) noexcept {
@@ -1740,22 +1802,20 @@ cn_status cn_force_dd_ws(int64_t n_i, const float* pos_i, int64_t n_j, const flo
 
 size_t cn_workspace_bytes(int variant, int64_t n_i, int64_t n_j) {
   return cn::guard_value<size_t>(0, [&]() -> size_t {
-    if (n_i <= 0 || n_j <= 0 || variant < cn::kF32 || variant > cn::kF32EpsIPot || variant == cn::kBatched ||
-        variant == cn::kBatchedPot || variant == cn::kSym)
-      return 0;
+    const size_t need = cn::one_sided_workspace_bytes(variant, n_i, n_j);
+    if (need == 0 || (variant != cn::kF32 && variant != cn::kF32Pot) || n_i != n_j) return need;
+    // one set against itself: the symmetric form's slots (a smaller buffer
+    // that holds the above is accepted, and takes the one-sided kernel)
     int dev = 0;
     DeviceInfo* d = nullptr;
-    if (current_device(&dev, &d) != CN_OK) return 0;
-    Plan p;
-    if (resolve_plan(dev, variant, n_i, n_j, false, nullptr, &p) != CN_OK) return 0;
-    Geometry g;
-    if (single_geometry(dev, *d, variant, false, p, n_i, n_j, &g) != CN_OK) return 0;
-    // the guarded (eps2 = 0) shape uses one i-particle per thread: size for the larger of the two
-    Plan pg = p;
-    pg.k = 1;
-    Geometry gg;
-    if (single_geometry(dev, *d, variant, true, pg, n_i, n_j, &gg) != CN_OK) return g.ws_bytes;
-    return std::max(g.ws_bytes, gg.ws_bytes);
+    if (current_device(&dev, &d) != CN_OK || !sym_pays(n_i, d->sms) || registered_tune(dev, variant, n_i, n_j))
+      return need;
+    const bool pot = variant == cn::kF32Pot;
+    SymPlan sp;
+    if (sym_fit(dev, *d, pot ? cn::kSymForcePot : cn::kSymForce, n_i, false, sym_default_plan(n_i, d->sms, pot), &sp) !=
+        CN_OK)
+      return need;
+    return std::max(need, sp.need);
   });
 }
 
@@ -2214,6 +2274,7 @@ cn_status cn_autotune(int variant, int64_t n_i, const float* pos_i, int64_t n_j,
     cn_tune best{};
     cn_status result = CN_OK;
     std::vector<cn_tune> cands;
+    bool self = false;
     {
       // the default shape of these sizes first (its j-tile fitted to the
       // schedule, which the grid below does not contain), so that the result
@@ -2223,6 +2284,7 @@ cn_status cn_autotune(int variant, int64_t n_i, const float* pos_i, int64_t n_j,
       cn_status st = current_device(&dev, &d);
       if (st != CN_OK) return st;
       cands.push_back(default_tune(variant, n_i, n_j, d->sms));
+      self = !dd && pos_i == pos_mass_j && n_i == n_j && sym_pays(n_i, d->sms);
     }
     for (int k : ks) {
       if (!valid_k(variant, k)) continue;
@@ -2262,9 +2324,16 @@ cn_status cn_autotune(int variant, int64_t n_i, const float* pos_i, int64_t n_j,
       return force_common(dd, n_i, pos_i, n_j, pos_mass_j, eps2, acc_out, pot ? pot_out : nullptr, nullptr, 0, true,
                           ts);
     };
+    // A set against itself takes the symmetric form (from sym_pays) unless a
+    // tune is registered: that default is timed first, as the candidate
+    // without an entry.
+    if (self) cands.insert(cands.begin(), cands.front());
+    bool untuned = self, best_untuned = false;
     for (const cn_tune& t : cands) {
       if (check_tune(variant, t) != CN_OK) continue;
-      cn_tune_set(variant, n_i, n_j, &t);
+      const bool bare = untuned;
+      untuned = false;
+      cn_tune_set(variant, n_i, n_j, bare ? nullptr : &t);
       cn_status st = call();  // warm-up (and workspace growth)
       if (st == CN_ERR_INVALID_ARG) continue;  // shape does not fit
       if (st != CN_OK) {
@@ -2300,6 +2369,7 @@ cn_status cn_autotune(int variant, int64_t n_i, const float* pos_i, int64_t n_j,
       if (ms < best_ms) {
         best_ms = ms;
         best = t;
+        best_untuned = bare;
       }
     }
     if (own_stream) {
@@ -2317,7 +2387,7 @@ cn_status cn_autotune(int variant, int64_t n_i, const float* pos_i, int64_t n_j,
       cn_tune_set(variant, n_i, n_j, nullptr);
       return fail(CN_ERR_INVALID_ARG, "no candidate launch shape fits");
     }
-    cn_tune_set(variant, n_i, n_j, &best);
+    cn_tune_set(variant, n_i, n_j, best_untuned ? nullptr : &best);
     if (best_out) *best_out = best;
     return CN_OK;
   });

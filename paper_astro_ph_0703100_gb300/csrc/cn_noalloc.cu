@@ -18,6 +18,7 @@
 #include <string>
 
 namespace cn {
+size_t one_sided_workspace_bytes(int variant, int64_t n_i, int64_t n_j);
 cn_status force_f32_on_workspace(int64_t n_i, const float* pos_i, int64_t n_j, const float* pos_mass_j, float eps2,
                                  float* acc_out, float* pot_out, void* ws, size_t ws_bytes, cudaStream_t s);
 cn_status set_error(cn_status st, const std::string& msg);
@@ -95,7 +96,7 @@ cn_status noalloc_call(int64_t n_i, const float* pos_i, int64_t n_j, const float
     // Scratch this problem needs under its launch shape (this also sets the
     // device up on a first call); 0 means the arguments or the device are
     // invalid, which the call below reports.
-    const size_t need = cn_workspace_bytes(pot_out ? CN_VARIANT_F32_POT : CN_VARIANT_F32, n_i, n_j);
+    const size_t need = cn::one_sided_workspace_bytes(pot_out ? CN_VARIANT_F32_POT : CN_VARIANT_F32, n_i, n_j);
     if (need > kStaticScratchBytes)
       return cn::set_error(CN_ERR_WORKSPACE,
                            "cn_force_noalloc: this problem needs " + std::to_string(need) +
