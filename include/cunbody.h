@@ -393,7 +393,11 @@ CN_API cn_status cn_list_plan_capture(cn_batch_plan *plan, const float *pos_i, c
  * of Eq. 1.
  *   pos_mass  : float[n][4]; w : float[n][3] (any 4-byte alignment)
  *   grad_pos  : float[n][3]; grad_mass : float[n] (both written)
- * FP32 pair arithmetic, per-tile FP32 partials, FP64 merge of split tiles.
+ * FP32 pair arithmetic, sums folded by TwoSum every 64 terms. Above 2048
+ * particles (on a GB300, eps2 of normal size, no tune registered) each
+ * unordered pair is evaluated once, as in cn_force_symmetric, with its slots
+ * in the library workspace; where those cannot be allocated, and below, every
+ * ordered pair is, with an FP64 merge of split tiles.
  */
 CN_API cn_status cn_force_adjoint(int64_t n, const float *pos_mass, float eps2, const float *w, float *grad_pos,
                            float *grad_mass, cn_stream stream);
@@ -413,7 +417,11 @@ CN_API cn_status cn_force_adjoint(int64_t n, const float *pos_mass, float eps2, 
  *   acc_out, jerk_out   : float[n_i][3]; pot_out : float[n_i] or NULL
  * All four record arrays 16-byte aligned. FP32 pair arithmetic (27 FP32
  * instructions and one MUFU inverse square root per pair), per-tile FP32
- * partials folded into running sums, FP64 merge of split tiles. The
+ * partials folded into running sums, FP64 merge of split tiles. One set
+ * against itself (pos_i == pos_mass_j and vel_i == vel_j, above 2048 particles
+ * on a GB300, no tune registered) takes each unordered pair once, as in
+ * cn_force_symmetric, with its slots in the library workspace, where those
+ * can be allocated. The
  * appendix hard-wires eps2 = 1/256^2; here it is an argument.
  */
 CN_API cn_status cn_force_jerk(int64_t n_i, const float *pos_i, const float *vel_i, int64_t n_j,

@@ -854,7 +854,7 @@ cn_status sym_occupancy(int dev, cn::SymForm form, const SymPlan& sp, int* ctas)
       return CN_OK;
     }
   }
-  const cudaError_t e = cn::occupancy_sym(form, sp.k, sp.guard, sp.threads, sp.smem, ctas);
+  const cudaError_t e = cn::sym_ops(form).occupancy(sp.k, sp.guard, sp.threads, sp.smem, ctas);
   if (e != cudaSuccess) return fail_cuda(e, "cudaOccupancyMaxActiveBlocksPerMultiprocessor");
   if (*ctas <= 0) return fail(CN_ERR_INVALID_ARG, "launch shape does not fit on one SM");
   std::lock_guard<std::mutex> lock(g_mu);
@@ -869,7 +869,8 @@ cn_status sym_occupancy(int dev, cn::SymForm form, const SymPlan& sp, int* ctas)
 // segments, one per (CTA, row). The shape's chunk_units, when set, fixes the
 // rows per band.
 cn_status sym_fit(int dev, const DeviceInfo& d, cn::SymForm form, int64_t n, bool guard, const Plan& p, SymPlan* sp) {
-  sp->k = guard ? 2 : std::max(2, p.k);
+  const cn::SymOps ops = cn::sym_ops(form);
+  sp->k = guard ? 2 : std::min(ops.max_k, std::max(2, p.k));
   sp->threads = p.threads;
   sp->guard = guard;
   sp->chunk = static_cast<int>(std::min<int64_t>(round_up(p.j_tile, cn::kSymBlock), 1024));
@@ -879,7 +880,7 @@ cn_status sym_fit(int dev, const DeviceInfo& d, cn::SymForm form, int64_t n, boo
   sp->n_blocks = ceil_div(n, cn::kSymBlock);
   sp->n_pad = sp->n_blocks * cn::kSymBlock;
   if (sp->tiles > 65535) return fail(CN_ERR_INVALID_ARG, "too many tiles for the symmetric form");
-  while ((sp->smem = cn::sym_smem_bytes(form, sp->threads, sp->k, sp->chunk, sp->stages)) > kMaxSmem) {
+  while ((sp->smem = ops.smem(sp->threads, sp->k, sp->chunk, sp->stages)) > kMaxSmem) {
     if (sp->stages > 2)
       --sp->stages;
     else if (sp->chunk > cn::kSymBlock)
@@ -891,7 +892,7 @@ cn_status sym_fit(int dev, const DeviceInfo& d, cn::SymForm form, int64_t n, boo
   cn_status st = sym_occupancy(dev, form, *sp, &occ);
   if (st != CN_OK) return st;
   sp->slots = static_cast<int64_t>(p.ctas_per_sm > 0 ? std::min(p.ctas_per_sm, occ) : occ) * d.sms;
-  const size_t word = sizeof(float) * static_cast<size_t>(cn::sym_sums(form));
+  const size_t word = sizeof(float) * static_cast<size_t>(ops.sums);
   const size_t row_b = static_cast<size_t>(sp->n_pad) * word;
   sp->band = sp->tiles;
   if (p.chunk_units > 0)
@@ -950,27 +951,50 @@ cn_status sym_launch(const std::string& what, const DeviceInfo& d, cn::SymForm f
                    static_cast<long long>(r1), static_cast<long long>(units), a.g.grid, sp.smem, sp.need);
     }
     if (inject("launch")) return fail(CN_ERR_CUDA, "kernel launch: injected launch failure");
-    const cudaError_t e = cn::launch_sym(form, a, m, sp.k, sp.guard, sp.threads, sp.smem, s);
+    const cudaError_t e = cn::sym_ops(form).launch(a, m, sp.k, sp.guard, sp.threads, sp.smem, s);
     if (e != cudaSuccess) return fail_cuda(e, "symmetric kernel launch");
   }
   return CN_OK;
 }
 
 // Size from which one particle set against itself (the same pointer as i and
-// j set) takes the symmetric form: just above the split-j band of the
-// smallest systems. Measured (us, one-sided / symmetric): 4096 11.1 / 14.1,
-// 5000 20.5 / 16.7, 8192 36.3 / 27.9, 16384 108 / 78, 131072 5981 / 4080.
-bool sym_pays(int64_t n, int sms) {
-  return n > 4096 && static_cast<double>(n) * std::sqrt(152.0 / std::max(sms, 1)) > 4096.0;
+// j set) takes the symmetric form: just above the one-launch split-j shapes
+// of the smallest systems, which merge nothing. Measured (us, one-sided /
+// symmetric): force 4096 11.1 / 14.1, 5000 20.5 / 16.7, 16384 108 / 78;
+// force + jerk + potential 2048 10.4 / 12.1, 3000 31.2 / 16.8, 16384 271 /
+// 178; adjoint 2048 12.3 / 14.4, 3000 34.9 / 18.5, 16384 284 / 174.
+bool sym_pays(cn::SymForm form, int64_t n, int sms) {
+  const int64_t from = form == cn::kSymForce || form == cn::kSymForcePot ? 4096 : 2048;
+  return n > from && static_cast<double>(n) * std::sqrt(152.0 / std::max(sms, 1)) > static_cast<double>(from);
 }
 
-Plan sym_default_plan(int64_t n, int sms, bool pot) {
-  const cn_tune t = sym_default_tune(n, sms, pot);
+// Launch shape of a symmetric form (the force: sym_default_tune). The jerk's
+// eight particles per thread (248 registers, one CTA of 256 per SM) share
+// the 14 shuffles of a step among twice the pairs: with the potential 65536
+// 2571 us against 2739 for four, 32768 659 / 687, 16384 184 / 178. Eight for
+// the adjoint: 65536 2392 / 2431, 50000 1484 / 1435, so it stays at four.
+// Below, two or four particles in smaller tiles: jerk 4096 21.9 us (2 x 256)
+// / 22.4 (4 x 128), 6000 37.7 / 36.3; adjoint 6000 36.9 (2 x 128) / 39.0 (4 x
+// 128), 10000 81.9 / 77.8, 24576 373 (4 x 128) / 371 (4 x 256).
+Plan sym_default_plan(cn::SymForm form, int64_t n, int sms) {
   Plan p;
-  p.k = t.i_per_thread;
-  p.threads = t.threads;
-  p.j_tile = t.j_tile;
-  p.stages = t.stages;
+  p.stages = 3;
+  if (form == cn::kSymForce || form == cn::kSymForcePot) {
+    const cn_tune t = sym_default_tune(n, sms, form == cn::kSymForcePot);
+    p.k = t.i_per_thread;
+    p.threads = t.threads;
+    p.j_tile = t.j_tile;
+    return p;
+  }
+  const double n_eff = static_cast<double>(n) * std::sqrt(152.0 / std::max(sms, 1));
+  p.j_tile = 128;
+  if (form == cn::kSymAdjoint) {
+    p.k = n_eff < 6500 ? 2 : 4;
+    p.threads = n_eff < 20000 ? 128 : 256;
+  } else {
+    p.k = n_eff < 5000 ? 2 : n_eff < 20000 ? 4 : 8;
+    p.threads = 256;
+  }
   return p;
 }
 
@@ -1012,7 +1036,7 @@ cn_status force_common(bool dd, int64_t n_i, const float* pos_i, int64_t n_j, co
                             : (dd ? (pot ? cn::kDDPot : cn::kDD) : (pot ? cn::kF32Pot : cn::kF32));
   // One set against itself: each unordered pair once (the i record's 4th slot
   // is then the same mass the j side reads).
-  const bool self = !dd && !eps_i && !guard && pos_i == pos_mass_j && n_i == n_j && sym_pays(n_i, d->sms);
+  const bool self = !dd && !eps_i && !guard && pos_i == pos_mass_j && n_i == n_j && sym_pays(cn::kSymForce, n_i, d->sms);
   struct Cached {
     PlanCache key;
     bool sym = false;
@@ -1038,7 +1062,7 @@ cn_status force_common(bool dd, int64_t n_i, const float* pos_i, int64_t n_j, co
     if ((st = single_geometry(dev, *d, variant, guard, now.p, n_i, n_j, &now.g)) != CN_OK) return st;
     bool wanted = self && !registered_tune(dev, variant, n_i, n_j);
     const cn::SymForm form = pot ? cn::kSymForcePot : cn::kSymForce;
-    if (wanted) wanted = sym_fit(dev, *d, form, n_i, false, sym_default_plan(n_i, d->sms, pot), &now.sp) == CN_OK;
+    if (wanted) wanted = sym_fit(dev, *d, form, n_i, false, sym_default_plan(form, n_i, d->sms), &now.sp) == CN_OK;
     if (wanted && lib_ws) {
       // not during a capture that would have to allocate, and not without memory
       now.sym = sym_workspace(s, now.sp.need, &now.sp.data) == CN_OK;
@@ -1081,6 +1105,26 @@ cn_status force_common(bool dd, int64_t n_i, const float* pos_i, int64_t n_j, co
   return CN_OK;
 }
 
+// The symmetric plan of a jerk or adjoint call of one set against itself,
+// with its workspace (extra: bytes after its slots, at data + need), or
+// nullptr where the call takes the one-sided kernel: a small set, a
+// registered tune, or no slots to be had (memory, a capture).
+const SymPlan* sym_self_plan(int dev, const DeviceInfo& d, cn::SymForm form, int variant, int64_t n, size_t extra,
+                             cudaStream_t s) {
+  if (!sym_pays(form, n, d.sms)) return nullptr;
+  thread_local SymPlan t_last;
+  const uint64_t gen0 = g_plan_gen.load(std::memory_order_acquire);
+  if (t_last.key.hit(gen0, dev, form, n, n, false, s)) return &t_last;
+  if (registered_tune(dev, variant, n, n)) return nullptr;
+  const uint64_t bumps0 = t_own_bumps;
+  t_last.key.valid = false;
+  if (sym_fit(dev, d, form, n, false, sym_default_plan(form, n, d.sms), &t_last) != CN_OK) return nullptr;
+  if (sym_workspace(s, t_last.need + extra, &t_last.data) != CN_OK) return nullptr;
+  const uint64_t gen1 = g_plan_gen.load(std::memory_order_acquire);
+  t_last.key = PlanCache{gen1 == gen0 + (t_own_bumps - bumps0), gen1, dev, form, n, n, false, s};
+  return &t_last;
+}
+
 cn_status jerk_common(int64_t n_i, const float* pos_i, const float* vel_i, int64_t n_j, const float* pos_mass_j,
                       const float* vel_j, float eps2, float* acc_out, float* jerk_out, float* pot_out,
                       cudaStream_t s) {
@@ -1120,6 +1164,15 @@ cn_status jerk_common(int64_t n_i, const float* pos_i, const float* vel_i, int64
   const bool pot = pot_out != nullptr;
   const bool guard = needs_guard(eps2);
   const int variant = pot ? cn::kJerkPot : cn::kJerk;
+  if (!guard && pos_i == pos_mass_j && vel_i == vel_j && n_i == n_j) {
+    const cn::SymForm form = pot ? cn::kSymJerkPot : cn::kSymJerk;
+    if (const SymPlan* sp = sym_self_plan(dev, *d, form, variant, n_i, 0, s)) {
+      float* const out[3] = {acc_out, jerk_out, pot_out};
+      std::string what;
+      if (log_enabled()) what = std::string("cn_force_jerk: variant ") + variant_name(variant) + " n " + std::to_string(n_i);
+      return sym_launch(what, *d, form, *sp, n_i, pos_i, vel_i, eps2, out, s);
+    }
+  }
   Plan p;
   if ((st = resolve_plan(dev, variant, n_i, n_j, guard, nullptr, &p)) != CN_OK) return st;
   Geometry g;
@@ -1808,13 +1861,11 @@ size_t cn_workspace_bytes(int variant, int64_t n_i, int64_t n_j) {
     // that holds the above is accepted, and takes the one-sided kernel)
     int dev = 0;
     DeviceInfo* d = nullptr;
-    if (current_device(&dev, &d) != CN_OK || !sym_pays(n_i, d->sms) || registered_tune(dev, variant, n_i, n_j))
+    if (current_device(&dev, &d) != CN_OK || !sym_pays(cn::kSymForce, n_i, d->sms) || registered_tune(dev, variant, n_i, n_j))
       return need;
-    const bool pot = variant == cn::kF32Pot;
+    const cn::SymForm form = variant == cn::kF32Pot ? cn::kSymForcePot : cn::kSymForce;
     SymPlan sp;
-    if (sym_fit(dev, *d, pot ? cn::kSymForcePot : cn::kSymForce, n_i, false, sym_default_plan(n_i, d->sms, pot), &sp) !=
-        CN_OK)
-      return need;
+    if (sym_fit(dev, *d, form, n_i, false, sym_default_plan(form, n_i, d->sms), &sp) != CN_OK) return need;
     return std::max(need, sp.need);
   });
 }
@@ -1971,6 +2022,17 @@ cn_status cn_force_adjoint(int64_t n, const float* pos_mass, float eps2, const f
     DeviceInfo* d = nullptr;
     if ((st = current_device(&dev, &d)) != CN_OK) return st;
     const bool guard = needs_guard(eps2);
+    if (!guard) {
+      if (const SymPlan* sp = sym_self_plan(dev, *d, cn::kSymAdjoint, cn::kAdjoint, n, un * 16 + 256, s)) {
+        float* wrec = reinterpret_cast<float*>(sp->data + align_up(sp->need, 256));
+        if (inject("launch")) return fail(CN_ERR_CUDA, "kernel launch: injected launch failure");
+        const cudaError_t e = cn::launch_pack_w(w, reinterpret_cast<float4*>(wrec), n, s);
+        if (e != cudaSuccess) return fail_cuda(e, "weight packing launch");
+        float* const out[3] = {grad_pos, grad_mass, nullptr};
+        const std::string what = log_enabled() ? "cn_force_adjoint: n " + std::to_string(n) : std::string();
+        return sym_launch(what, *d, cn::kSymAdjoint, *sp, n, pos_mass, wrec, eps2, out, s);
+      }
+    }
     Plan p;
     if ((st = resolve_plan(dev, cn::kAdjoint, n, n, guard, nullptr, &p)) != CN_OK) return st;
     Geometry g;
@@ -2284,7 +2346,7 @@ cn_status cn_autotune(int variant, int64_t n_i, const float* pos_i, int64_t n_j,
       cn_status st = current_device(&dev, &d);
       if (st != CN_OK) return st;
       cands.push_back(default_tune(variant, n_i, n_j, d->sms));
-      self = !dd && pos_i == pos_mass_j && n_i == n_j && sym_pays(n_i, d->sms);
+      self = !dd && pos_i == pos_mass_j && n_i == n_j && sym_pays(cn::kSymForce, n_i, d->sms);
     }
     for (int k : ks) {
       if (!valid_k(variant, k)) continue;

@@ -34,7 +34,7 @@
 //
 // Shared memory per CTA: a ring of staged chunks (bulk copies), three buffers
 // of the j-side sums of a chunk, one row per warp, and the i-side (hi, lo)
-// sums of the current row of tiles, folded from registers every kSymFold
+// sums of the current row of tiles, folded from registers every kFold
 // records by TwoSum. The warps are not held together by a barrier: a warp
 // that has swept chunk k waits for the "done" barrier of chunk k - 1 (long
 // complete unless a warp is a whole chunk behind), adds up its share of
@@ -52,7 +52,6 @@
 
 namespace cn {
 
-constexpr int kSymFold = 512;          // j records summed in FP32 registers between TwoSum folds
 constexpr float kSymFar = 1e11f;       // |coordinate| up to which r^-3 stays a normal number
 constexpr float kSymSoft = 1e-20f;     // eps2 from which it stays finite
 constexpr int kSymUnroll = 4;          // steps per loop trip (must divide 32)
@@ -67,11 +66,21 @@ __device__ __forceinline__ float2 sym_dup(float v) { return make_float2(v, v); }
 __device__ __forceinline__ float& sym_half(float2& v, int k) { return (k & 1) ? v.y : v.x; }
 
 // ------------------------------------------------------------------ policies
-// A policy holds K i-particles and their FP32 sums, and adds one j record's
-// terms to both sides (`pair`) or to the i side alone (`one`). kSumsI and
-// kSumsJ sums per particle; i-side sum c is folded as sign(c) * scale * sum;
-// with equal masses, `scale` is the j mass and j-side sums are multiplied by
-// the warp's own mass at the end of a block.
+// A policy holds K i-particles and their FP32 sums (`acc`), and adds one j
+// record's terms to both sides (`pair`) or to the i side alone (`one`):
+//   kSumsI, kSumsJ  sums per particle and side
+//   kRec            float4 words per record (2: a velocity or a loss weight)
+//   kMinBlocks      256-thread CTAs per SM the registers are limited for
+//   kFold           j records summed in FP32 registers between TwoSum folds
+//   kWide           offers the kSymWide terms
+//   kSameMass       equal masses factor out only if the warp's and the
+//                   chunk's are the same
+//   kOwnSign        sign of the warp's own masses handed to `pair`
+//   weight          factor of i-side sum c when it is folded (mass: the
+//                   chunk's mass where the masses are factored out, else 1)
+//   back            factor of j-side sum c at the end of a block (own: the
+//                   particle's own mass there, else 1)
+//   output          where the merged sum c of a particle goes
 //
 // Force (and potential): per pair, d = x_j - x_i, s = |d|^2 + eps2, r =
 // s^-1/2; i: m_j r^3 d (and m_j r), j: -m_i r^3 d (and -m_i r). The
@@ -84,8 +93,12 @@ struct SymForcePolicy {
   static constexpr int kSumsJ = POT ? 4 : 3;
   static constexpr int kRec = 1;
   static constexpr bool kGuard = GUARD;
+  static constexpr int kFold = 512;
+  static constexpr int kMinBlocks = 2;
+  static constexpr bool kWide = true;
+  static constexpr bool kSameMass = false;
+  static constexpr float kOwnSign = -1.f;
   float2 nx[P][3], acc[P][kSumsI];
-  static constexpr bool kOwnMass = true;  // general terms need the warp's own masses
 
   __device__ __forceinline__ void load(const SymArgs& a, int64_t p, bool valid, int k, float& mass, float& reach) {
     float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -155,11 +168,14 @@ struct SymForcePolicy {
     term<MODE, true>(*reinterpret_cast<const float4*>(reinterpret_cast<const char*>(ring) + off), e2, nm, c);
   }
   template <int MODE>
-  __device__ __forceinline__ void one(const float4* js, int /*chunk*/, float2 e2, int /*self*/) {
+  __device__ __forceinline__ void one(const float4* js, int /*chunk*/, float2 e2, int /*self*/, int /*nt*/) {
     float2 none[kSumsJ], own[P];
     term<MODE, false>(js[0], e2, own, none);
   }
-  __device__ static constexpr float sign(int c) { return c == 3 ? -1.f : 1.f; }  // phi = -sum m r
+  __device__ static __forceinline__ float weight(int c, float mass) { return c == 3 ? -mass : mass; }  // phi = -sum m r
+  __device__ static __forceinline__ float back(int /*c*/, int mode, float own) {
+    return mode == kSymUniform ? -own : 1.f;
+  }
 
   __device__ static __forceinline__ void output(const SymMerge& m, int64_t p, int c, float v) {
     if (c < 3)
@@ -173,14 +189,15 @@ struct SymForcePolicy {
 // The off-diagonal blocks of a chunk against the warp's particles, both
 // sides. `off`: byte offset of the chunk in the ring (a multiple of 512), so
 // that record l ^ t of a block is at its offset ^ (l ^ t) * 16. The j-side
-// sums of each block go to this warp's row, multiplied by `own`; `mass`: the
+// sums of each block go to this warp's row; `mass`: the
 // thread's own masses in shared memory (mass[k * nt]).
 template <class Pol, int MODE>
 __device__ __forceinline__ void sym_sweep(Pol& acc, const float4* ring, uint32_t off, int chunk, int blocks, int lane,
-                                          float2 e2, float own, const float* mass, int nt, float* row) {
+                                          float2 e2, const float* mass, int nt, float* row) {
   float2 nm[Pol::P];
 #pragma unroll
-  for (int k = 0; k < Pol::K; ++k) sym_half(nm[k >> 1], k) = MODE == kSymUniform ? 0.f : -mass[k * nt];
+  for (int k = 0; k < Pol::K; ++k) sym_half(nm[k >> 1], k) = MODE == kSymUniform ? 0.f : Pol::kOwnSign * mass[k * nt];
+  const float own = MODE == kSymUniform ? mass[0] : 1.f;
 #pragma unroll 1
   for (; blocks > 0; --blocks) {
     float2 c[Pol::kSumsJ];
@@ -202,19 +219,20 @@ __device__ __forceinline__ void sym_sweep(Pol& acc, const float4* ring, uint32_t
       }
     }
 #pragma unroll
-    for (int d = 0; d < Pol::kSumsJ; ++d) row[d * chunk + lane] = own * (c[d].x + c[d].y);
+    for (int d = 0; d < Pol::kSumsJ; ++d) row[d * chunk + lane] = Pol::back(d, MODE, own) * (c[d].x + c[d].y);
     off += kSymBlock * 16;
     row += kSymBlock;
   }
 }
 
-// Diagonal blocks: every ordered pair, i side only.
+// Diagonal blocks: every ordered pair, i side only (self: the thread's first
+// particle's index relative to js[0]; its others follow nt apart).
 template <class Pol, int MODE>
-__device__ __forceinline__ void sym_diag(Pol& acc, const float4* js, int chunk, int count, float2 e2, int self) {
+__device__ __forceinline__ void sym_diag(Pol& acc, const float4* js, int chunk, int count, float2 e2, int self, int nt) {
 #pragma unroll 1
   for (int j = 0; j < count; j += 8) {
 #pragma unroll
-    for (int jj = 0; jj < 8; ++jj) acc.template one<MODE>(js + j + jj, chunk, e2, self - (j + jj));
+    for (int jj = 0; jj < 8; ++jj) acc.template one<MODE>(js + j + jj, chunk, e2, self - (j + jj), nt);
   }
 }
 
@@ -279,7 +297,7 @@ __device__ __noinline__ void sym_produce(const SymArgs& a, SymControl* ctl, floa
 }
 
 template <class Pol>
-__global__ void __launch_bounds__(256, 2) sym_kernel(const __grid_constant__ SymArgs a) {
+__global__ void __launch_bounds__(256, Pol::kMinBlocks) sym_kernel(const __grid_constant__ SymArgs a) {
   extern __shared__ __align__(1024) unsigned char smem[];
   constexpr int K = Pol::K, P = Pol::P, NI = Pol::kSumsI, NJ = Pol::kSumsJ, JR = Pol::kRec;
   const int NT = blockDim.x;
@@ -316,7 +334,7 @@ __global__ void __launch_bounds__(256, 2) sym_kernel(const __grid_constant__ Sym
   const float2 e2 = sym_dup(a.eps2);
   int32_t cur_I = -1;
   float scale = 1.f;   // of the sums in registers
-  int held = 0;        // j records in them
+  int held = 0;        // j blocks in them
   bool own_uniform = false, own_near = false;  // the warp's masses are equal; its positions are in range
 
   // adds the register sums to the row's (hi, lo) sums (each thread its own
@@ -329,7 +347,7 @@ __global__ void __launch_bounds__(256, 2) sym_kernel(const __grid_constant__ Sym
         float* h = sums + c * B + k * NT + tid;
         float* l = h + NI * B;
         float s, e;
-        two_sum(*h, __fmul_rn(Pol::sign(c) * scale, sym_half(acc.acc[k >> 1][c], k)), s, e);
+        two_sum(*h, __fmul_rn(Pol::weight(c, scale), sym_half(acc.acc[k >> 1][c], k)), s, e);
         *h = s;
         *l = __fadd_rn(*l, e);
       }
@@ -424,7 +442,7 @@ __global__ void __launch_bounds__(256, 2) sym_kernel(const __grid_constant__ Sym
     const uint32_t off = slot * static_cast<uint32_t>(JR * CH) * 16u;
     const float4* js = ring + slot * static_cast<uint32_t>(JR * CH);
     const int count = ch.nb * kSymBlock;
-    int mode = kSymWide;
+    int mode = Pol::kWide ? kSymWide : kSymGeneral;
     float factor = 1.f;
     if constexpr (!Pol::kGuard) {
       const float mj = js[0].w;
@@ -434,35 +452,49 @@ __global__ void __launch_bounds__(256, 2) sym_kernel(const __grid_constant__ Sym
         same = same && v.w == mj;
         near = near && fmaxf(fabsf(v.x), fmaxf(fabsf(v.y), fabsf(v.z))) <= kSymFar;
       }
+      if (Pol::kSameMass)
+        same = same && own_uniform && mass[tid] == mj;
+      else
+        same = same && (ch.diag || own_uniform);
       if (__all_sync(0xffffffffu, near)) {
         mode = kSymGeneral;
-        if (__all_sync(0xffffffffu, same) && (ch.diag || own_uniform)) {
+        if (__all_sync(0xffffffffu, same)) {
           mode = kSymUniform;
           factor = mj;
         }
       }
     }
-    if (held > 0 && (factor != scale || held + count > kSymFold)) fold();
-    scale = factor;
-    held += count;
-    if (ch.diag) {
-      const int self = cur_I * B - ch.blk * kSymBlock + tid;
-      if constexpr (!Pol::kGuard) {
-        if (mode == kSymUniform)
-          sym_diag<Pol, kSymUniform>(acc, js, CH, count, e2, self);
-        else if (mode == kSymGeneral)
-          sym_diag<Pol, kSymGeneral>(acc, js, CH, count, e2, self);
+    constexpr int kStep = Pol::kFold / kSymBlock;  // blocks between folds, at most
+    for (int b0 = 0; b0 < ch.nb; b0 += kStep) {
+      const int nb = ch.nb - b0 < kStep ? ch.nb - b0 : kStep;
+      if (held > 0 && (factor != scale || held + nb > kStep)) fold();
+      scale = factor;
+      held += nb;
+      if (ch.diag) {
+        const float4* js0 = js + b0 * kSymBlock;
+        const int self = cur_I * B - (ch.blk + b0) * kSymBlock + tid;
+        if constexpr (!Pol::kGuard) {
+          if (mode == kSymUniform)
+            sym_diag<Pol, kSymUniform>(acc, js0, CH, nb * kSymBlock, e2, self, NT);
+          else if (mode == kSymGeneral)
+            sym_diag<Pol, kSymGeneral>(acc, js0, CH, nb * kSymBlock, e2, self, NT);
+        }
+        if constexpr (Pol::kWide) {
+          if (mode == kSymWide) sym_diag<Pol, kSymWide>(acc, js0, CH, nb * kSymBlock, e2, self, NT);
+        }
+      } else {
+        float* mine = rows + (q % 3) * (NW * NJ * CH) + warp * (NJ * CH) + b0 * kSymBlock;
+        const uint32_t off0 = off + static_cast<uint32_t>(b0) * (kSymBlock * 16);
+        if constexpr (!Pol::kGuard) {
+          if (mode == kSymUniform)
+            sym_sweep<Pol, kSymUniform>(acc, ring, off0, CH, nb, lane, e2, mass + tid, NT, mine);
+          else if (mode == kSymGeneral)
+            sym_sweep<Pol, kSymGeneral>(acc, ring, off0, CH, nb, lane, e2, mass + tid, NT, mine);
+        }
+        if constexpr (Pol::kWide) {
+          if (mode == kSymWide) sym_sweep<Pol, kSymWide>(acc, ring, off0, CH, nb, lane, e2, mass + tid, NT, mine);
+        }
       }
-      if (mode == kSymWide) sym_diag<Pol, kSymWide>(acc, js, CH, count, e2, self);
-    } else {
-      float* mine = rows + (q % 3) * (NW * NJ * CH) + warp * (NJ * CH);
-      if constexpr (!Pol::kGuard) {
-        if (mode == kSymUniform)
-          sym_sweep<Pol, kSymUniform>(acc, ring, off, CH, ch.nb, lane, e2, -mass[tid], mass + tid, NT, mine);
-        else if (mode == kSymGeneral)
-          sym_sweep<Pol, kSymGeneral>(acc, ring, off, CH, ch.nb, lane, e2, 1.f, mass + tid, NT, mine);
-      }
-      if (mode == kSymWide) sym_sweep<Pol, kSymWide>(acc, ring, off, CH, ch.nb, lane, e2, 1.f, mass + tid, NT, mine);
     }
     if (q > 0) settle(q - 1);
     __syncwarp();
@@ -571,32 +603,47 @@ __global__ void __launch_bounds__(32 * kSymMergeWarps) sym_merge_kernel(const __
 }
 
 // ------------------------------------------------------------------ host side
-template <class Pol>
-size_t sym_smem_of(int threads, int chunk, int stages) {
-  return 1024 + static_cast<size_t>(stages) * Pol::kRec * chunk * 16 +
-         (static_cast<size_t>(3) * (threads / 32) * Pol::kSumsJ * chunk +
-          static_cast<size_t>(2 * Pol::kSumsI + 1) * threads * Pol::K) * sizeof(float);
-}
-
-template <class Pol>
-cudaError_t occupancy_sym_of(int threads, size_t smem, int* ctas) {
-  const void* f = reinterpret_cast<const void*>(&sym_kernel<Pol>);
-  cudaError_t e = prepare_kernel(f, smem);
-  if (e != cudaSuccess) return e;
-  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(ctas, f, threads, smem);
-}
-
-template <class Pol>
-cudaError_t launch_sym_of(const SymArgs& a, const SymMerge& m, int threads, size_t smem, cudaStream_t s) {
-  const void* f = reinterpret_cast<const void*>(&sym_kernel<Pol>);
-  cudaError_t e = prepare_kernel(f, smem);
-  if (e != cudaSuccess) return e;
-  void* args[] = {const_cast<SymArgs*>(&a)};
-  e = launch_pdl(f, dim3(static_cast<unsigned>(a.g.grid)), dim3(threads), args, smem, s);
-  if (e != cudaSuccess) return e;
-  void* margs[] = {const_cast<SymMerge*>(&m)};
-  return launch_pdl(reinterpret_cast<const void*>(&sym_merge_kernel<Pol>),
-                    dim3(static_cast<unsigned>(m.g.n_blocks)), dim3(32 * kSymMergeWarps), margs, 0, s);
-}
+// The launch functions of a form, over its policies with 2, 4 and 8 particles
+// per thread and the guarded one (eps2 = 0).
+template <class P2, class P4, class P8, class PG>
+struct SymTable {
+  template <class F>
+  static auto pick(int k, bool guard, F&& f) {
+    if (guard) return f(PG{});
+    if (k >= 8) return f(P8{});
+    if (k >= 4) return f(P4{});
+    return f(P2{});
+  }
+  static size_t smem(int threads, int k, int chunk, int stages) {
+    return pick(k, false, [&](auto pol) {
+      using Pol = decltype(pol);
+      return 1024 + static_cast<size_t>(stages) * Pol::kRec * chunk * 16 +
+             (static_cast<size_t>(3) * (threads / 32) * Pol::kSumsJ * chunk +
+              static_cast<size_t>(2 * Pol::kSumsI + 1) * threads * Pol::K) * sizeof(float);
+    });
+  }
+  static cudaError_t occupancy(int k, bool guard, int threads, size_t bytes, int* ctas) {
+    return pick(k, guard, [&](auto pol) {
+      const void* f = reinterpret_cast<const void*>(&sym_kernel<decltype(pol)>);
+      const cudaError_t e = prepare_kernel(f, bytes);
+      return e != cudaSuccess ? e : cudaOccupancyMaxActiveBlocksPerMultiprocessor(ctas, f, threads, bytes);
+    });
+  }
+  static cudaError_t launch(const SymArgs& a, const SymMerge& m, int k, bool guard, int threads, size_t bytes,
+                            cudaStream_t s) {
+    return pick(k, guard, [&](auto pol) {
+      const void* f = reinterpret_cast<const void*>(&sym_kernel<decltype(pol)>);
+      cudaError_t e = prepare_kernel(f, bytes);
+      if (e != cudaSuccess) return e;
+      void* args[] = {const_cast<SymArgs*>(&a)};
+      e = launch_pdl(f, dim3(static_cast<unsigned>(a.g.grid)), dim3(threads), args, bytes, s);
+      if (e != cudaSuccess) return e;
+      void* margs[] = {const_cast<SymMerge*>(&m)};
+      return launch_pdl(reinterpret_cast<const void*>(&sym_merge_kernel<decltype(pol)>),
+                        dim3(static_cast<unsigned>(m.g.n_blocks)), dim3(32 * kSymMergeWarps), margs, 0, s);
+    });
+  }
+  static SymOps ops(int max_k) { return SymOps{P2::kSumsI, max_k, &smem, &occupancy, &launch}; }
+};
 
 }  // namespace cn

@@ -143,12 +143,37 @@ struct SymMerge {
   int32_t last;
 };
 
-enum SymForm : int { kSymForce = 0, kSymForcePot = 1 };
+enum SymForm : int {
+  kSymForce = 0,
+  kSymForcePot = 1,
+  kSymJerk = 2,
+  kSymJerkPot = 3,
+  kSymAdjoint = 4,
+};
 
-int sym_sums(SymForm form);  // sums per particle
-size_t sym_smem_bytes(SymForm form, int threads, int k, int chunk, int stages);
-cudaError_t occupancy_sym(SymForm form, int k, bool guard, int threads, size_t smem, int* ctas);
-cudaError_t launch_sym(SymForm form, const SymArgs& a, const SymMerge& m, int k, bool guard, int threads, size_t smem,
-                       cudaStream_t s);
+// A form's kernels: sums per particle, most particles per thread, shared
+// memory of a shape, resident CTAs per SM, and the launch of one band (pair
+// kernel and merge).
+struct SymOps {
+  int sums;
+  int max_k;
+  size_t (*smem)(int threads, int k, int chunk, int stages);
+  cudaError_t (*occupancy)(int k, bool guard, int threads, size_t smem, int* ctas);
+  cudaError_t (*launch)(const SymArgs& a, const SymMerge& m, int k, bool guard, int threads, size_t smem,
+                        cudaStream_t s);
+};
+
+SymOps sym_force_ops(bool pot);    // cn_sym.cu
+SymOps sym_jerk_ops(bool pot);     // cn_sym_jerk.cu
+SymOps sym_adjoint_ops();          // cn_sym_adjoint.cu
+inline SymOps sym_ops(SymForm form) {
+  switch (form) {
+    case kSymForce: return sym_force_ops(false);
+    case kSymForcePot: return sym_force_ops(true);
+    case kSymJerk: return sym_jerk_ops(false);
+    case kSymJerkPot: return sym_jerk_ops(true);
+    default: return sym_adjoint_ops();
+  }
+}
 
 }  // namespace cn

@@ -1,0 +1,129 @@
+// Symmetric adjoint form: the gradient of L = sum_i w_i . a_i, each unordered
+// pair evaluated once.
+#include "cn_sym.cuh"
+
+namespace cn {
+namespace {
+
+// Per pair, with d = x_j - x_i, s = |d|^2 + eps2, r = s^-1/2, g = r^3 and u =
+// m_i w_j - m_j w_i, particle i gets F = g (u - 3 r^2 (d . u) d) in dL/dx and
+// -g (w_j . d) in dL/dm, particle j gets -F and g (w_i . d). With a = w_j . d
+// and b = -w_i . d (both needed for dL/dm), d . u is m_i a + m_j b. 35 lane
+// operations per unordered pair; where the warp's and the chunk's masses are
+// all the same, u is w_j - w_i times that mass and d . u is a + b: 31; against
+// 2 x 30 for the ordered pairs. The sums cancel heavily (the weights are
+// signed): registers are folded into the (hi, lo) sums every kFold records,
+// and a travelling sum takes 32 K / 2 terms per half before it is joined.
+// The pair of a particle with itself is skipped by its index (u of the
+// general term rounds to a residual there).
+template <int K_>
+struct SymAdjointPolicy {
+  static constexpr int K = K_;
+  static constexpr int P = K / 2;
+  static constexpr int kSumsI = 4;
+  static constexpr int kSumsJ = 4;
+  static constexpr int kRec = 2;
+  static constexpr bool kGuard = false;
+  static constexpr int kFold = 64;
+  static constexpr int kMinBlocks = 2;
+  static constexpr bool kWide = false;
+  static constexpr bool kSameMass = true;
+  static constexpr float kOwnSign = 1.f;
+  float2 nx[P][3], nw[P][3], acc[P][kSumsI];
+  float2 mi[P];
+
+  __device__ __forceinline__ void load(const SymArgs& a, int64_t p, bool valid, int k, float& mass, float& reach) {
+    float4 v = make_float4(0.f, 0.f, 0.f, 0.f), u = v;
+    if (valid) {
+      v = __ldg(a.pos + p);
+      u = __ldg(a.rec2 + p);
+    }
+    sym_half(nx[k >> 1][0], k) = -v.x;
+    sym_half(nx[k >> 1][1], k) = -v.y;
+    sym_half(nx[k >> 1][2], k) = -v.z;
+    sym_half(nw[k >> 1][0], k) = -u.x;
+    sym_half(nw[k >> 1][1], k) = -u.y;
+    sym_half(nw[k >> 1][2], k) = -u.z;
+    sym_half(mi[k >> 1], k) = v.w;
+    mass = v.w;
+    reach = 0.f;  // g = r^3 is formed in either mode, as in the one-sided kernel
+  }
+
+  template <int MODE, bool BOTH>
+  __device__ __forceinline__ void term(const float4 r0, const float4 r1, float2 e2, const float2 (&m)[P], int self,
+                                       int nt, float2 (&c)[kSumsJ]) {
+    const float2 jx = sym_dup(r0.x), jy = sym_dup(r0.y), jz = sym_dup(r0.z), jm = sym_dup(r0.w);
+    const float2 wx = sym_dup(r1.x), wy = sym_dup(r1.y), wz = sym_dup(r1.z), m3 = sym_dup(-3.f);
+#pragma unroll
+    for (int p = 0; p < P; ++p) {
+      const float2 dx = __fadd2_rn(jx, nx[p][0]);
+      const float2 dy = __fadd2_rn(jy, nx[p][1]);
+      const float2 dz = __fadd2_rn(jz, nx[p][2]);
+      const float2 s = __ffma2_rn(dx, dx, __ffma2_rn(dy, dy, __ffma2_rn(dz, dz, e2)));
+      float2 r = make_float2(rsqrt_mufu(s.x), rsqrt_mufu(s.y));
+      if constexpr (!BOTH) {  // diagonal blocks: not the particle with itself
+        if (self + 2 * p * nt == 0) r.x = 0.f;
+        if (self + (2 * p + 1) * nt == 0) r.y = 0.f;
+      }
+      const float2 rr = __fmul2_rn(r, r);
+      const float2 g = __fmul2_rn(rr, r);
+      const float2 a = __ffma2_rn(wx, dx, __ffma2_rn(wy, dy, __fmul2_rn(wz, dz)));
+      const float2 b = __ffma2_rn(nw[p][0], dx, __ffma2_rn(nw[p][1], dy, __fmul2_rn(nw[p][2], dz)));
+      float2 ux, uy, uz, du;
+      if constexpr (MODE == kSymUniform) {
+        ux = __fadd2_rn(wx, nw[p][0]);
+        uy = __fadd2_rn(wy, nw[p][1]);
+        uz = __fadd2_rn(wz, nw[p][2]);
+        du = __fadd2_rn(a, b);
+      } else {
+        ux = __ffma2_rn(m[p], wx, __fmul2_rn(jm, nw[p][0]));
+        uy = __ffma2_rn(m[p], wy, __fmul2_rn(jm, nw[p][1]));
+        uz = __ffma2_rn(m[p], wz, __fmul2_rn(jm, nw[p][2]));
+        du = __ffma2_rn(m[p], a, __fmul2_rn(jm, b));
+      }
+      const float2 t = __fmul2_rn(__fmul2_rn(m3, rr), du);
+      const float2 vx = __ffma2_rn(t, dx, ux);
+      const float2 vy = __ffma2_rn(t, dy, uy);
+      const float2 vz = __ffma2_rn(t, dz, uz);
+      acc[p][0] = __ffma2_rn(g, vx, acc[p][0]);
+      acc[p][1] = __ffma2_rn(g, vy, acc[p][1]);
+      acc[p][2] = __ffma2_rn(g, vz, acc[p][2]);
+      acc[p][3] = __ffma2_rn(g, a, acc[p][3]);
+      if constexpr (BOTH) {
+        c[0] = __ffma2_rn(g, vx, c[0]);
+        c[1] = __ffma2_rn(g, vy, c[1]);
+        c[2] = __ffma2_rn(g, vz, c[2]);
+        c[3] = __ffma2_rn(g, b, c[3]);
+      }
+    }
+  }
+  template <int MODE>
+  __device__ __forceinline__ void pair(const float4* ring, uint32_t off, int chunk, float2 e2, const float2 (&m)[P],
+                                       float2 (&c)[kSumsJ]) {
+    const float4* rec = reinterpret_cast<const float4*>(reinterpret_cast<const char*>(ring) + off);
+    term<MODE, true>(rec[0], rec[chunk], e2, m, 0, 0, c);
+  }
+  template <int MODE>
+  __device__ __forceinline__ void one(const float4* js, int chunk, float2 e2, int self, int nt) {
+    float2 none[kSumsJ];
+    term<MODE, false>(js[0], js[chunk], e2, mi, self, nt, none);
+  }
+  __device__ static __forceinline__ float weight(int c, float mass) { return c == 3 ? -1.f : mass; }
+  __device__ static __forceinline__ float back(int c, int mode, float own) {
+    return c == 3 || mode != kSymUniform ? -1.f : -own;
+  }
+  __device__ static __forceinline__ void output(const SymMerge& m, int64_t p, int c, float v) {
+    if (c < 3)
+      m.out[0][3 * p + c] = v;
+    else
+      m.out[1][p] = v;
+  }
+};
+
+using AdjointTable = SymTable<SymAdjointPolicy<2>, SymAdjointPolicy<4>, SymAdjointPolicy<4>, SymAdjointPolicy<2>>;
+
+}  // namespace
+
+SymOps sym_adjoint_ops() { return AdjointTable::ops(4); }
+
+}  // namespace cn
