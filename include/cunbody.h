@@ -310,6 +310,12 @@ CN_API cn_status cn_batch_plan_info(const cn_batch_plan *plan, int64_t *n_total,
  *               the library workspace of `stream`.
  * No allocation happens when a workspace is passed, so the call can be
  * captured into a CUDA graph (see cn_batch_plan_capture).
+ * A plan made without a tune (none registered, every eps2 of normal size)
+ * takes the symmetric form, each cluster's unordered pairs once, where that is
+ * expected to be the faster one; its slots are then part of the workspace
+ * bytes asked for. A smaller workspace that holds the one-sided kernel's
+ * partial sums is accepted and takes that kernel, as does a call whose slots
+ * the library workspace cannot get.
  */
 CN_API cn_status cn_force_batched(const cn_batch_plan *plan, const float *pos_mass, float *acc_out, float *pot_out,
                            void *workspace, size_t ws_bytes, cn_stream stream);

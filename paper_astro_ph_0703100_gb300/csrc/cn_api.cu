@@ -53,6 +53,16 @@ struct cn_batch_plan {
   size_t ws_bytes = 0;
   size_t ctrl_bytes = 0;
   size_t data_bytes = 0;
+  // The symmetric form of an ensemble, where it is expected to be the faster
+  // one (sym_rows > 0); the above stays for calls without room for its slots.
+  int32_t sym_rows = 0;
+  int32_t sym_merge = 0;  // merge CTAs
+  int sym_k = 0, sym_threads = 0, sym_chunk = 0, sym_stages = 0;
+  size_t sym_smem = 0, sym_jslot_b = 0, sym_bytes = 0;
+  int64_t sym_seg = 0;
+  cn::SymGrid sym_grid{};
+  cn::SymRow* d_rows = nullptr;
+  cn::SymMergeBlock* d_blocks = nullptr;
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t exec = nullptr;
 };
@@ -873,7 +883,7 @@ cn_status sym_fit(int dev, const DeviceInfo& d, cn::SymForm form, int64_t n, boo
   sp->k = guard ? 2 : std::min(ops.max_k, std::max(2, p.k));
   sp->threads = p.threads;
   sp->guard = guard;
-  sp->chunk = static_cast<int>(std::min<int64_t>(round_up(p.j_tile, cn::kSymBlock), 1024));
+  sp->chunk = static_cast<int>(std::min<int64_t>(round_up(p.j_tile, cn::kSymBlock), 256));
   sp->stages = std::max(2, p.stages);  // a stage is refilled a chunk after it was read
   sp->tile = static_cast<int64_t>(sp->k) * sp->threads;
   sp->tiles = ceil_div(n, sp->tile);
@@ -930,6 +940,7 @@ cn_status sym_launch(const std::string& what, const DeviceInfo& d, cn::SymForm f
   for (int o = 0; o < 3; ++o) m.out[o] = out[o];
   m.n_pad = sp.n_pad;
   m.tile = static_cast<int32_t>(sp.tile);
+  m.n_merge = static_cast<int32_t>(sp.n_blocks);
   for (int64_t r0 = 0; r0 < sp.tiles; r0 += sp.band) {
     const int64_t r1 = std::min(sp.tiles, r0 + sp.band);
     a.g.row0 = static_cast<int32_t>(r0);
@@ -1241,6 +1252,45 @@ cn_status symmetric_common(int64_t n, const float* pos_mass, float eps2, float* 
   return sym_launch(what, *d, form, t_last, n, pos_mass, nullptr, eps2, out, s);
 }
 
+// ------------------------------------------------------------------ symmetric ensembles
+cn_status launch_ensemble(const DeviceInfo& d, const cn_batch_plan* plan, const float* pos, float* acc_out,
+                          float* pot_out, char* data, cudaStream_t s) {
+  const cn::SymForm form = plan->pot ? cn::kSymBatchedPot : cn::kSymBatched;
+  cn::SymArgs a{};
+  a.g = plan->sym_grid;
+  a.pos = reinterpret_cast<const float4*>(pos);
+  a.slots_j = reinterpret_cast<float*>(data);
+  a.slots_seg = reinterpret_cast<float*>(data + plan->sym_jslot_b);
+  a.n_seg = plan->sym_seg;
+  a.status = d.status;
+  a.chunk = plan->sym_chunk;
+  a.stages = plan->sym_stages;
+  a.wait_ns = g_wait_ns.load();
+  a.rows = plan->d_rows;
+  a.n_rows = plan->sym_rows;
+  cn::SymMerge m{};
+  m.g = a.g;
+  m.slots_seg = a.slots_seg;
+  m.slots_j = a.slots_j;
+  m.out[0] = acc_out;
+  m.out[1] = pot_out;
+  m.tile = plan->sym_k * plan->sym_threads;
+  m.first = m.last = 1;
+  m.rows = plan->d_rows;
+  m.blocks = plan->d_blocks;
+  m.n_merge = plan->sym_merge;
+  if (log_enabled())
+    std::fprintf(stderr,
+                 "[cunbody] cn_force_batched: variant %s n %lld clusters %d | symmetric: K %d threads %d chunk %d stages "
+                 "%d | rows %d cost %lld grid %d smem %zu slots %zu bytes\n",
+                 variant_name(plan->pot ? cn::kBatchedPot : cn::kBatched), static_cast<long long>(plan->n_total),
+                 plan->n_clusters, plan->sym_k, plan->sym_threads, plan->sym_chunk, plan->sym_stages, plan->sym_rows,
+                 static_cast<long long>(a.g.cost), a.g.grid, plan->sym_smem, plan->sym_bytes);
+  if (inject("launch")) return fail(CN_ERR_CUDA, "kernel launch: injected launch failure");
+  const cudaError_t e = cn::sym_ops(form).launch(a, m, plan->sym_k, false, plan->sym_threads, plan->sym_smem, s);
+  return e == cudaSuccess ? CN_OK : fail_cuda(e, "symmetric ensemble launch");
+}
+
 cn_status run_batched(const cn_batch_plan* plan, const float* pos_i, const float* pos_j, float* acc_out,
                       float* pot_out, void* ws, size_t ws_bytes, cudaStream_t s) {
   if (!plan) return fail(CN_ERR_INVALID_ARG, "plan is NULL");
@@ -1266,6 +1316,15 @@ cn_status run_batched(const cn_batch_plan* plan, const float* pos_i, const float
     if (n && pot_out && (e = cudaMemsetAsync(pot_out, 0, n * 4, s)) != cudaSuccess)
       return fail_cuda(e, "cudaMemsetAsync");
     if (plan->units == 0) return CN_OK;
+  }
+  if (plan->sym_rows > 0) {
+    char* slots = nullptr;
+    if (!ws) {
+      if (sym_workspace(s, plan->sym_bytes, &slots) != CN_OK) slots = nullptr;
+    } else if (aligned(ws, 256) && ws_bytes >= std::max(plan->sym_bytes, plan->ws_bytes)) {
+      slots = static_cast<char*>(ws);
+    }
+    if (slots) return launch_ensemble(*d, plan, pos_j, acc_out, pot_out, slots, s);
   }
   Geometry g;
   g.units = plan->units;
@@ -1308,6 +1367,127 @@ struct Group {
   float eps2;
 };
 
+// The symmetric form of an ensemble: its shape by a model of its time, its
+// table of rows and merge blocks, uploaded with the plan. Nothing is kept
+// when the one-sided shape is expected to take less (`one_sided_s`), or when
+// the slots would pass kSymEnsembleCap.
+//
+// The model is off-diagonal pairs / pairs + diagonal pairs / diag + fixed,
+// padding counted as work (unordered pairs of whole 32-record blocks against
+// whole tiles), least squares over 17 ensembles measured in every shape (8 ..
+// 4096 clusters of 64 .. 65536; residuals 5-9%). Its choice is the fastest
+// shape measured for 29 of the 34 (with and without the potential), 6% off at
+// worst: 512 clusters of 256 .. 16384 8 x 128 4849 us (8 x 256 5010, 4 x 128
+// 5274, one-sided 7010), 1000 of 1024 4 x 64 370 us (4 x 128 386, one-sided
+// 428), 4096 of 256 one-sided 115 us (2 x 64 149).
+constexpr size_t kSymEnsembleCap = static_cast<size_t>(1) << 30;
+
+cn_status fit_ensemble(int dev, const DeviceInfo& d, const std::vector<Group>& groups, double one_sided_s,
+                       cn_batch_plan* plan) {
+  struct Shape {
+    int k, threads, chunk;
+    double pairs, diag, fixed_s;  // rates on 152 SMs
+  };
+  static const Shape plain[] = {{8, 256, 128, 2.15e12, 2.70e12, 16e-6}, {8, 128, 128, 2.06e12, 2.51e12, 20e-6},
+                                {4, 128, 128, 1.81e12, 2.19e12, 13e-6}, {4, 64, 128, 1.70e12, 1.82e12, 14e-6},
+                                {2, 128, 128, 1.45e12, 1.80e12, 9e-6},  {2, 64, 128, 1.32e12, 1.52e12, 11e-6}};
+  static const Shape with_pot[] = {{8, 256, 64, 1.67e12, 2.12e12, 18e-6},  {8, 128, 128, 1.61e12, 1.95e12, 19e-6},
+                                   {4, 128, 128, 1.46e12, 1.83e12, 15e-6}, {4, 64, 128, 1.24e12, 1.39e12, 16e-6},
+                                   {2, 128, 128, 1.16e12, 1.54e12, 10e-6}, {2, 64, 128, 1.04e12, 1.34e12, 12e-6}};
+  const cn::SymForm form = plan->pot ? cn::kSymBatchedPot : cn::kSymBatched;
+  const cn::SymOps ops = cn::sym_ops(form);
+  double best_s = one_sided_s;
+  SymPlan best;
+  for (const Shape& sh : plan->pot ? with_pot : plain) {
+    SymPlan sp;
+    sp.k = sh.k;
+    sp.threads = sh.threads;
+    sp.chunk = sh.chunk;
+    sp.stages = 3;
+    sp.tile = static_cast<int64_t>(sh.k) * sh.threads;
+    sp.smem = ops.smem(sp.threads, sp.k, sp.chunk, sp.stages);
+    const double block = static_cast<double>(sp.tile) * cn::kSymBlock;
+    double work_s = 0.0, bytes = 0.0;
+    for (const Group& gr : groups) {
+      const int64_t tb = sp.tile / cn::kSymBlock, nb = ceil_div(gr.ni, cn::kSymBlock), t = ceil_div(nb, tb);
+      // blocks behind the diagonal tiles of all the cluster's rows
+      const double off = static_cast<double>(t) * nb - static_cast<double>(tb) * (static_cast<double>(t) * (t + 1) / 2) +
+                         static_cast<double>(t * tb - nb);
+      work_s += block * (off / sh.pairs + static_cast<double>(nb) / sh.diag);
+      bytes += off * cn::kSymBlock * 4.0 * ops.sums;
+    }
+    const double time_s = work_s * 152.0 / d.sms + sh.fixed_s;
+    if (bytes <= static_cast<double>(kSymEnsembleCap) && time_s < best_s) {
+      best_s = time_s;
+      best = sp;
+    }
+  }
+  if (best.k == 0) return CN_OK;
+  int occ = 0;
+  cn_status st = sym_occupancy(dev, form, best, &occ);
+  if (st != CN_OK) return st;
+  best.slots = static_cast<int64_t>(occ) * d.sms;
+  std::vector<cn::SymRow> rows;
+  std::vector<cn::SymMergeBlock> blocks;
+  const int64_t tb = best.tile / cn::kSymBlock;
+  int64_t cost = 0, slot = 0;
+  for (const Group& gr : groups) {
+    if (gr.ni == 0) continue;
+    const int64_t nb = ceil_div(gr.ni, cn::kSymBlock);
+    const size_t first = rows.size();
+    for (int64_t b0 = 0; b0 < nb; b0 += tb) {
+      cn::SymRow r{};
+      r.cost = cost;
+      r.p0 = gr.i_begin;
+      r.slot = slot;
+      r.n = static_cast<int32_t>(gr.ni);
+      r.n_blocks = static_cast<int32_t>(nb);
+      r.blk0 = static_cast<int32_t>(b0);
+      r.diag_end = static_cast<int32_t>(std::min(nb, b0 + tb));
+      r.plane = static_cast<int32_t>((nb - r.diag_end) * cn::kSymBlock);
+      r.eps2 = gr.eps2;
+      cost += r.length();
+      slot += static_cast<int64_t>(r.plane) * ops.sums;
+      rows.push_back(r);
+    }
+    for (int64_t b = 0; b < nb; ++b)
+      blocks.push_back(cn::SymMergeBlock{static_cast<int32_t>(first), static_cast<int32_t>(first + b / tb),
+                                         static_cast<int32_t>(b)});
+  }
+  if (rows.empty() || rows.size() > static_cast<size_t>(INT32_MAX) || blocks.size() > static_cast<size_t>(INT32_MAX))
+    return CN_OK;
+  cudaError_t e = cudaMalloc(reinterpret_cast<void**>(&plan->d_rows), rows.size() * sizeof(cn::SymRow));
+  if (e == cudaSuccess)
+    e = cudaMalloc(reinterpret_cast<void**>(&plan->d_blocks), blocks.size() * sizeof(cn::SymMergeBlock));
+  if (e == cudaSuccess)
+    e = cudaMemcpy(plan->d_rows, rows.data(), rows.size() * sizeof(cn::SymRow), cudaMemcpyHostToDevice);
+  if (e == cudaSuccess)
+    e = cudaMemcpy(plan->d_blocks, blocks.data(), blocks.size() * sizeof(cn::SymMergeBlock), cudaMemcpyHostToDevice);
+  if (e != cudaSuccess) {
+    cudaFree(plan->d_rows);
+    cudaFree(plan->d_blocks);
+    plan->d_rows = nullptr;
+    plan->d_blocks = nullptr;
+    cudaGetLastError();  // the plan goes on without them
+    return fail_cuda(e, "uploading the ensemble's rows");
+  }
+  plan->sym_k = best.k;
+  plan->sym_threads = best.threads;
+  plan->sym_chunk = best.chunk;
+  plan->sym_stages = best.stages;
+  plan->sym_smem = best.smem;
+  plan->sym_grid.n = plan->n_total;
+  plan->sym_grid.cost = cost;
+  plan->sym_grid.grid = static_cast<int32_t>(std::max<int64_t>(1, std::min<int64_t>(best.slots, cost / cn::kSymCostPair)));
+  plan->sym_seg = plan->sym_grid.grid + static_cast<int64_t>(rows.size());
+  plan->sym_jslot_b = align_up(static_cast<size_t>(slot) * sizeof(float), 256);
+  plan->sym_bytes =
+      plan->sym_jslot_b + static_cast<size_t>(plan->sym_seg) * best.tile * sizeof(float) * static_cast<size_t>(ops.sums);
+  plan->sym_merge = static_cast<int32_t>(blocks.size());
+  plan->sym_rows = static_cast<int32_t>(rows.size());
+  return CN_OK;
+}
+
 // Builds the (group, i-tile, j-tile) unit table of a plan and uploads it.
 // index_host (gathering list plans): n_index list entries, each the index of
 // a j record; the groups' j ranges then count entries of this array.
@@ -1331,6 +1511,7 @@ cn_status build_group_plan(const std::vector<Group>& groups, bool lists, int64_t
   const int variant = with_pot ? cn::kBatchedPot : cn::kBatched;
   const int64_t key_i = static_cast<int64_t>(groups.size());
   cn_tune fitted{};
+  double one_sided_s = 0.0;
   if (!tune && !registered_tune(dev, variant, key_i, n_i_total)) {
     // i-tile fitted to the group sizes: every group is cut into whole i-tiles,
     // so a tile larger than the typical group leaves lanes idle, and every
@@ -1383,6 +1564,11 @@ cn_status build_group_plan(const std::vector<Group>& groups, bool lists, int64_t
       if (fitted.j_lanes < 2) fitted.j_lanes = 0;
     }
     tune = &fitted;
+    // that shape's expected time: 0.78 of the FP32 bound times its score, 14
+    // operations with the potential, and 10 us (4096 clusters of 256: 113 us
+    // against 115 measured, 512 of 256 .. 16384: 7.4 ms against 7.0)
+    one_sided_s =
+        10e-6 + pairs / (std::max(best, 1e-3) * 0.78 * 3.356e12 * (with_pot ? 12.0 / 14.0 : 1.0) * d->sms / 152.0);
   }
   Plan p;
   if ((st = resolve_plan(dev, variant, key_i, n_i_total, guard, tune, &p)) != CN_OK) return st;
@@ -1479,6 +1665,9 @@ cn_status build_group_plan(const std::vector<Group>& groups, bool lists, int64_t
       return fail_cuda(e, "uploading the batched unit table");
     }
   }
+  // an ensemble in its default shape: the symmetric form too, where it is
+  // expected to be the faster one (a plan without it when its table cannot be had)
+  if (!lists && !guard && tune == &fitted && !tiles.empty()) fit_ensemble(dev, *d, groups, one_sided_s, plan);
   *out = plan;
   return CN_OK;
 }
@@ -1885,12 +2074,16 @@ cn_status cn_batch_plan_destroy(cn_batch_plan* plan) {
     if (plan->graph) cudaGraphDestroy(plan->graph);
     if (plan->d_tiles) cudaFree(plan->d_tiles);
     if (plan->d_index) cudaFree(plan->d_index);
+    if (plan->d_rows) cudaFree(plan->d_rows);
+    if (plan->d_blocks) cudaFree(plan->d_blocks);
     delete plan;
     return CN_OK;
   });
 }
 
-size_t cn_batch_plan_workspace_bytes(const cn_batch_plan* plan) { return plan ? plan->ws_bytes : 0; }
+size_t cn_batch_plan_workspace_bytes(const cn_batch_plan* plan) {
+  return plan ? std::max(plan->ws_bytes, plan->sym_bytes) : 0;
+}
 
 cn_status cn_batch_plan_info(const cn_batch_plan* plan, int64_t* n_total, double* pairs) {
   return cn::guard([&]() -> cn_status {
@@ -2474,7 +2667,18 @@ cn_status cn_autotune_batched(int32_t n_clusters, const int64_t* offsets_host, c
     float best_ms = 1e30f;
     cn_tune best{};
     cn_status result = CN_OK;
-    std::vector<cn_tune> cands;
+    // The default first (a plan without a tune, which may take the symmetric
+    // form): when nothing beats it, no entry is stored and best_out is its
+    // one-sided shape.
+    const int64_t n_total = offsets_host[n_clusters];
+    int dev = 0;
+    cudaGetDevice(&dev);
+    cn_tune before{}, bare_shape{};
+    const bool had = registered_tune(dev, variant, n_clusters, n_total);
+    if (had) cn_tune_get(variant, n_clusters, n_total, &before);
+    cn_tune_set(variant, n_clusters, n_total, nullptr);
+    bool best_bare = false;
+    std::vector<cn_tune> cands{bare_shape};
     for (int k : ks)
       for (int th : ths)
         for (int jt : tiles)
@@ -2486,7 +2690,9 @@ cn_status cn_autotune_batched(int32_t n_clusters, const int64_t* offsets_host, c
     for (const cn_tune& t : cands) {
       if (result != CN_OK) break;
       cn_batch_plan* plan = nullptr;
-      cn_status st = build_batch_plan(n_clusters, offsets_host, eps2_host, &t, pot_out != nullptr, &plan);
+      const bool is_bare = &t == &cands.front();
+      cn_status st =
+          build_batch_plan(n_clusters, offsets_host, eps2_host, is_bare ? nullptr : &t, pot_out != nullptr, &plan);
       if (st != CN_OK) {
         if (st == CN_ERR_INVALID_ARG) continue;
         result = st;
@@ -2503,6 +2709,10 @@ cn_status cn_autotune_batched(int32_t n_clusters, const int64_t* offsets_host, c
           if (ms < best_ms) {
             best_ms = ms;
             best = t;
+            best_bare = is_bare;
+            if (is_bare)
+              best = cn_tune{plan->plan.k, plan->plan.threads, plan->plan.j_tile, plan->plan.stages, 0,
+                             static_cast<int32_t>(plan->plan.chunk_units), plan->plan.j_lanes};
           }
         } else {
           st = fail(CN_ERR_CUDA, "autotune: event synchronisation failed");
@@ -2513,10 +2723,12 @@ cn_status cn_autotune_batched(int32_t n_clusters, const int64_t* offsets_host, c
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
-    if (result != CN_OK) return result;
-    if (best_ms >= 1e30f) return fail(CN_ERR_INVALID_ARG, "no candidate launch shape fits");
-    const int64_t n_total = offsets_host[n_clusters];
-    cn_tune_set(variant, n_clusters, n_total, &best);
+    if (result != CN_OK || best_ms >= 1e30f) {
+      if (had) cn_tune_set(variant, n_clusters, n_total, &before);
+      if (result != CN_OK) return result;
+      return fail(CN_ERR_INVALID_ARG, "no candidate launch shape fits");
+    }
+    if (!best_bare) cn_tune_set(variant, n_clusters, n_total, &best);
     if (best_out) *best_out = best;
     return CN_OK;
   });

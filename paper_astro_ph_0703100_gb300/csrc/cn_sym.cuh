@@ -14,7 +14,8 @@
 // needed: against summing each record over the warp by a reduce-scatter
 // this takes 24 shuffles and 24 additions per 8 records to 48 shuffles and
 // none, which leaves the FP32 pipe to the pair terms (inner loop at K = 8 x
-// 256 threads, 2.07 GHz: 1.93e12 -> 2.03e12 unordered pairs/s).
+// 256 threads, 2.07 GHz: 1.93e12 -> 2.03e12 unordered pairs/s; whole calls at
+// N = 131072 with equal masses: 4653 -> 4000 us).
 //
 // What bounds the loop: the FP32 pipe, and with it the register file. A
 // packed multiply-add whose three operands are different registers issues
@@ -54,7 +55,8 @@ namespace cn {
 
 constexpr float kSymFar = 1e11f;       // |coordinate| up to which r^-3 stays a normal number
 constexpr float kSymSoft = 1e-20f;     // eps2 from which it stays finite
-constexpr int kSymUnroll = 4;          // steps per loop trip (must divide 32)
+
+constexpr int kSymMostStage = 256;     // records per stage, at most
 
 enum SymMode : int {
   kSymUniform = 0,  // equal masses, factored out of the pair terms
@@ -71,6 +73,7 @@ __device__ __forceinline__ float& sym_half(float2& v, int k) { return (k & 1) ? 
 //   kSumsI, kSumsJ  sums per particle and side
 //   kRec            float4 words per record (2: a velocity or a loss weight)
 //   kMinBlocks      256-thread CTAs per SM the registers are limited for
+//   kUnroll         steps per loop trip (divides 32)
 //   kFold           j records summed in FP32 registers between TwoSum folds
 //   kWide           offers the kSymWide terms
 //   kSameMass       equal masses factor out only if the warp's and the
@@ -85,7 +88,7 @@ __device__ __forceinline__ float& sym_half(float2& v, int k) { return (k & 1) ? 
 // Force (and potential): per pair, d = x_j - x_i, s = |d|^2 + eps2, r =
 // s^-1/2; i: m_j r^3 d (and m_j r), j: -m_i r^3 d (and -m_i r). The
 // potential skips pairs at exactly zero separation.
-template <int K_, bool POT, bool GUARD>
+template <int K_, bool POT, bool GUARD, int UNROLL>
 struct SymForcePolicy {
   static constexpr int K = K_;
   static constexpr int P = K / 2;
@@ -93,6 +96,7 @@ struct SymForcePolicy {
   static constexpr int kSumsJ = POT ? 4 : 3;
   static constexpr int kRec = 1;
   static constexpr bool kGuard = GUARD;
+  static constexpr int kUnroll = UNROLL;
   static constexpr int kFold = 512;
   static constexpr int kMinBlocks = 2;
   static constexpr bool kWide = true;
@@ -180,7 +184,7 @@ struct SymForcePolicy {
   __device__ static __forceinline__ void output(const SymMerge& m, int64_t p, int c, float v) {
     if (c < 3)
       m.out[0][3 * p + c] = v;
-    else
+    else if (m.out[1])  // a plan with the potential may be run without it
       m.out[1][p] = v;
   }
 };
@@ -204,13 +208,13 @@ __device__ __forceinline__ void sym_sweep(Pol& acc, const float4* ring, uint32_t
 #pragma unroll
     for (int d = 0; d < Pol::kSumsJ; ++d) c[d] = make_float2(0.f, 0.f);
 #pragma unroll 1
-    for (int u = 0; u < kSymBlock; u += kSymUnroll) {
+    for (int u = 0; u < kSymBlock; u += Pol::kUnroll) {
       const uint32_t o = off + (static_cast<uint32_t>(lane ^ u) << 4);
-      const int next = ((kSymUnroll - 1) ^ u ^ (u + kSymUnroll)) & 31;  // exchange into the next trip
+      const int next = ((Pol::kUnroll - 1) ^ u ^ (u + Pol::kUnroll)) & 31;  // exchange into the next trip
 #pragma unroll
-      for (int s = 0; s < kSymUnroll; ++s) {
+      for (int s = 0; s < Pol::kUnroll; ++s) {
         acc.template pair<MODE>(ring, o ^ static_cast<uint32_t>(s << 4), chunk, e2, nm, c);
-        const int m = s + 1 < kSymUnroll ? s ^ (s + 1) : next;
+        const int m = s + 1 < Pol::kUnroll ? s ^ (s + 1) : next;
 #pragma unroll
         for (int d = 0; d < Pol::kSumsJ; ++d) {
           c[d].x = __shfl_xor_sync(0xffffffffu, c[d].x, m);
@@ -242,6 +246,10 @@ __device__ __forceinline__ void sym_diag(Pol& acc, const float4* js, int chunk, 
 struct SymChunk {
   int32_t row, blk, nb, diag;  // nb = 0: no more chunks
 };
+struct SymSlot {               // ensembles: a chunk's j-side slots, and their plane
+  int64_t at;
+  int64_t plane;
+};
 struct SymControl {
   uint64_t full[8];
   uint64_t done[3];  // a chunk swept by every warp (and the chunk before it added up)
@@ -250,11 +258,12 @@ struct SymControl {
   SymCursor ahead;   // the next one (thread 0)
   int64_t end;
   SymChunk chunk[16];
+  SymSlot slot[16];
 };
 static_assert(sizeof(SymControl) <= 1024, "control block");
 
 // Stages the next chunk of this CTA (thread 0), or marks the end.
-template <class Pol>
+template <class Pol, bool BATCHED>
 __device__ __noinline__ void sym_produce(const SymArgs& a, SymControl* ctl, float4* ring) {
   constexpr int JR = Pol::kRec;
   const uint32_t q = ctl->issued;
@@ -263,12 +272,32 @@ __device__ __noinline__ void sym_produce(const SymArgs& a, SymControl* ctl, floa
   SymCursor cur = ctl->ahead;
   bool diag = false;
   ch.nb = 0;
-  if (cur.s < ctl->end) cur.take(a.g, ctl->end, a.chunk / kSymBlock, &ch.row, &ch.blk, &ch.nb, &diag);
+  int64_t p0 = 0, n = a.g.n;
+  if (cur.s < ctl->end) {
+    if constexpr (BATCHED) {
+      sym_take_rows(cur, a.rows, a.n_rows, ctl->end, a.chunk / kSymBlock, &ch.row, &ch.blk, &ch.nb, &diag);
+      const SymRow r = a.rows[ch.row];
+      p0 = r.p0;
+      n = r.n;
+      ctl->slot[q & 15u] = SymSlot{r.slot + static_cast<int64_t>(ch.blk - r.diag_end) * kSymBlock, r.plane};
+    } else {
+      cur.take(a.g, ctl->end, a.chunk / kSymBlock, &ch.row, &ch.blk, &ch.nb, &diag);
+    }
+  }
   ch.diag = diag;
 #ifdef CN_DEBUG_BOUNDS
-  if (ch.nb != 0 && (ch.row < a.g.row0 || ch.row >= a.g.row1 || ch.nb < 1 || ch.nb > a.chunk / kSymBlock ||
-                     ch.blk < ch.row * a.g.tile_blocks || ch.blk + ch.nb > a.g.n_blocks ||
-                     static_cast<int64_t>(blockIdx.x) + (ch.row - a.g.row0) >= a.n_seg)) {
+  bool bad = false;
+  if (ch.nb != 0) {
+    if constexpr (BATCHED)
+      bad = ch.row < 0 || ch.row >= a.n_rows || ch.blk < a.rows[ch.row].blk0 ||
+            ch.blk + ch.nb > a.rows[ch.row].n_blocks || p0 < 0 || p0 + n > a.g.n;
+    else
+      bad = ch.row < a.g.row0 || ch.row >= a.g.row1 || ch.blk < ch.row * a.g.tile_blocks ||
+            ch.blk + ch.nb > a.g.n_blocks;
+    bad = bad || ch.nb < 1 || ch.nb > a.chunk / kSymBlock ||
+          static_cast<int64_t>(blockIdx.x) + (ch.row - a.g.row0) >= a.n_seg;
+  }
+  if (bad) {
     set_status(a.status, kStatusBadSchedule);
     ch.nb = 0;  // the CTA stops here
   }
@@ -280,8 +309,8 @@ __device__ __noinline__ void sym_produce(const SymArgs& a, SymControl* ctl, floa
     mbar_arrive(&ctl->full[slot]);
     return;
   }
-  const int64_t first = static_cast<int64_t>(ch.blk) * kSymBlock;
-  const int64_t left = a.g.n - first;
+  const int64_t left = n - static_cast<int64_t>(ch.blk) * kSymBlock;
+  const int64_t first = p0 + static_cast<int64_t>(ch.blk) * kSymBlock;
   const int want = ch.nb * kSymBlock;
   const int cnt = static_cast<int>(left < want ? left : want);
   float4* dst = ring + static_cast<size_t>(slot) * JR * a.chunk;
@@ -296,7 +325,7 @@ __device__ __noinline__ void sym_produce(const SymArgs& a, SymControl* ctl, floa
     bulk_copy_g2s(dst + a.chunk, a.rec2 + first, static_cast<uint32_t>(cnt) * 16u, &ctl->full[slot]);
 }
 
-template <class Pol>
+template <class Pol, bool BATCHED>
 __global__ void __launch_bounds__(256, Pol::kMinBlocks) sym_kernel(const __grid_constant__ SymArgs a) {
   extern __shared__ __align__(1024) unsigned char smem[];
   constexpr int K = Pol::K, P = Pol::P, NI = Pol::kSumsI, NJ = Pol::kSumsJ, JR = Pol::kRec;
@@ -322,16 +351,19 @@ __global__ void __launch_bounds__(256, Pol::kMinBlocks) sym_kernel(const __grid_
     ctl->issued = 0;
     mbar_init_fence();
     ctl->end = a.g.part(static_cast<int64_t>(blockIdx.x) + 1);
-    ctl->ahead.seek(a.g, a.g.part(blockIdx.x));
+    if constexpr (BATCHED)  // the plan's table: written when the plan was made
+      sym_seek_rows(ctl->ahead, a.rows, a.n_rows, a.g.part(blockIdx.x));
+    else
+      ctl->ahead.seek(a.g, a.g.part(blockIdx.x));
   }
   __syncthreads();
-  // only shared memory so far: global memory after the previous kernel ends
+  // no call's data so far: that only after the previous kernel ends
   grid_dependency_wait();
   if (tid == 0)
-    for (uint32_t s = 0; s < S; ++s) sym_produce<Pol>(a, ctl, ring);
+    for (uint32_t s = 0; s < S; ++s) sym_produce<Pol, BATCHED>(a, ctl, ring);
 
   Pol acc;
-  const float2 e2 = sym_dup(a.eps2);
+  float2 e2 = sym_dup(a.eps2);
   int32_t cur_I = -1;
   float scale = 1.f;   // of the sums in registers
   int held = 0;        // j blocks in them
@@ -381,18 +413,24 @@ __global__ void __launch_bounds__(256, Pol::kMinBlocks) sym_kernel(const __grid_
     }
     live = __all_sync(0xffffffffu, live);
     if (!live) return;
-    if (tid == 0) sym_produce<Pol>(a, ctl, ring);
+    if (tid == 0) sym_produce<Pol, BATCHED>(a, ctl, ring);
     const SymChunk ch = ctl->chunk[q & 15u];
     if (ch.diag) return;
     const float* row = rows + b * (NW * NJ * CH);
-    float* slot = a.slots_j + static_cast<size_t>(ch.row - a.g.row0) * NJ * a.n_pad +
-                  static_cast<size_t>(ch.blk) * kSymBlock;
+    float* slot = a.slots_j;
+    size_t plane = static_cast<size_t>(a.n_pad);
+    if constexpr (BATCHED) {
+      slot += ctl->slot[q & 15u].at;
+      plane = static_cast<size_t>(ctl->slot[q & 15u].plane);
+    } else {
+      slot += static_cast<size_t>(ch.row - a.g.row0) * NJ * a.n_pad + static_cast<size_t>(ch.blk) * kSymBlock;
+    }
     for (int it = warp; it < NJ * ch.nb; it += NW) {
       const int d = it % NJ, j = (it / NJ) * kSymBlock + lane;
       const float* r = row + d * CH + j;
       float v = r[0];
       for (int w = 1; w < NW; ++w) v += r[w * (NJ * CH)];
-      slot[static_cast<size_t>(d) * a.n_pad + j] = v;
+      slot[static_cast<size_t>(d) * plane + j] = v;
     }
   };
 
@@ -416,18 +454,25 @@ __global__ void __launch_bounds__(256, Pol::kMinBlocks) sym_kernel(const __grid_
       cur_I = ch.row;
       bool same = true, near = true;
       float m0 = 0.f;
+      int64_t p0 = static_cast<int64_t>(cur_I) * B, pn = a.g.n;
+      if constexpr (BATCHED) {
+        const SymRow r = a.rows[cur_I];
+        p0 = r.p0 + static_cast<int64_t>(r.blk0) * kSymBlock;
+        pn = r.p0 + r.n;
+        e2 = sym_dup(r.eps2);
+      }
 #pragma unroll
       for (int k = 0; k < K; ++k) {
-        const int64_t p = static_cast<int64_t>(cur_I) * B + k * NT + tid;
+        const int64_t p = p0 + k * NT + tid;
         float m, reach;
-        acc.load(a, p, p < a.g.n, k, m, reach);
+        acc.load(a, p, p < pn, k, m, reach);
         mass[k * NT + tid] = m;
         if (k == 0) m0 = __shfl_sync(0xffffffffu, m, 0);
         same = same && m == m0;
         near = near && reach <= kSymFar;
       }
       own_uniform = __all_sync(0xffffffffu, same && fabsf(m0) <= 3.4e38f);
-      own_near = __all_sync(0xffffffffu, near && a.eps2 >= kSymSoft);
+      own_near = __all_sync(0xffffffffu, near && e2.x >= kSymSoft);
 #pragma unroll
       for (int p = 0; p < P; ++p)
 #pragma unroll
@@ -465,8 +510,8 @@ __global__ void __launch_bounds__(256, Pol::kMinBlocks) sym_kernel(const __grid_
       }
     }
     constexpr int kStep = Pol::kFold / kSymBlock;  // blocks between folds, at most
-    for (int b0 = 0; b0 < ch.nb; b0 += kStep) {
-      const int nb = ch.nb - b0 < kStep ? ch.nb - b0 : kStep;
+    // the blocks b0 .. b0 + nb - 1 of the chunk
+    auto sweep = [&](int b0, int nb) {
       if (held > 0 && (factor != scale || held + nb > kStep)) fold();
       scale = factor;
       held += nb;
@@ -495,6 +540,11 @@ __global__ void __launch_bounds__(256, Pol::kMinBlocks) sym_kernel(const __grid_
           if (mode == kSymWide) sym_sweep<Pol, kSymWide>(acc, ring, off0, CH, nb, lane, e2, mass + tid, NT, mine);
         }
       }
+    };
+    if constexpr (Pol::kFold >= kSymMostStage) {
+      sweep(0, ch.nb);
+    } else {
+      for (int b0 = 0; b0 < ch.nb; b0 += kStep) sweep(b0, ch.nb - b0 < kStep ? ch.nb - b0 : kStep);
     }
     if (q > 0) settle(q - 1);
     __syncwarp();
@@ -524,29 +574,49 @@ __global__ void __launch_bounds__(256, Pol::kMinBlocks) sym_kernel(const __grid_
 // N = 4096 .. 16384); the warps' sums are added in warp order. All sums
 // are FP32 (hi, lo) pairs by TwoSum: six FP32 operations, where an FP64
 // addition and its conversion take 32 times as long on this GPU.
-constexpr int kSymMergeWarps = 8;
-template <class Pol>
-__global__ void __launch_bounds__(32 * kSymMergeWarps) sym_merge_kernel(const __grid_constant__ SymMerge m) {
-  constexpr int NI = Pol::kSumsI, NW = kSymMergeWarps;
+// An ensemble's particles have few of either: 2 warps there.
+template <bool BATCHED>
+constexpr int kSymMergeWarps = BATCHED ? 2 : 8;
+template <class Pol, bool BATCHED>
+__global__ void __launch_bounds__(32 * kSymMergeWarps<BATCHED>) sym_merge_kernel(const __grid_constant__ SymMerge m) {
+  constexpr int NI = Pol::kSumsI, NW = kSymMergeWarps<BATCHED>;
   __shared__ float2 part[NW][NI][32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int64_t p = blockIdx.x * static_cast<int64_t>(32) + lane;
-  const bool valid = p < m.g.n;
-  const int32_t I = static_cast<int32_t>((blockIdx.x * static_cast<int64_t>(32)) / m.tile);  // 32 divides the tile
-  const int32_t jend = I < m.g.row1 ? I : m.g.row1;
-  const int nj = jend > m.g.row0 ? jend - m.g.row0 : 0;
-  // i-side: the CTAs whose parts hold the units of row I (when it is one of the launch's rows)
-  int ns = 0;
+  int64_t p, jrow = 0;  // the particle; the first row with a slot of it
+  bool valid;
+  int nj = 0, ns = 0;   // its slots and segments
   const float* seg = nullptr;
-  if (I >= m.g.row0 && I < m.g.row1) {
-    const int64_t s0 = m.g.row_start(I), s1 = m.g.row_start(static_cast<int64_t>(I) + 1);
-    const int64_t last = s1 - (m.g.diag_end(I) < m.g.n_blocks ? kSymCostPair : kSymCostDiag);
-    const int64_t c0 = m.g.owner(s0), c1 = m.g.owner(last);
-    ns = static_cast<int>(c1 - c0 + 1);
-    seg = m.slots_seg + (static_cast<size_t>(c0) + static_cast<size_t>(I - m.g.row0)) * NI * m.tile +
-          static_cast<size_t>(p - static_cast<int64_t>(I) * m.tile);
+  const float* slot = nullptr;
+  int32_t blk = static_cast<int32_t>(blockIdx.x);
+  if constexpr (BATCHED) {
+    const SymMergeBlock mb = m.blocks[blockIdx.x];
+    const SymRow r = m.rows[mb.row];
+    blk = mb.blk;
+    const int32_t local = blk * kSymBlock + lane;
+    p = r.p0 + local;
+    valid = local < r.n;
+    jrow = mb.first;
+    nj = mb.row - mb.first;
+    const int64_t c0 = m.g.owner(r.cost);
+    ns = static_cast<int>(m.g.owner(r.last()) - c0 + 1);
+    seg = m.slots_seg + static_cast<size_t>(c0 + mb.row) * NI * m.tile + (local - r.blk0 * kSymBlock);
+  } else {
+    p = static_cast<int64_t>(blk) * kSymBlock + lane;
+    valid = p < m.g.n;
+    const int32_t I = static_cast<int32_t>((static_cast<int64_t>(blk) * kSymBlock) / m.tile);  // 32 divides the tile
+    const int32_t jend = I < m.g.row1 ? I : m.g.row1;
+    nj = jend > m.g.row0 ? jend - m.g.row0 : 0;
+    // i-side: the CTAs whose parts hold the units of row I (when it is one of the launch's rows)
+    if (I >= m.g.row0 && I < m.g.row1) {
+      const int64_t s0 = m.g.row_start(I), s1 = m.g.row_start(static_cast<int64_t>(I) + 1);
+      const int64_t last = s1 - (m.g.diag_end(I) < m.g.n_blocks ? kSymCostPair : kSymCostDiag);
+      const int64_t c0 = m.g.owner(s0), c1 = m.g.owner(last);
+      ns = static_cast<int>(c1 - c0 + 1);
+      seg = m.slots_seg + (static_cast<size_t>(c0) + static_cast<size_t>(I - m.g.row0)) * NI * m.tile +
+            static_cast<size_t>(p - static_cast<int64_t>(I) * m.tile);
+    }
+    slot = m.slots_j + static_cast<size_t>(p);
   }
-  const float* slot = m.slots_j + static_cast<size_t>(p);
   const int total = nj + ns;
   grid_dependency_wait();  // the slots are complete once the symmetric kernel has ended
   grid_launch_dependents();
@@ -560,9 +630,18 @@ __global__ void __launch_bounds__(32 * kSymMergeWarps) sym_merge_kernel(const __
     for (int u = 0; u < kAhead; ++u) {
       const int e = q + u * NW;
       if (e < total && valid) {
-        const float* src = e < nj ? slot + static_cast<size_t>(e) * NI * m.n_pad
-                                  : seg + static_cast<size_t>(e - nj) * NI * m.tile;
-        const size_t plane = e < nj ? static_cast<size_t>(m.n_pad) : static_cast<size_t>(m.tile);
+        const float* src = seg + static_cast<int64_t>(e - nj) * NI * m.tile;
+        int64_t plane = m.tile;
+        if (e < nj) {
+          if constexpr (BATCHED) {
+            const SymRow& r = m.rows[jrow + e];
+            src = m.slots_j + r.slot + static_cast<int64_t>(blk - r.diag_end) * kSymBlock + lane;
+            plane = r.plane;
+          } else {
+            src = slot + static_cast<size_t>(e) * NI * m.n_pad;
+            plane = m.n_pad;
+          }
+        }
 #pragma unroll
         for (int c = 0; c < NI; ++c) w[u][c] = __ldcs(src + c * plane);
       }
@@ -581,31 +660,31 @@ __global__ void __launch_bounds__(32 * kSymMergeWarps) sym_merge_kernel(const __
 #pragma unroll
   for (int c = 0; c < NI; ++c) part[warp][c][lane] = make_float2(hi[c], lo[c]);
   __syncthreads();
-  if (warp >= NI || !valid) return;
-  // warp c: component c
-  const int c = warp;
-  float h = 0.f, l = 0.f;
-  if (!m.first) {
-    const float2 v = m.carry[static_cast<size_t>(c) * m.n_pad + p];
-    h = v.x;
-    l = v.y;
-  }
+  if (!valid) return;
+  for (int c = warp; c < NI; c += NW) {
+    float h = 0.f, l = 0.f;
+    if (!m.first) {
+      const float2 v = m.carry[static_cast<size_t>(c) * m.n_pad + p];
+      h = v.x;
+      l = v.y;
+    }
 #pragma unroll
-  for (int w = 0; w < NW; ++w) {
-    float e;
-    two_sum(h, part[w][c][lane].x, h, e);
-    l = __fadd_rn(l, __fadd_rn(e, part[w][c][lane].y));
+    for (int w = 0; w < NW; ++w) {
+      float e;
+      two_sum(h, part[w][c][lane].x, h, e);
+      l = __fadd_rn(l, __fadd_rn(e, part[w][c][lane].y));
+    }
+    if (m.last)
+      Pol::output(m, p, c, __fadd_rn(h, l));
+    else
+      m.carry[static_cast<size_t>(c) * m.n_pad + p] = make_float2(h, l);
   }
-  if (m.last)
-    Pol::output(m, p, c, __fadd_rn(h, l));
-  else
-    m.carry[static_cast<size_t>(c) * m.n_pad + p] = make_float2(h, l);
 }
 
 // ------------------------------------------------------------------ host side
 // The launch functions of a form, over its policies with 2, 4 and 8 particles
 // per thread and the guarded one (eps2 = 0).
-template <class P2, class P4, class P8, class PG>
+template <class P2, class P4, class P8, class PG, bool BATCHED = false>
 struct SymTable {
   template <class F>
   static auto pick(int k, bool guard, F&& f) {
@@ -624,7 +703,7 @@ struct SymTable {
   }
   static cudaError_t occupancy(int k, bool guard, int threads, size_t bytes, int* ctas) {
     return pick(k, guard, [&](auto pol) {
-      const void* f = reinterpret_cast<const void*>(&sym_kernel<decltype(pol)>);
+      const void* f = reinterpret_cast<const void*>(&sym_kernel<decltype(pol), BATCHED>);
       const cudaError_t e = prepare_kernel(f, bytes);
       return e != cudaSuccess ? e : cudaOccupancyMaxActiveBlocksPerMultiprocessor(ctas, f, threads, bytes);
     });
@@ -632,15 +711,15 @@ struct SymTable {
   static cudaError_t launch(const SymArgs& a, const SymMerge& m, int k, bool guard, int threads, size_t bytes,
                             cudaStream_t s) {
     return pick(k, guard, [&](auto pol) {
-      const void* f = reinterpret_cast<const void*>(&sym_kernel<decltype(pol)>);
+      const void* f = reinterpret_cast<const void*>(&sym_kernel<decltype(pol), BATCHED>);
       cudaError_t e = prepare_kernel(f, bytes);
       if (e != cudaSuccess) return e;
       void* args[] = {const_cast<SymArgs*>(&a)};
       e = launch_pdl(f, dim3(static_cast<unsigned>(a.g.grid)), dim3(threads), args, bytes, s);
       if (e != cudaSuccess) return e;
       void* margs[] = {const_cast<SymMerge*>(&m)};
-      return launch_pdl(reinterpret_cast<const void*>(&sym_merge_kernel<decltype(pol)>),
-                        dim3(static_cast<unsigned>(m.g.n_blocks)), dim3(32 * kSymMergeWarps), margs, 0, s);
+      return launch_pdl(reinterpret_cast<const void*>(&sym_merge_kernel<decltype(pol), BATCHED>),
+                        dim3(static_cast<unsigned>(m.n_merge)), dim3(32 * kSymMergeWarps<BATCHED>), margs, 0, s);
     });
   }
   static SymOps ops(int max_k) { return SymOps{P2::kSumsI, max_k, &smem, &occupancy, &launch}; }

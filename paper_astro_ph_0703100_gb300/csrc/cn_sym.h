@@ -106,6 +106,82 @@ struct SymCursor {
   }
 };
 
+// An ensemble's rows: every cluster's own triangle, one after the other on
+// one cost line. Slots are kept for the off-diagonal blocks only.
+struct SymRow {
+  int64_t cost;      // cost line position of the row's first unit
+  int64_t p0;        // the cluster's first particle
+  int64_t slot;      // j-side slots: sum d of block b is at slot + d * plane + (b - diag_end) * 32
+  int32_t n;         // the cluster's particles
+  int32_t n_blocks;  // its blocks
+  int32_t blk0;      // the row's first block
+  int32_t diag_end;  // one past its last diagonal block
+  int32_t plane;     // (n_blocks - diag_end) * 32
+  float eps2;
+
+  __host__ __device__ int64_t length() const {
+    return static_cast<int64_t>(kSymCostDiag) * (diag_end - blk0) +
+           static_cast<int64_t>(kSymCostPair) * (n_blocks - diag_end);
+  }
+  // cost line position of its last unit
+  __host__ __device__ int64_t last() const {
+    return cost + length() - (diag_end < n_blocks ? kSymCostPair : kSymCostDiag);
+  }
+};
+
+// seek and take along an ensemble's rows (as SymCursor's own, by table)
+inline __host__ __device__ void sym_seek_rows(SymCursor& c, const SymRow* rows, int32_t n_rows, int64_t x) {
+  int32_t lo = 0, hi = n_rows - 1;
+  while (lo < hi) {
+    const int32_t mid = (lo + hi + 1) >> 1;
+    if (rows[mid].cost <= x)
+      lo = mid;
+    else
+      hi = mid - 1;
+  }
+  const SymRow r = rows[lo];
+  const int64_t left = x - r.cost, nd = r.diag_end - r.blk0;
+  int64_t idx;
+  if (left <= kSymCostDiag * nd)
+    idx = (left + kSymCostDiag - 1) / kSymCostDiag;
+  else
+    idx = nd + (left - kSymCostDiag * nd + kSymCostPair - 1) / kSymCostPair;
+  c.row = lo;
+  c.s = r.cost + (idx <= nd ? kSymCostDiag * idx : kSymCostDiag * nd + kSymCostPair * (idx - nd));
+  c.blk = r.blk0 + static_cast<int32_t>(idx);
+  if (c.blk >= r.n_blocks) {
+    ++c.row;
+    c.blk = c.row < n_rows ? rows[c.row].blk0 : 0;
+  }
+}
+inline __host__ __device__ void sym_take_rows(SymCursor& c, const SymRow* rows, int32_t n_rows, int64_t end,
+                                              int32_t most, int32_t* row, int32_t* blk, int32_t* count, bool* diag) {
+  const SymRow r = rows[c.row];
+  const bool dg = c.blk < r.diag_end;
+  const int64_t left = dg ? (end - c.s + kSymCostDiag - 1) / kSymCostDiag : (end - c.s + kSymCostPair - 1) / kSymCostPair;
+  int32_t n = (dg ? r.diag_end : r.n_blocks) - c.blk;
+  if (n > most) n = most;
+  if (n > left) n = static_cast<int32_t>(left);
+  *row = c.row;
+  *blk = c.blk;
+  *count = n;
+  *diag = dg;
+  c.s += static_cast<int64_t>(dg ? kSymCostDiag : kSymCostPair) * n;
+  c.blk += n;
+  if (c.blk >= r.n_blocks) {
+    ++c.row;
+    c.blk = c.row < n_rows ? rows[c.row].blk0 : 0;
+  }
+}
+
+// 32 particles of an ensemble in the merge: their block, their row and their
+// cluster's first row.
+struct SymMergeBlock {
+  int32_t first;
+  int32_t row;
+  int32_t blk;
+};
+
 // A launch. Sum d of the i side of particle p goes to plane d of the (CTA c,
 // row I) segment, slots_seg[((c + I - row0) * sums + d) * tile + p - I tile]
 // (c + I - row0 is unique per segment, since along the cost line neither the
@@ -124,6 +200,8 @@ struct SymArgs {
   int32_t stages;
   float eps2;
   uint64_t wait_ns;
+  const SymRow* rows;  // ensembles: the rows (g then holds only the cost line and the CTAs)
+  int32_t n_rows;
 };
 
 // Per-particle merge of one launch: the j-side slots of rows I < P (the
@@ -141,6 +219,9 @@ struct SymMerge {
   int32_t tile;
   int32_t first;
   int32_t last;
+  const SymRow* rows;            // ensembles
+  const SymMergeBlock* blocks;
+  int32_t n_merge;               // merge CTAs
 };
 
 enum SymForm : int {
@@ -149,6 +230,8 @@ enum SymForm : int {
   kSymJerk = 2,
   kSymJerkPot = 3,
   kSymAdjoint = 4,
+  kSymBatched = 5,
+  kSymBatchedPot = 6,
 };
 
 // A form's kernels: sums per particle, most particles per thread, shared
@@ -166,12 +249,15 @@ struct SymOps {
 SymOps sym_force_ops(bool pot);    // cn_sym.cu
 SymOps sym_jerk_ops(bool pot);     // cn_sym_jerk.cu
 SymOps sym_adjoint_ops();          // cn_sym_adjoint.cu
+SymOps sym_batched_ops(bool pot);  // cn_sym_batched.cu
 inline SymOps sym_ops(SymForm form) {
   switch (form) {
     case kSymForce: return sym_force_ops(false);
     case kSymForcePot: return sym_force_ops(true);
     case kSymJerk: return sym_jerk_ops(false);
     case kSymJerkPot: return sym_jerk_ops(true);
+    case kSymBatched: return sym_batched_ops(false);
+    case kSymBatchedPot: return sym_batched_ops(true);
     default: return sym_adjoint_ops();
   }
 }

@@ -24,6 +24,7 @@ struct SymAdjointPolicy {
   static constexpr int kSumsJ = 4;
   static constexpr int kRec = 2;
   static constexpr bool kGuard = false;
+  static constexpr int kUnroll = 8;
   static constexpr int kFold = 64;
   static constexpr int kMinBlocks = 2;
   static constexpr bool kWide = false;

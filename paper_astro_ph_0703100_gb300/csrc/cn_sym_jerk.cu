@@ -23,6 +23,7 @@ struct SymJerkPolicy {
   static constexpr int kSumsJ = kSumsI;
   static constexpr int kRec = 2;
   static constexpr bool kGuard = false;
+  static constexpr int kUnroll = K >= 8 ? 4 : 8;
   static constexpr int kFold = 256;
   static constexpr int kMinBlocks = 1;
   static constexpr bool kWide = true;

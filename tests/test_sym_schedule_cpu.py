@@ -1,5 +1,5 @@
 """The symmetric forms' work split (csrc/cn_sym.h), compiled for the host and
-enumerated: over tiles, sizes, CTA counts, stage sizes and bands, every unit
+enumerated: for one system and for an ensemble's table of rows, over tiles, sizes, CTA counts, stage sizes and bands, every unit
 (row of tiles, block) on or above the diagonal belongs to exactly one CTA,
 every CTA has one, no two segments share a slot, and the merge's view of
 which CTAs hold a row agrees."""
@@ -69,6 +69,61 @@ int main() {
       }
       ++launches;
     }
+  }
+  // ensembles: the rows of several clusters on one cost line
+  for (int64_t tile : {64, 512, 2048})
+  for (int set = 0; set < 4; ++set)
+  for (int slots : {1, 5, 152, 1216})
+  for (int most : {1, 2, 8}) {
+    const std::vector<std::vector<int>> sizes = {{1}, {700, 1, 33, 64, 2048, 31}, {5000, 512, 511, 513}, {32, 32, 32, 32}};
+    std::vector<SymRow> rows;
+    int64_t cost = 0, n = 0;
+    int c = 0;
+    for (int m : sizes[set]) {
+      const int nb = (m + 31) / 32, tb = tile / 32;
+      for (int b = 0; b < nb; b += tb) {
+        SymRow r{};
+        r.cost = cost; r.p0 = n; r.n = m; r.n_blocks = nb; r.blk0 = b; r.diag_end = std::min(nb, b + tb);
+        cost += r.length();
+        rows.push_back(r);
+      }
+      n += m;
+    }
+    SymGrid g{};
+    g.n = n; g.cost = cost; g.grid = std::max<int64_t>(1, std::min<int64_t>(slots, cost / kSymCostPair));
+    std::vector<std::vector<int>> own;
+    for (const SymRow& r : rows) own.push_back(std::vector<int>(r.n_blocks, -1));
+    std::vector<char> seg(g.grid + rows.size(), 0);
+    for (c = 0; c < g.grid; ++c) {
+      SymCursor cur;
+      sym_seek_rows(cur, rows.data(), rows.size(), g.part(c));
+      int units = 0, last = -1;
+      while (cur.s < g.part(c + 1)) {
+        const int64_t s0 = cur.s;
+        int32_t I, b, nb;
+        bool diag;
+        sym_take_rows(cur, rows.data(), rows.size(), g.part(c + 1), most, &I, &b, &nb, &diag);
+        CHECK(I >= 0 && I < (int)rows.size() && nb >= 1 && nb <= most && b >= rows[I].blk0 && b + nb <= rows[I].n_blocks)
+        for (int k = 0; k < nb; ++k, ++units) {
+          CHECK(own[I][b + k] == -1 && (b + k < rows[I].diag_end) == diag)
+          own[I][b + k] = c;
+          CHECK(g.owner(s0 + (int64_t)k * (diag ? kSymCostDiag : kSymCostPair)) == c)
+        }
+        if (I != last) {
+          CHECK(c + I < (int)seg.size() && !seg[c + I])
+          seg[c + I] = 1;
+          last = I;
+        }
+      }
+      CHECK(units > 0)
+    }
+    for (size_t I = 0; I < rows.size(); ++I) {
+      for (int b = 0; b < rows[I].n_blocks; ++b) CHECK((own[I][b] != -1) == (b >= rows[I].blk0))
+      CHECK(g.owner(rows[I].cost) == own[I][rows[I].blk0] && g.owner(rows[I].last()) == own[I].back())
+      for (int64_t o = g.owner(rows[I].cost); o <= g.owner(rows[I].last()); ++o)
+        CHECK(std::find(own[I].begin(), own[I].end(), (int)o) != own[I].end())
+    }
+    ++launches;
   }
   std::printf("ok %ld\n", launches);
   return 0;
