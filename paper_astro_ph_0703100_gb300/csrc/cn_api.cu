@@ -883,7 +883,7 @@ cn_status sym_fit(int dev, const DeviceInfo& d, cn::SymForm form, int64_t n, boo
   sp->k = guard ? 2 : std::min(ops.max_k, std::max(2, p.k));
   sp->threads = p.threads;
   sp->guard = guard;
-  sp->chunk = static_cast<int>(std::min<int64_t>(round_up(p.j_tile, cn::kSymBlock), 256));
+  sp->chunk = static_cast<int>(std::min<int64_t>(round_up(p.j_tile, cn::kSymBlock), ops.max_stage));
   sp->stages = std::max(2, p.stages);  // a stage is refilled a chunk after it was read
   sp->tile = static_cast<int64_t>(sp->k) * sp->threads;
   sp->tiles = ceil_div(n, sp->tile);

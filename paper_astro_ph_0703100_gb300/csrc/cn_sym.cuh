@@ -56,8 +56,6 @@ namespace cn {
 constexpr float kSymFar = 1e11f;       // |coordinate| up to which r^-3 stays a normal number
 constexpr float kSymSoft = 1e-20f;     // eps2 from which it stays finite
 
-constexpr int kSymMostStage = 256;     // records per stage, at most
-
 enum SymMode : int {
   kSymUniform = 0,  // equal masses, factored out of the pair terms
   kSymGeneral = 1,  // r^-3 times either mass
@@ -75,6 +73,7 @@ __device__ __forceinline__ float& sym_half(float2& v, int k) { return (k & 1) ? 
 //   kMinBlocks      256-thread CTAs per SM the registers are limited for
 //   kUnroll         steps per loop trip (divides 32)
 //   kFold           j records summed in FP32 registers between TwoSum folds
+//   kStage          records per stage, at most
 //   kWide           offers the kSymWide terms
 //   kSameMass       equal masses factor out only if the warp's and the
 //                   chunk's are the same
@@ -88,7 +87,7 @@ __device__ __forceinline__ float& sym_half(float2& v, int k) { return (k & 1) ? 
 // Force (and potential): per pair, d = x_j - x_i, s = |d|^2 + eps2, r =
 // s^-1/2; i: m_j r^3 d (and m_j r), j: -m_i r^3 d (and -m_i r). The
 // potential skips pairs at exactly zero separation.
-template <int K_, bool POT, bool GUARD, int UNROLL>
+template <int K_, bool POT, bool GUARD, int UNROLL, int FOLD = 512>
 struct SymForcePolicy {
   static constexpr int K = K_;
   static constexpr int P = K / 2;
@@ -97,7 +96,8 @@ struct SymForcePolicy {
   static constexpr int kRec = 1;
   static constexpr bool kGuard = GUARD;
   static constexpr int kUnroll = UNROLL;
-  static constexpr int kFold = 512;
+  static constexpr int kFold = FOLD;
+  static constexpr int kStage = FOLD < 256 ? FOLD : 256;
   static constexpr int kMinBlocks = 2;
   static constexpr bool kWide = true;
   static constexpr bool kSameMass = false;
@@ -541,7 +541,7 @@ __global__ void __launch_bounds__(256, Pol::kMinBlocks) sym_kernel(const __grid_
         }
       }
     };
-    if constexpr (Pol::kFold >= kSymMostStage) {
+    if constexpr (Pol::kFold >= Pol::kStage) {
       sweep(0, ch.nb);
     } else {
       for (int b0 = 0; b0 < ch.nb; b0 += kStep) sweep(b0, ch.nb - b0 < kStep ? ch.nb - b0 : kStep);
@@ -722,7 +722,7 @@ struct SymTable {
                         dim3(static_cast<unsigned>(m.n_merge)), dim3(32 * kSymMergeWarps<BATCHED>), margs, 0, s);
     });
   }
-  static SymOps ops(int max_k) { return SymOps{P2::kSumsI, max_k, &smem, &occupancy, &launch}; }
+  static SymOps ops(int max_k) { return SymOps{P2::kSumsI, max_k, P2::kStage, &smem, &occupancy, &launch}; }
 };
 
 }  // namespace cn

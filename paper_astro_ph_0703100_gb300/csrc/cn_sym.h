@@ -234,12 +234,14 @@ enum SymForm : int {
   kSymBatchedPot = 6,
 };
 
-// A form's kernels: sums per particle, most particles per thread, shared
+// A form's kernels: sums per particle, most particles per thread and records
+// per stage, shared
 // memory of a shape, resident CTAs per SM, and the launch of one band (pair
 // kernel and merge).
 struct SymOps {
   int sums;
   int max_k;
+  int max_stage;
   size_t (*smem)(int threads, int k, int chunk, int stages);
   cudaError_t (*occupancy)(int k, bool guard, int threads, size_t smem, int* ctas);
   cudaError_t (*launch)(const SymArgs& a, const SymMerge& m, int k, bool guard, int threads, size_t smem,

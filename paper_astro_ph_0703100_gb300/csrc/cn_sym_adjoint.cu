@@ -26,6 +26,7 @@ struct SymAdjointPolicy {
   static constexpr bool kGuard = false;
   static constexpr int kUnroll = 8;
   static constexpr int kFold = 64;
+  static constexpr int kStage = 256;
   static constexpr int kMinBlocks = 2;
   static constexpr bool kWide = false;
   static constexpr bool kSameMass = true;

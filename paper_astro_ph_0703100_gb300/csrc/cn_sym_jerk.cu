@@ -25,6 +25,7 @@ struct SymJerkPolicy {
   static constexpr bool kGuard = false;
   static constexpr int kUnroll = K >= 8 ? 4 : 8;
   static constexpr int kFold = 256;
+  static constexpr int kStage = 256;
   static constexpr int kMinBlocks = 1;
   static constexpr bool kWide = true;
   static constexpr bool kSameMass = false;
