@@ -4,6 +4,7 @@
 #include "cunbody.h"
 #include "cn_guard.h"
 #include "cn_kernels.h"
+#include "cn_rows.h"
 #include "cn_sym.h"
 
 #include <nvtx3/nvToolsExt.h>
@@ -1009,6 +1010,104 @@ Plan sym_default_plan(cn::SymForm form, int64_t n, int sms) {
   return p;
 }
 
+// ------------------------------------------------------------------ one-sided rows
+struct RowPlan {
+  int k = 0, wi = 0, chunk = 0, stages = 0;
+  size_t smem = 0, need = 0;
+  int64_t tile = 0, rows = 0, blocks = 0, units = 0;
+  int grid = 0;
+};
+
+// Shape of the row kernel. Small tiles (four particles per thread, all warps
+// on the same 128) waste the least on small sets: 4000 x 16384 31.6 us against
+// 32.6 for 8 x 32 and 56 for eight warps along i. Large plain sets take eight
+// per thread (2048 x 262144 209 against 213 us); with the potential or
+// per-particle softening the registers of four suit better, and the latter's
+// large sets take the warps along i (32768 x 32768 with the potential 461 us,
+// 466 with all warps on the same, 482 with eight per thread).
+cn_status rows_fit(int dev, const DeviceInfo& d, cn::RowForm form, int64_t n_i, int64_t n_j, RowPlan* rp) {
+  const double pairs = static_cast<double>(n_i) * static_cast<double>(n_j);
+  rp->k = form == cn::kRowForce && pairs >= 1.5e8 ? 8 : 4;
+  rp->wi = form != cn::kRowForce && pairs >= 5e8 && n_i >= 16384 ? 8 : 1;
+  rp->stages = 3;
+  rp->chunk = rp->wi == 8 ? 256 : 1024;
+  rp->tile = static_cast<int64_t>(32) * rp->k * rp->wi;
+  rp->rows = ceil_div(n_i, rp->tile);
+  rp->blocks = ceil_div(n_j, cn::kRowBlock);
+  rp->units = rp->rows * rp->blocks;
+  if (rp->rows > INT32_MAX / 2 || rp->blocks > INT32_MAX / 2) return fail(CN_ERR_INVALID_ARG, "problem too large for one launch");
+  rp->smem = cn::rows_smem_bytes(form, rp->k, rp->chunk, rp->stages);
+  const auto key = std::make_tuple(dev, 2000 + static_cast<int>(form), false, 1, rp->k, 256, rp->smem);
+  int occ = 0;
+  {
+    std::lock_guard<std::mutex> lock(g_mu);
+    auto it = g_occ.find(key);
+    if (it != g_occ.end()) occ = it->second;
+  }
+  if (occ == 0) {
+    const cudaError_t e = cn::occupancy_rows(form, rp->k, rp->smem, &occ);
+    if (e != cudaSuccess) return fail_cuda(e, "cudaOccupancyMaxActiveBlocksPerMultiprocessor");
+    if (occ <= 0) return fail(CN_ERR_INVALID_ARG, "launch shape does not fit on one SM");
+    std::lock_guard<std::mutex> lock(g_mu);
+    g_occ[key] = occ;
+  }
+  rp->grid = static_cast<int>(std::min<int64_t>(static_cast<int64_t>(occ) * d.sms, rp->units));
+  const bool pot = form == cn::kRowForcePot || form == cn::kRowEpsIPot;
+  rp->need = static_cast<size_t>(2) * rp->grid * (pot ? 4 : 3) * rp->tile * sizeof(float);
+  return CN_OK;
+}
+
+cn_status rows_launch(const std::string& what, const DeviceInfo& d, cn::RowForm form, const RowPlan& rp, int64_t n_i,
+                      const float* pos_i, int64_t n_j, const float* pos_j, float eps2, float* acc_out, float* pot_out,
+                      char* data, cudaStream_t s) {
+  cn::RowArgs a{};
+  a.pos_i = reinterpret_cast<const float4*>(pos_i);
+  a.pos_j = reinterpret_cast<const float4*>(pos_j);
+  a.acc_out = acc_out;
+  a.pot_out = pot_out;
+  a.segs = reinterpret_cast<float*>(data);
+  a.status = d.status;
+  a.n_i = n_i;
+  a.n_j = n_j;
+  a.units = rp.units;
+  a.n_rows = static_cast<int32_t>(rp.rows);
+  a.blocks = static_cast<int32_t>(rp.blocks);
+  a.grid = rp.grid;
+  a.tile = static_cast<int32_t>(rp.tile);
+  a.wi = rp.wi;
+  a.chunk = rp.chunk;
+  a.stages = rp.stages;
+  a.eps2 = eps2;
+  a.wait_ns = g_wait_ns.load();
+  if (log_enabled())
+    std::fprintf(stderr, "[cunbody] %s | rows: K %d tile %lld rows %lld chunk %d stages %d | units %lld grid %d smem %zu ws %zu\n",
+                 what.c_str(), rp.k, static_cast<long long>(rp.tile), static_cast<long long>(rp.rows), rp.chunk, rp.stages,
+                 static_cast<long long>(rp.units), rp.grid, rp.smem, rp.need);
+  if (inject("launch")) return fail(CN_ERR_CUDA, "kernel launch: injected launch failure");
+  const cudaError_t e = cn::launch_rows(form, rp.k, a, rp.smem, s);
+  return e == cudaSuccess ? CN_OK : fail_cuda(e, "row kernel launch");
+}
+
+// Whether the row kernel is the faster one for any masses, on a device with
+// `sms` multiprocessors (pairs and particles counted per SM). Below 2.4e7 pairs
+// the pair kernel's small shapes are (4500 x 4500 15.6 us against 17.6, 8192 x
+// 2500 15.7 / 17.8), and fewer than 128 i-particles leave lanes idle (40 x
+// 600000 38.2 / 60.8). Above, with per-particle softening always (5000 x 5000
+// 22.5 / 19.3 us, 65536 x 65536 1713 / 1634). Plain sets and those with the
+// potential: the middle is the row kernel's (300 x 70000 31.7 / 27.4, 4000 x
+// 16384 39.8 / 33.6, 2048 x 262144 241 / 211, 8192 x 8192 36.3 / 34.9, 7000 x
+// 20000 66.6 / 63.3), and large sets keep the pair kernel (8192 x 100003 309 /
+// 320, 10007 x 100003 376 / 388, 16384 x 16384 108.1 / 109.5): unequal masses
+// throughout.
+bool rows_pays(cn::RowForm form, int64_t n_i, int64_t n_j, int sms) {
+  const double share = 152.0 / std::max(sms, 1);
+  const double pairs = static_cast<double>(n_i) * static_cast<double>(n_j) * share;
+  if (n_i < 128 || pairs < 2.4e7) return false;
+  if (form == cn::kRowEpsI || form == cn::kRowEpsIPot) return true;
+  const double rows = static_cast<double>(n_i) * share;
+  return (rows <= 4096.0 && pairs <= 5.5e8) || (rows <= 8192.0 && pairs <= 1.5e8);
+}
+
 // ------------------------------------------------------------------ single-system force
 // eps_i: the softening of each pair is its i-particle's, from the 4th slot
 // of its record (eps2 is not used); the kernels then always take the s = 0
@@ -1048,21 +1147,26 @@ cn_status force_common(bool dd, int64_t n_i, const float* pos_i, int64_t n_j, co
   // One set against itself: each unordered pair once (the i record's 4th slot
   // is then the same mass the j side reads).
   const bool self = !dd && !eps_i && !guard && pos_i == pos_mass_j && n_i == n_j && sym_pays(cn::kSymForce, n_i, d->sms);
+  const cn::RowForm row_form =
+      eps_i ? (pot ? cn::kRowEpsIPot : cn::kRowEpsI) : (pot ? cn::kRowForcePot : cn::kRowForce);
+  const bool apart = !dd && (eps_i || !guard) && !self && rows_pays(row_form, n_i, n_j, d->sms);
   struct Cached {
     PlanCache key;
     bool sym = false;
+    bool rows = false;
     SymPlan sp;
+    RowPlan rp;
     Plan p;
     Geometry g;
     char* ctrl = nullptr;
     char* data = nullptr;
   };
-  thread_local Cached t_last;
-  Cached now;
+  thread_local Cached t_last, t_now;  // of the last call; of a call that is planned anew
   const int key = variant + (self ? 64 : 0);
   const uint64_t gen0 = g_plan_gen.load(std::memory_order_acquire);
   const Cached* c = &t_last;
   if (!(lib_ws && t_last.key.hit(gen0, dev, key, n_i, n_j, guard, s))) {
+    Cached& now = t_now = Cached{};
     c = &now;
     const uint64_t bumps0 = t_own_bumps;
     // the per-particle kernels are guarded in every shape, so K is not
@@ -1081,12 +1185,28 @@ cn_status force_common(bool dd, int64_t n_i, const float* pos_i, int64_t n_j, co
       now.sym = true;
       now.sp.data = static_cast<char*>(ws);
     }
-    if (!now.sym && (st = launch_workspace(s, now.g, ws, ws_bytes, lib_ws, &now.ctrl, &now.data)) != CN_OK) return st;
+    bool wanted_rows = apart && !registered_tune(dev, variant, n_i, n_j);
+    if (wanted_rows) wanted_rows = rows_fit(dev, *d, row_form, n_i, n_j, &now.rp) == CN_OK;
+    if (wanted_rows && lib_ws) {
+      now.rows = sym_workspace(s, now.rp.need, &now.data) == CN_OK;
+    } else if (wanted_rows && ws && aligned(ws, 256) && ws_bytes >= std::max(now.rp.need, now.g.ws_bytes)) {
+      now.rows = true;
+      now.data = static_cast<char*>(ws);
+    }
+    // The library's workspace of the one-sided kernel is there after any call
+    // of these sizes, also one that did without it: a capture may then make
+    // a call that has to fall back on it.
+    if (!now.sym && !now.rows) {
+      if ((st = launch_workspace(s, now.g, ws, ws_bytes, lib_ws, &now.ctrl, &now.data)) != CN_OK) return st;
+    } else if (lib_ws) {
+      char *ctrl = nullptr, *data = nullptr;
+      library_workspace(s, now.g.ctrl_bytes, now.g.data_bytes, &ctrl, &data);
+    }
     // cache only a plan that nothing changed under (another thread's tuning
     // or workspace change would show as a generation step not our own), and
     // not one that had to do without its slots
     const uint64_t gen1 = g_plan_gen.load(std::memory_order_acquire);
-    if (lib_ws && now.sym == wanted && gen1 == gen0 + (t_own_bumps - bumps0)) {
+    if (lib_ws && now.sym == wanted && now.rows == wanted_rows && gen1 == gen0 + (t_own_bumps - bumps0)) {
       now.key = PlanCache{true, gen1, dev, key, n_i, n_j, guard, s};
       t_last = now;
     }
@@ -1098,6 +1218,14 @@ cn_status force_common(bool dd, int64_t n_i, const float* pos_i, int64_t n_j, co
       what = std::string("cn_force: variant ") + variant_name(variant) + " n_i " + std::to_string(n_i) + " n_j " +
              std::to_string(n_j);
     return sym_launch(what, *d, pot ? cn::kSymForcePot : cn::kSymForce, c->sp, n_i, pos_i, nullptr, eps2, out, s);
+  }
+  if (c->rows) {
+    std::string what;
+    if (log_enabled())
+      what = std::string(eps_i ? "cn_force_eps_i" : "cn_force") + ": variant " + variant_name(variant) + " n_i " +
+             std::to_string(n_i) + " n_j " + std::to_string(n_j);
+    return rows_launch(what, *d, row_form, c->rp, n_i, pos_i, n_j, pos_mass_j, eps2, static_cast<float*>(acc_out),
+                       static_cast<float*>(pot_out), c->data, s);
   }
   const Plan& p = c->p;
   const Geometry& g = c->g;
@@ -1131,6 +1259,13 @@ const SymPlan* sym_self_plan(int dev, const DeviceInfo& d, cn::SymForm form, int
   t_last.key.valid = false;
   if (sym_fit(dev, d, form, n, false, sym_default_plan(form, n, d.sms), &t_last) != CN_OK) return nullptr;
   if (sym_workspace(s, t_last.need + extra, &t_last.data) != CN_OK) return nullptr;
+  // the one-sided kernel's workspace too, for a later call that has to fall back on it during a capture
+  Plan one;
+  Geometry g;
+  char *ctrl = nullptr, *data = nullptr;
+  if (resolve_plan(dev, variant, n, n, false, nullptr, &one) == CN_OK &&
+      single_geometry(dev, d, variant, false, one, n, n, &g) == CN_OK)
+    library_workspace(s, g.ctrl_bytes, g.data_bytes, &ctrl, &data);
   const uint64_t gen1 = g_plan_gen.load(std::memory_order_acquire);
   t_last.key = PlanCache{gen1 == gen0 + (t_own_bumps - bumps0), gen1, dev, form, n, n, false, s};
   return &t_last;
@@ -2044,18 +2179,25 @@ cn_status cn_force_dd_ws(int64_t n_i, const float* pos_i, int64_t n_j, const flo
 
 size_t cn_workspace_bytes(int variant, int64_t n_i, int64_t n_j) {
   return cn::guard_value<size_t>(0, [&]() -> size_t {
-    const size_t need = cn::one_sided_workspace_bytes(variant, n_i, n_j);
-    if (need == 0 || (variant != cn::kF32 && variant != cn::kF32Pot) || n_i != n_j) return need;
-    // one set against itself: the symmetric form's slots (a smaller buffer
-    // that holds the above is accepted, and takes the one-sided kernel)
+    size_t need = cn::one_sided_workspace_bytes(variant, n_i, n_j);
+    if (need == 0 || (variant != cn::kF32 && variant != cn::kF32Pot)) return need;
+    // the slots of the symmetric form (one set against itself) and the
+    // segments of the row kernel; a smaller buffer that holds the above is
+    // accepted, and takes the pair kernel
     int dev = 0;
     DeviceInfo* d = nullptr;
-    if (current_device(&dev, &d) != CN_OK || !sym_pays(cn::kSymForce, n_i, d->sms) || registered_tune(dev, variant, n_i, n_j))
-      return need;
-    const cn::SymForm form = variant == cn::kF32Pot ? cn::kSymForcePot : cn::kSymForce;
+    if (current_device(&dev, &d) != CN_OK || registered_tune(dev, variant, n_i, n_j)) return need;
+    const bool pot = variant == cn::kF32Pot;
+    const cn::SymForm form = pot ? cn::kSymForcePot : cn::kSymForce;
+    const cn::RowForm rows = pot ? cn::kRowForcePot : cn::kRowForce;
     SymPlan sp;
-    if (sym_fit(dev, *d, form, n_i, false, sym_default_plan(form, n_i, d->sms), &sp) != CN_OK) return need;
-    return std::max(need, sp.need);
+    if (n_i == n_j && sym_pays(form, n_i, d->sms) &&
+        sym_fit(dev, *d, form, n_i, false, sym_default_plan(form, n_i, d->sms), &sp) == CN_OK)
+      need = std::max(need, sp.need);
+    RowPlan rp;
+    if (rows_pays(rows, n_i, n_j, d->sms) && rows_fit(dev, *d, rows, n_i, n_j, &rp) == CN_OK)
+      need = std::max(need, rp.need);
+    return need;
   });
 }
 

@@ -81,11 +81,13 @@ def test_first_call_inside_a_capture():
     torch = torch_cuda()
     n = 7000
     d = dev_tensor(synth.plummer(n, 4))
-    one, _ = cn.cn_force(d, d.clone(), 1e-3)
+    cn.cn_tune_set("f32", n, n, cn.cn_tune_get("f32", n, n))
+    one, _ = cn.cn_force(d, d, 1e-3)  # the one-sided kernel
+    cn.cn_tune_set("f32", n, n, None)
     s = torch.cuda.Stream()
     out = torch.zeros((n, 3), device="cuda")
     with torch.cuda.stream(s):
-        cn.cn_force(d, d.clone(), 1e-3)  # the one-sided workspace of this stream
+        cn.cn_force(d, d.clone(), 1e-3)
         torch.cuda.synchronize()
         g = torch.cuda.CUDAGraph()
         with torch.cuda.graph(g, stream=s):
