@@ -164,9 +164,60 @@ def _variant(name):
     return VARIANT[name] if isinstance(name, str) else int(name)
 
 
+# ------------------------------------------------------------------ native marshalling
+
+_native = None  # the compiled marshalling, False where there is none
+
+
+def _load_native():
+    """The compiled marshalling (csrc/cn_binding.cpp) if it was built for this
+    PyTorch, else False: the calls below then marshal in Python."""
+    global _native
+    torch = _torch()
+    try:
+        from . import _binding
+
+        _native = _binding if _binding.torch_version == str(torch.__version__) else False
+    except ImportError:
+        _native = False
+    return _native
+
+
+def _call_native(fn, double, pos_i, pos_mass_j, eps2, acc, pot, potential, stream):
+    """The call of entry point `fn` (eps2: a tuple of that argument, empty for
+    cn_force_eps_i) through the compiled marshalling: (status or
+    -1 where that declines the call, acc, pot). cn_force on 1024 particles
+    with given outputs and potential takes 7.4 us a call without it, 2.7
+    with it; on 2048, without potential, 6.6 / 3.7."""
+    native = _native if _native is not None else _load_native()
+    if native is False:
+        return -1, acc, pot
+    if acc is None or (potential and pot is None):
+        n = native.rows(pos_i, pos_mass_j)
+        if n < 0:
+            return -1, acc, pot
+        torch = _torch()
+        dt = torch.float64 if double else torch.float32
+        if acc is None:
+            acc = torch.empty((n, 3), dtype=dt, device=pos_i.device)
+        if potential and pot is None:
+            pot = torch.empty((n,), dtype=dt, device=pos_i.device)
+    if stream is not None:
+        stream = int(stream.cuda_stream)
+    call = native.force if eps2 else native.force_eps_i
+    return call(load().addresses[fn], double, pos_i, pos_mass_j, *eps2, acc, pot, stream), acc, pot
+
+
 # ------------------------------------------------------------------ force
 
 def _force(fn, double, pos_i, pos_mass_j, eps2, acc_out, pot_out, potential, stream, ws=None):
+    if ws is None:
+        st, acc_out, pot_out = _call_native(fn, double, pos_i, pos_mass_j, (eps2,), acc_out, pot_out, potential,
+                                            stream)
+        if st == 0:
+            return acc_out, pot_out
+        if st > 0:
+            check(st, fn)
     torch = _torch()
     _records(pos_i, "pos_i")
     _records(pos_mass_j, "pos_mass_j")
@@ -196,6 +247,12 @@ def cn_force(pos_i, pos_mass_j, eps2, acc_out=None, pot_out=None, potential=Fals
 def cn_force_eps_i(pos_eps_i, pos_mass_j, acc_out=None, pot_out=None, potential=False, stream=None):
     """FP32 accelerations (and potentials) with each i-particle's softening
     eps2_i taken from the 4th slot of its record (x, y, z, eps2_i)."""
+    st, acc_out, pot_out = _call_native("cn_force_eps_i", False, pos_eps_i, pos_mass_j, (), acc_out, pot_out,
+                                        potential, stream)
+    if st == 0:
+        return acc_out, pot_out
+    if st > 0:
+        check(st, "cn_force_eps_i")
     torch = _torch()
     _records(pos_eps_i, "pos_eps_i")
     _records(pos_mass_j, "pos_mass_j")

@@ -4,16 +4,22 @@ Each ``csrc/*.cu`` translation unit is compiled in parallel into
 ``_build/``; the objects are linked into ``libcunbody.so`` next to this
 file (the CUDA runtime is linked statically, so the library loads without
 a CUDA runtime on the library path). Rebuilds only when a source or
-header is newer than the library.
+header is newer than the library. ``csrc/cn_binding.cpp``, the native part of
+the Python binding, is compiled beside it against the installed PyTorch;
+where that cannot be done the binding marshals in Python.
 """
 
 from __future__ import annotations
 
 import concurrent.futures as cf
 import glob
+import importlib.util
 import os
+import re
 import shutil
 import subprocess
+import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
@@ -24,6 +30,8 @@ LIB = os.path.join(HERE, "libcunbody.so")
 # debug variant: every schedule index checked on the device (CN_DEBUG_BOUNDS)
 DEBUG_BUILD_DIR = os.path.join(HERE, "_build_debug")
 DEBUG_LIB = os.path.join(HERE, "libcunbody_debug.so")
+BINDING_SRC = os.path.join(CSRC, "cn_binding.cpp")
+BINDING = os.path.join(HERE, "_binding.so")
 
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 NVCC_FLAGS = ["-O3", "-std=c++17", "-lineinfo", "-ftz=true", "-Xcompiler", "-fPIC,-O2,-fvisibility=hidden",
@@ -79,5 +87,35 @@ def build(force: bool = False, verbose: bool = False, debug_bounds: bool = False
     return lib
 
 
+def build_binding(force: bool = False):
+    """Compile _binding.so against the installed PyTorch (nothing of it is
+    imported); returns its path, or None where that cannot be done."""
+    spec = importlib.util.find_spec("torch")
+    if spec is None or not spec.submodule_search_locations:
+        return None
+    home = spec.submodule_search_locations[0]
+    try:
+        with open(os.path.join(home, "version.py")) as f:
+            version = re.search(r"__version__ = ['\"]([^'\"]+)", f.read()).group(1)
+        inputs = [BINDING_SRC, os.path.abspath(__file__), os.path.join(home, "version.py")]
+        if not force and os.path.exists(BINDING) and os.path.getmtime(BINDING) >= max(map(os.path.getmtime, inputs)):
+            return BINDING
+        cuda = os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(nvcc()))), "include")
+        tmp = BINDING + f".tmp{os.getpid()}"
+        cmd = ["g++", "-O2", "-std=c++17", "-fPIC", "-shared", "-fvisibility=hidden", "-w",
+               f'-DCN_TORCH_VERSION="{version}"', "-I", sysconfig.get_paths()["include"],
+               "-I", os.path.join(home, "include"), "-I", cuda, BINDING_SRC, "-o", tmp,
+               "-L", os.path.join(home, "lib"), "-ltorch_python", "-ltorch_cpu", "-lc10", "-lc10_cuda"]
+        res = subprocess.run(cmd, capture_output=True, text=True)
+        if res.returncode != 0:
+            raise RuntimeError(res.stderr[-2000:])
+        os.replace(tmp, BINDING)
+        return BINDING
+    except (OSError, AttributeError, RuntimeError) as e:
+        print(f"the native part of the Python binding was not built: {e}", file=sys.stderr)
+        return None
+
+
 if __name__ == "__main__":
+    build_binding(force=True)
     print(build(force=True, verbose=True))

@@ -123,6 +123,7 @@ def load(path: str | None = None):
             fn = getattr(lib, name)
             fn.restype = res
             fn.argtypes = args
+        lib.addresses = {name: ctypes.cast(getattr(lib, name), vp).value for name in SIGNATURES}
         _lib = lib
         return lib
 
