@@ -187,8 +187,8 @@ def _call_native(fn, double, pos_i, pos_mass_j, eps2, acc, pot, potential, strea
     """The call of entry point `fn` (eps2: a tuple of that argument, empty for
     cn_force_eps_i) through the compiled marshalling: (status or
     -1 where that declines the call, acc, pot). cn_force on 1024 particles
-    with given outputs and potential takes 7.4 us a call without it, 2.7
-    with it; on 2048, without potential, 6.6 / 3.7."""
+    with given outputs and potential takes 7.4 us of host time without it,
+    2.7 with it."""
     native = _native if _native is not None else _load_native()
     if native is False:
         return -1, acc, pot

@@ -15,7 +15,7 @@
 // this takes 24 shuffles and 24 additions per 8 records to 48 shuffles and
 // none, which leaves the FP32 pipe to the pair terms (inner loop at K = 8 x
 // 256 threads, 2.07 GHz: 1.93e12 -> 2.03e12 unordered pairs/s; whole calls at
-// N = 131072 with equal masses: 4653 -> 4000 us).
+// N = 131072 with equal masses: 4653 -> 4015 us).
 //
 // What bounds the loop: the FP32 pipe, and with it the register file. A
 // packed multiply-add whose three operands are different registers issues
@@ -36,7 +36,9 @@
 // Shared memory per CTA: a ring of staged chunks (bulk copies), three buffers
 // of the j-side sums of a chunk, one row per warp, and the i-side (hi, lo)
 // sums of the current row of tiles, folded from registers every kFold
-// records by TwoSum. The warps are not held together by a barrier: a warp
+// records by TwoSum (force: 512 are 0.4% faster at N = 131072 and 0.8% at 50001,
+// but leave a larger error than the reduce-scatter form did: with the potential
+// 4.8e-8 against 4.1e-8 at 9836, 256 4.0e-8). The warps are not held together by a barrier: a warp
 // that has swept chunk k waits for the "done" barrier of chunk k - 1 (long
 // complete unless a warp is a whole chunk behind), adds up its share of
 // chunk k - 1's rows and arrives on chunk k's barrier. A __syncthreads per
@@ -87,7 +89,7 @@ __device__ __forceinline__ float& sym_half(float2& v, int k) { return (k & 1) ? 
 // Force (and potential): per pair, d = x_j - x_i, s = |d|^2 + eps2, r =
 // s^-1/2; i: m_j r^3 d (and m_j r), j: -m_i r^3 d (and -m_i r). The
 // potential skips pairs at exactly zero separation.
-template <int K_, bool POT, bool GUARD, int UNROLL, int FOLD = 512>
+template <int K_, bool POT, bool GUARD, int UNROLL, int FOLD = 256>
 struct SymForcePolicy {
   static constexpr int K = K_;
   static constexpr int P = K / 2;

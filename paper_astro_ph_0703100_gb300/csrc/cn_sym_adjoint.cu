@@ -12,7 +12,8 @@ namespace {
 // operations per unordered pair; where the warp's and the chunk's masses are
 // all the same, u is w_j - w_i times that mass and d . u is a + b: 31; against
 // 2 x 30 for the ordered pairs. The sums cancel heavily (the weights are
-// signed): registers are folded into the (hi, lo) sums every kFold records,
+// signed): registers are folded into the (hi, lo) sums every 32 records (64: 2.7%
+// faster at N = 65536, gradient error 1.98e-7 for 1.84e-7, one-sided 1.94e-7),
 // and a travelling sum takes 32 K / 2 terms per half before it is joined.
 // The pair of a particle with itself is skipped by its index (u of the
 // general term rounds to a residual there).
@@ -25,7 +26,7 @@ struct SymAdjointPolicy {
   static constexpr int kRec = 2;
   static constexpr bool kGuard = false;
   static constexpr int kUnroll = 8;
-  static constexpr int kFold = 64;
+  static constexpr int kFold = 32;
   static constexpr int kStage = 256;
   static constexpr int kMinBlocks = 2;
   static constexpr bool kWide = false;
