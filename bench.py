@@ -3,12 +3,13 @@
 
 One step = one evaluation of the accelerations of an equal-mass Plummer
 sphere of N = 131072 particles (i set = j set, eps = 4 / N^(1/3), FP32
-records) with the plain FP32 kernel: N^2 pair interactions. The headline
+records): N^2 pair interactions, which the library resolves from the N (N + 1) / 2
+unordered pairs of the set. The headline
 value is pair interactions per second over the K timed steps (CUDA events
 on the launching stream, L2 flushed between steps by writing 256 MiB).
 Beside it the line reports the compensated form (FP32 pair with its
 roundings recovered, (hi, lo) sums, FP64 folds) on the
-same input, the roofline fraction of the pair kernel, the end-to-end rate
+same input, the roofline fraction of the kernel, the end-to-end rate
 through the host-buffer C-ABI call (copies included), and the FP64 oracle
 timed on the host cores on a bounded sample of the same workload.
 
@@ -38,10 +39,12 @@ METRIC = "pair interactions/s and % of FP32/MUFU roofline at N=131072, FP32 vs c
 UNIT = "pairs/s"
 N_DEFAULT = 131072
 FLOP_PER_PAIR = 38  # the paper's counting convention (Eq. 4)
-# The plain kernel issues its FP32 work as packed f32x2 instructions (6 per
-# pair + 1 MUFU), so the bound is the FP32 pipe: 12 lane operations per pair
-# at 128 lanes per SM per clock.
+# The kernels issue their FP32 work as packed f32x2 instructions, so the bound
+# is the FP32 pipe at 128 lanes per SM per clock. One set on another: 12 lane
+# operations per pair. One set on itself: 14 per unordered pair where all masses
+# of a warp and a chunk are equal (they are factored out), 16 otherwise.
 FP32_LANE_OPS_PER_PAIR = 12
+SYM_LANE_OPS_PER_UNORDERED_PAIR = {"equal": 14, "unequal": 16}
 FP32_LANES_PER_SM = 128
 SM_MAX_MHZ = 2070.0
 PAPER_PAIRS_PER_S = 256e9 / FLOP_PER_PAIR  # 8800GTX, N = 131072 (Table 3): context only
@@ -169,8 +172,8 @@ def gpu_selector(torch, device):
 
 # ------------------------------------------------------------------ profile evidence
 
-KERNEL_SOURCES = ("cn_pair.cuh", "cn_device.cuh", "cn_kernels.h", "cn_force_f32.cu")
-PROFILE_F32 = os.path.join(ROOT, "profiles", "pair_f32_n131072.json")
+KERNEL_SOURCES = ("cn_sym.cuh", "cn_sym.h", "cn_device.cuh", "cn_kernels.h", "cn_sym.cu")
+PROFILE_F32 = os.path.join(ROOT, "profiles", "sym_n131072.json")
 
 
 def kernel_source_hash() -> str:
@@ -185,7 +188,7 @@ def kernel_source_hash() -> str:
 
 def profiled_traffic(shape: dict):
     """DRAM bytes per launch from the committed ncu record of the headline
-    kernel (profiles/pair_f32_n131072.json), if it was taken on the kernel
+    kernel (profiles/sym_n131072.json), if it was taken on the kernel
     sources as they are now and in this launch shape; else None."""
     try:
         with open(PROFILE_F32) as f:
@@ -278,6 +281,7 @@ def run_ours(args):
     acc_dd = torch.empty((n, 3), dtype=torch.float64, device=device)
 
     tuned = tuned_dd = None
+    ws_default = cn.cn_workspace_bytes("f32", n, n)
     if args.autotune:
         tuned = cn.cn_autotune("f32", t, t, eps2, reps=2)
         tuned_dd = cn.cn_autotune("dd", t, t, eps2, reps=1)
@@ -325,7 +329,13 @@ def run_ours(args):
     pairs = float(n) * float(n)
     value = aggregate_rate(pairs * args.steps, world, total_s)
     sms = torch.cuda.get_device_properties(device).multi_processor_count
-    peak = sms * FP32_LANES_PER_SM * SM_MAX_MHZ * 1e6 / FP32_LANE_OPS_PER_PAIR
+    lane_rate = sms * FP32_LANES_PER_SM * SM_MAX_MHZ * 1e6
+    pair_peak = lane_rate / FP32_LANE_OPS_PER_PAIR
+    # each unordered pair once above 4096 particles, unless a one-sided shape was registered (its workspace is smaller)
+    symmetric = n > 4096 and cn.cn_workspace_bytes("f32", n, n) == ws_default
+    lane_ops = SYM_LANE_OPS_PER_UNORDERED_PAIR["equal"] / 2 if symmetric else FP32_LANE_OPS_PER_PAIR
+    peak = lane_rate / lane_ops
+    shape = cn.cn_tune_get("symmetric" if symmetric else "f32", n, n)
     achieved = pairs / mean_kernel_s
     dd_rate = pairs / dd_mean_s
     peaks = cn.cn_probe_peaks()
@@ -350,7 +360,7 @@ def run_ours(args):
             "eps2": eps2,
             "pairs_per_step": pairs,
             "l2": "flushed between timed steps (256 MiB write outside the events); inputs 2 MiB",
-            "launch_shape_f32": tuned or cn.cn_tune_get("f32", n, n),
+            "launch_shape_f32": shape,
             "launch_shape_dd": tuned_dd or cn.cn_tune_get("dd", n, n),
         },
         "gflops_at_38": value * FLOP_PER_PAIR / 1e9,
@@ -360,11 +370,12 @@ def run_ours(args):
             "peak": peak / 1e9,
             "unit": "Gpair/s",
             "frac": achieved / peak,
-            "traffic": profiled_traffic(tuned or cn.cn_tune_get("f32", n, n)),
+            "traffic": profiled_traffic(shape),
             "peak_basis": f"{sms} SMs x {FP32_LANES_PER_SM} FP32 lanes x {SM_MAX_MHZ:.0f} MHz / "
-                          f"{FP32_LANE_OPS_PER_PAIR} FP32 lane operations per pair (packed f32x2 issue)",
+                          f"{lane_ops:g} FP32 lane operations per ordered pair (packed f32x2 issue"
+                          + (", each unordered pair once, equal masses factored out)" if symmetric else ")"),
             "frac_at_observed_clock": achieved / (peak * obs_mhz / SM_MAX_MHZ),
-            "frac_of_probe_ffma_rate": achieved * FP32_LANE_OPS_PER_PAIR / peaks["ffma_per_s"],
+            "frac_of_probe_ffma_rate": achieved * lane_ops / peaks["ffma_per_s"],
             "probe_scalar_pair_mix": peaks["pair_mix_per_s"] / 1e9,
             "probe_ffma_per_s": peaks["ffma_per_s"],
             "probe_mufu_per_s": peaks["mufu_rsqrt_per_s"],
@@ -373,8 +384,8 @@ def run_ours(args):
             "value": dd_rate * world,
             "unit": UNIT,
             "ms_per_step": 1e3 * dd_mean_s,
-            "frac_of_fp32_peak": dd_rate / peak,
-            "frac_of_own_roofline": dd_rate / (peak * FP32_LANE_OPS_PER_PAIR / DD_LANE_OPS_PER_PAIR),
+            "frac_of_fp32_peak": dd_rate / pair_peak,
+            "frac_of_own_roofline": dd_rate / (lane_rate / DD_LANE_OPS_PER_PAIR),
             "own_roofline_basis": f"{DD_LANE_OPS_PER_PAIR} FP32 lane operations per pair (packed f32x2 issue)",
             "launch_shape": tuned_dd or cn.cn_tune_get("dd", n, n),
             "steps": args.dd_steps,
@@ -394,7 +405,7 @@ def run_ours(args):
         line["cpu_baseline"] = cpu_baseline(p, eps2, {"f32": acc.cpu().numpy(), "dd": acc_dd.cpu().numpy()},
                                             args.cpu_budget)
     if not args.no_rows:
-        line["rows"] = measure_rows(args, cn, torch, device, peak)
+        line["rows"] = measure_rows(args, cn, torch, device, pair_peak)
     return line
 
 
@@ -494,17 +505,13 @@ def c_call_timing(p, eps2, potential, calls=2000):
             "calls": calls, "note": "C program, back-to-back cn_force on device buffers, one stream"}
 
 
-# FP32 lane operations per pair of the packed (f32x2) adjoint and
-# force-jerk-potential kernels: the FP32 pipe is their bound, as for the
-# plain kernel. The compensated kernel (packed f32x2 issue) does 82 FP32
+# FP32 lane operations per ordered pair of the adjoint and force-jerk-potential
+# kernels, which evaluate each unordered pair once (31 and 34, equal masses): the
+# FP32 pipe is their bound, as for the plain kernel. The compensated kernel (packed f32x2 issue) does 82 FP32
 # lane operations per pair (plus 6 FMNMX on the ALU pipe and 1 MUFU).
-ADJOINT_LANE_OPS_PER_PAIR = 30
+ADJOINT_LANE_OPS_PER_PAIR = 31 / 2
 DD_LANE_OPS_PER_PAIR = 82
-JERK_POT_LANE_OPS_PER_PAIR = 29  # 27 + 1 (d^2 then + eps2) + 1 (potential sum)
-# symmetric form (packed f32x2 issue): 16 FP32 lane operations per unordered
-# pair, plus per j record and lane 3 FADD joining the two packed halves and
-# 24/8 FADD of the warp reduce-scatter, over K = 8 pairs
-SYM_LANE_OPS_PER_UNORDERED_PAIR = 16 + (3 + 24 / 8) / 8
+JERK_POT_LANE_OPS_PER_PAIR = 34 / 2
 
 
 def _events_ms(torch, fn, reps, stream):
@@ -538,6 +545,7 @@ def measure_rows(args, cn, torch, device, peak):
     rows = {}
     sms = torch.cuda.get_device_properties(device).multi_processor_count
     lane_rate = sms * FP32_LANES_PER_SM * SM_MAX_MHZ * 1e6
+    sym_peak = {k: 2.0 * lane_rate / v for k, v in SYM_LANE_OPS_PER_UNORDERED_PAIR.items()}
 
     # C1: N = 1024, acceleration + potential, one evaluation (latency-bound size)
     p = synth.plummer(1024, 1001)
@@ -574,7 +582,8 @@ def measure_rows(args, cn, torch, device, peak):
         rows[f"c2_plummer{n}"] = {
             "pairs_per_s": float(n) * n / (us_dev / 1e6), "us_per_eval_device": us_dev,
             "us_per_call_direct": 1e3 * ms, "c_calls": c_call_timing(p, eps2, False) if n <= 4096 else None,
-            "frac": float(n) * n / (us_dev / 1e6) / peak, "launch_shape": cn.cn_tune_get("f32", n, n),
+            "frac": float(n) * n / (us_dev / 1e6) / (sym_peak["equal"] if n > 4096 else peak),
+            "launch_shape": cn.cn_tune_get("symmetric" if n > 4096 else "f32", n, n),
             "gflops_at_38": float(n) * n / (us_dev / 1e6) * FLOP_PER_PAIR / 1e9,
             "paper_gflops_8800gtx": paper_gflops[n],
             "emax": oracle.e_max(acc.cpu().numpy()[r], ref),
@@ -600,7 +609,7 @@ def measure_rows(args, cn, torch, device, peak):
     edd = oracle.rel_errors(add.cpu().numpy()[r], ref)
     pairs = float(n) * n
     rows["c3_hernquist_2p20"] = {
-        "f32": {"pairs_per_s": pairs / (ms32 / 1e3), "frac": pairs / (ms32 / 1e3) / peak,
+        "f32": {"pairs_per_s": pairs / (ms32 / 1e3), "frac": pairs / (ms32 / 1e3) / sym_peak["unequal"],
                 "emax": float(e32.max()), "p99": float(np.percentile(e32, 99)), "median": float(np.median(e32))},
         "compensated": {"pairs_per_s": pairs / (msdd / 1e3),
                         "frac_of_own_roofline": pairs / (msdd / 1e3) / (lane_rate / DD_LANE_OPS_PER_PAIR),
@@ -613,7 +622,7 @@ def measure_rows(args, cn, torch, device, peak):
     # C4: 512 clusters in one persistent launch (graph-captured) vs per-cluster launches
     rec, offs, eps2s = synth.ensemble(512, 512)
     t = torch.from_numpy(rec).to(device)
-    tuned = cn.cn_autotune_batched(offs, eps2s, t, reps=2)
+    cn.cn_autotune_batched(offs, eps2s, t, reps=2)  # keeps a shape only where it beats the default
     plan = cn.BatchPlan(offs, eps2s)
     side = torch.cuda.Stream(device)
     acc_b = torch.empty((rec.shape[0], 3), dtype=torch.float32, device=device)
@@ -653,11 +662,10 @@ def measure_rows(args, cn, torch, device, peak):
     rows["c4_ensemble512"] = {
         "useful_pairs": useful,
         "persistent_graph": {"pairs_per_s": useful / (ms_graph / 1e3), "ms": ms_graph,
-                             "frac": useful / (ms_graph / 1e3) / peak},
+                             "frac": useful / (ms_graph / 1e3) / sym_peak["equal"]},
         "persistent_direct": {"pairs_per_s": useful / (ms_direct / 1e3), "ms": ms_direct},
         "separate_launches": {"pairs_per_s": useful / (ms_sep / 1e3), "ms": ms_sep},
         "graph_of_separate_launches": {"pairs_per_s": useful / (ms_sep_graph / 1e3), "ms": ms_sep_graph},
-        "launch_shape": tuned,
         "emax": max(errs),
         "cpu_baseline": {"value": n_rows / t_or, "unit": UNIT, "cores": oracle.max_threads(), "kind": "oracle",
                          "sample": "64 seeded rows of every 4th cluster"}}
@@ -700,7 +708,7 @@ def measure_rows(args, cn, torch, device, peak):
     t0 = time.perf_counter()
     ra, _ = oracle.force(p, p, eps2, rows=r, potential=False)
     dt = time.perf_counter() - t0
-    sym_roof = 2.0 * lane_rate / SYM_LANE_OPS_PER_UNORDERED_PAIR
+    sym_roof = sym_peak["equal"]
     rows["symmetric131072"] = {
         "pairs_per_s": float(n) * n / (ms / 1e3), "ms": ms,
         "with_potential": {"pairs_per_s": float(n) * n / (ms_pot / 1e3), "ms": ms_pot},

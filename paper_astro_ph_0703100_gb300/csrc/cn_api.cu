@@ -365,8 +365,9 @@ int64_t round_up(int64_t x, int64_t m) { return (x + m - 1) / m * m; }
 // (8 x 256 2.2e12 unordered pairs/s in the inner loop, 4 x 128 2.0e12, both
 // at 16 warps per SM); smaller ones cut the work finer over the CTAs and
 // waste less on the diagonal tiles, which are evaluated one-sided. Measured
-// (us, equal masses, 152 SMs; the lines lie where the order changes, and
-// another SM count moves them by the work per SM):
+// (us, equal masses, 152 SMs, sums folded every 512 records, 8 steps per
+// trip: now 1 to 2% less at the large end; the lines lie where the order
+// changes, and another SM count moves them by the work per SM):
 //   n       2x128/128  4x128/256  8x128/128  8x256/128
 //   5000      16.7       16.8       19.3+      19.3+
 //   7000      25.3       23.6       25.0       25.2
@@ -974,7 +975,8 @@ cn_status sym_launch(const std::string& what, const DeviceInfo& d, cn::SymForm f
 // of the smallest systems, which merge nothing. Measured (us, one-sided /
 // symmetric): force 4096 11.1 / 14.1, 5000 20.5 / 16.7, 16384 108 / 78;
 // force + jerk + potential 2048 10.4 / 12.1, 3000 31.2 / 16.8, 16384 271 /
-// 178; adjoint 2048 12.3 / 14.4, 3000 34.9 / 18.5, 16384 284 / 174.
+// 178; adjoint (folded every 64 records, now 32) 2048 12.3 / 14.4, 3000 34.9 /
+// 18.5, 16384 284 / 174.
 bool sym_pays(cn::SymForm form, int64_t n, int sms) {
   const int64_t from = form == cn::kSymForce || form == cn::kSymForcePot ? 4096 : 2048;
   return n > from && static_cast<double>(n) * std::sqrt(152.0 / std::max(sms, 1)) > static_cast<double>(from);
@@ -984,7 +986,8 @@ bool sym_pays(cn::SymForm form, int64_t n, int sms) {
 // eight particles per thread (248 registers, one CTA of 256 per SM) share
 // the 14 shuffles of a step among twice the pairs: with the potential 65536
 // 2571 us against 2739 for four, 32768 659 / 687, 16384 184 / 178. Eight for
-// the adjoint: 65536 2392 / 2431, 50000 1484 / 1435, so it stays at four.
+// the adjoint (folded every 64 records, now 32: 65536 2485): 65536 2392 /
+// 2431, 50000 1484 / 1435, so it stays at four.
 // Below, two or four particles in smaller tiles: jerk 4096 21.9 us (2 x 256)
 // / 22.4 (4 x 128), 6000 37.7 / 36.3; adjoint 6000 36.9 (2 x 128) / 39.0 (4 x
 // 128), 10000 81.9 / 77.8, 24576 373 (4 x 128) / 371 (4 x 256).
