@@ -433,6 +433,36 @@ int32_t fit_j_tile(int64_t n_i, int64_t n_j, int64_t i_tile, int32_t lo, int32_t
   return best_t;
 }
 
+// The j-tile of a small compensated call in tiles of 64 i-particles (one per
+// thread). Such a call is a chain of latencies, not work: a pair term takes
+// about 0.06 us of one warp, and one warp per scheduler (two CTAs of 64
+// threads per SM) runs at full speed, further units queue behind it; the CTA
+// that arrives last adds its tile's parts one after the other, each as long
+// as 13 records, and a unit's start costs about 24. Of the multiples of 32 this picks the
+// j-tile with the least of the sum; in a sweep of 13 j-tiles it was the
+// fastest one at every size tried up to 2600 (us, 2 x 64 threads with 128
+// records before / now: 256 22.3 / 11.5, 1100 31.8 / 19.6, 2048 41.6 / 27.6, 2600
+// 61.6 / 35.3, 100 x 4000 59.7 / 31.2). From 1.4e7 pairs on the units of a
+// round no longer wait for one another and tiles up to 256 are the better ones
+// (4095: 224 records 72 us, 512 91, 480 102).
+int32_t dd_small_j_tile(int64_t n_i, int64_t n_j, int sms) {
+  const int64_t rows = (n_i + 63) / 64;
+  const int64_t most = static_cast<double>(n_i) * static_cast<double>(n_j) <= 1.4e7 ? 768 : 256;
+  const int64_t hi = std::min<int64_t>(most, (std::max<int64_t>(n_j, 1) + 31) / 32 * 32);
+  int32_t best_t = 32;
+  int64_t best = -1;
+  for (int64_t t = 32; t <= hi; t += 32) {
+    const int64_t parts = (std::max<int64_t>(n_j, 1) + t - 1) / t;
+    const int64_t rounds = (rows * parts + 2 * sms - 1) / (2 * sms);
+    const int64_t c = rounds * (t + 24) + 13 * parts;
+    if (best < 0 || c < best) {
+      best = c;
+      best_t = static_cast<int32_t>(t);
+    }
+  }
+  return best_t;
+}
+
 // Default launch shape of a variant for these sizes on a device with `sms`
 // multiprocessors (queried, never assumed).
 cn_tune default_tune(int variant, int64_t n_i, int64_t n_j, int sms) {
@@ -549,10 +579,19 @@ cn_tune default_tune(int variant, int64_t n_i, int64_t n_j, int sms) {
     t.i_per_thread = 4;
     t.threads = 256;
     t.j_tile = fit_j_tile(n_i, n_j, 1024, 256, 1024, 16, sms, 9);
-  } else if (dd && n >= 4096 && n < 12000) {
-    // compensated form, small systems: one i-particle per thread keeps the
-    // i-tiles small enough to fill the SMs (N = 8192: 0.595 of its bound
-    // against 0.548 for K = 2 x 128; 4096: 0.418 against 0.397)
+  } else if (dd && n < 10500) {
+    // compensated form, small systems: one i-particle per thread in CTAs of 64
+    // threads fills the SMs and its CTAs are many enough to even out the last
+    // round. Up to 1.85e7 pairs the j-tile is fitted (dd_small_j_tile); above,
+    // 96 records are within 8% of the best of 13 at every size tried (us, 1 x
+    // 128 threads with 256 records / this: 4500 114.5 / 84.4, 5400 133.1 /
+    // 103.7, 7200 181.5 / 165.1, 9000 281.6 / 249.6, 10000 335 / 312, but
+    // 12000 416 / 438)
+    t.i_per_thread = 1;
+    t.threads = 64;
+    t.j_tile = static_cast<double>(n_i) * static_cast<double>(n_j) <= 1.85e7 ? dd_small_j_tile(n_i, n_j, sms) : 96;
+  } else if (dd && n < 12000) {
+    // K = 1 x 128, the j-tile of 256 records (11000: 373 us)
     t.i_per_thread = 1;
     t.j_tile = 256;
   } else if (n >= 32768) {
