@@ -582,14 +582,24 @@ cn_tune default_tune(int variant, int64_t n_i, int64_t n_j, int sms) {
   } else if (dd && n < 10500) {
     // compensated form, small systems: one i-particle per thread in CTAs of 64
     // threads fills the SMs and its CTAs are many enough to even out the last
-    // round. Up to 1.85e7 pairs the j-tile is fitted (dd_small_j_tile); above,
+    // round. Up to 1.894e7 pairs the j-tile is fitted (dd_small_j_tile); above,
     // 96 records are within 8% of the best of 13 at every size tried (us, 1 x
     // 128 threads with 256 records / this: 4500 114.5 / 84.4, 5400 133.1 /
     // 103.7, 7200 181.5 / 165.1, 9000 281.6 / 249.6, 10000 335 / 312, but
     // 12000 416 / 438)
+    // Where the units of 128 x 256 fill 94% of whole rounds of four CTAs per
+    // SM, those stay ahead by 2 to 3% (6144 131.5 / 135.7, 8704 238 / 244)
     t.i_per_thread = 1;
     t.threads = 64;
-    t.j_tile = static_cast<double>(n_i) * static_cast<double>(n_j) <= 1.85e7 ? dd_small_j_tile(n_i, n_j, sms) : 96;
+    const int64_t units = (n_i + 127) / 128 * ((n_j + 255) / 256), round = 4 * static_cast<int64_t>(sms);
+    if (static_cast<double>(n_i) * static_cast<double>(n_j) <= 1.894e7) {
+      t.j_tile = dd_small_j_tile(n_i, n_j, sms);
+    } else if (static_cast<double>(units) >= 0.94 * static_cast<double>((units + round - 1) / round * round)) {
+      t.threads = 128;
+      t.j_tile = 256;
+    } else {
+      t.j_tile = 96;
+    }
   } else if (dd && n < 12000) {
     // K = 1 x 128, the j-tile of 256 records (11000: 373 us)
     t.i_per_thread = 1;
