@@ -983,6 +983,9 @@ cn_status sym_launch(const std::string& what, const DeviceInfo& d, cn::SymForm f
   a.chunk = sp.chunk;
   a.stages = sp.stages;
   a.eps2 = eps2;
+  // a mass-free term of these forms is at most 4 eps^-3 |w| with |w| <= 2 sqrt(3) of the largest component, and
+  // at most 256 of them are added before they are scaled
+  a.fast = static_cast<float>(std::min(3e38, 5e34 * std::pow(static_cast<double>(eps2), 1.5)));
   a.wait_ns = g_wait_ns.load();
   cn::SymMerge m{};
   m.slots_seg = a.slots_seg;

@@ -15,7 +15,7 @@
 // share a warp), cuts the work at any block instead of at whole j-tiles, and
 // merges split rows with as many threads as they have sums (there the last
 // CTA of a tile adds all its partials alone). With per-particle softening the
-// s = 0 guard is taken only by warps that hold one below kRowSoft. Measured
+// s = 0 guard is taken only by warps that hold one outside kRowSoft .. kRowStiff. Measured
 // (us, pair kernel / this one with equal / unequal masses): 1024 x 65536 47.0
 // / 33.6 / 35.3, 4000 x 16384 39.6 / 31.8 / 33.6, 2048 x 262144 241 / 193 /
 // 211; per-particle softening 16384 x 16384 135.8 / 104.6 / 113.4. Unequal
@@ -42,6 +42,8 @@ constexpr int kRowWarps = 8;
 constexpr int kRowThreads = 32 * kRowWarps;
 constexpr float kRowFar = 1e11f;     // |coordinate| up to which r^-3 stays a normal number
 constexpr float kRowSoft = 1e-20f;   // eps2 from which it stays finite
+constexpr float kRowStiff = 1e24f;   // eps2 up to which it stays a normal number
+constexpr float kRowHeavySoft = 1e12f;  // eps2 up to which the sums r^-3 d of masses above 1 are well above underflow
 
 enum RowMode : int {
   kRowUniform = 0,  // equal masses, factored out
@@ -204,7 +206,7 @@ __global__ void __launch_bounds__(kRowThreads, 2) rows_kernel(const __grid_const
   const float2 e2 = row_dup(a.eps2);
   float scale = 1.f;  // of the sums in registers
   int held = 0;       // j records in them, about
-  bool near_i = false;
+  bool near_i = false, heavy_i = false;  // positions and softenings in range; for masses above 1 too
   float* const mine = sums + warp * kPer + lane;  // the thread's sums: mine[c * kAll + 32 k]
 
   auto fold = [&]() {
@@ -266,7 +268,7 @@ __global__ void __launch_bounds__(kRowThreads, 2) rows_kernel(const __grid_const
       if (row >= 0) flush();
       row = ch.row;
       const int64_t i0 = static_cast<int64_t>(row) * a.tile;
-      bool near = EPSI || a.eps2 >= kRowSoft;
+      bool near = EPSI || (a.eps2 >= kRowSoft && a.eps2 <= kRowStiff), heavy = EPSI || a.eps2 <= kRowHeavySoft;
 #pragma unroll
       for (int k = 0; k < K; ++k) {
         const int64_t p = i0 + wi * kPer + 32 * k + lane;
@@ -277,11 +279,13 @@ __global__ void __launch_bounds__(kRowThreads, 2) rows_kernel(const __grid_const
         row_half(acc.nx[k >> 1][2], k) = -v.z;
         if constexpr (EPSI) {
           row_half(acc.ei[k >> 1], k) = v.w;
-          near = near && v.w >= kRowSoft;
+          near = near && v.w >= kRowSoft && v.w <= kRowStiff;
+          heavy = heavy && v.w <= kRowHeavySoft;
         }
         near = near && fmaxf(fabsf(v.x), fmaxf(fabsf(v.y), fabsf(v.z))) <= kRowFar;
       }
       near_i = __all_sync(0xffffffffu, near);
+      heavy_i = __all_sync(0xffffffffu, heavy);
 #pragma unroll
       for (int p = 0; p < P; ++p)
 #pragma unroll
@@ -314,7 +318,7 @@ __global__ void __launch_bounds__(kRowThreads, 2) rows_kernel(const __grid_const
         near = near && fmaxf(fabsf(v.x), fmaxf(fabsf(v.y), fabsf(v.z))) <= kRowFar;
       }
       near = __all_sync(0xffffffffu, near);
-      same = __all_sync(0xffffffffu, same && near && fabsf(mj) <= 3.4e38f);
+      same = __all_sync(0xffffffffu, same && near && fabsf(mj) <= (heavy_i ? 3.4e38f : 1.f));
       const float factor = same ? mj : 1.f;
       if (held > 0 && (factor != scale || held + count > kRowFold)) fold();
       scale = factor;

@@ -29,9 +29,13 @@
 // (14 instead of 16 lane operations per unordered pair: 2.20e12 pairs/s).
 // That is decided per chunk and warp from the records themselves (the
 // warp's own masses equal too). It needs r^-3 within the FP32 range, as
-// does the general term's r^-3 m: beyond coordinates of 1e11 or below a
-// softening of 1e-10 the term is formed as (m r)(r r), the order of the
-// one-sided kernel.
+// does the general term's r^-3 m: beyond coordinates of 1e11 and outside
+// softenings of 1e-10 .. 1e12 the term is formed as (m r)(r r), the order of the
+// one-sided kernel. The unscaled sums r^-3 d must stay in that range too. They
+// cannot overflow there (at most eps^-2 a term); a mass above 1 that would have
+// kept a product from underflowing stays in its term unless the softening is
+// below 1e6 (kHeavySoft). Sums r^-3 w of a velocity or weight underflow and
+// overflow with w: see kHeavyReach and SymArgs::fast.
 //
 // Shared memory per CTA: a ring of staged chunks (bulk copies), three buffers
 // of the j-side sums of a chunk, one row per warp, and the i-side (hi, lo)
@@ -57,6 +61,8 @@ namespace cn {
 
 constexpr float kSymFar = 1e11f;       // |coordinate| up to which r^-3 stays a normal number
 constexpr float kSymSoft = 1e-20f;     // eps2 from which it stays finite
+constexpr float kSymStiff = 1e24f;     // eps2 up to which it stays a normal number
+constexpr float kSymHuge = 3.4e38f;    // finite
 
 enum SymMode : int {
   kSymUniform = 0,  // equal masses, factored out of the pair terms
@@ -64,6 +70,9 @@ enum SymMode : int {
   kSymWide = 2,     // (m r)(r r): any range
 };
 
+__device__ __forceinline__ float sym_reach(const float4& v) {
+  return fmaxf(fabsf(v.x), fmaxf(fabsf(v.y), fabsf(v.z)));
+}
 __device__ __forceinline__ float2 sym_dup(float v) { return make_float2(v, v); }
 __device__ __forceinline__ float& sym_half(float2& v, int k) { return (k & 1) ? v.y : v.x; }
 
@@ -79,6 +88,9 @@ __device__ __forceinline__ float& sym_half(float2& v, int k) { return (k & 1) ? 
 //   kWide           offers the kSymWide terms
 //   kSameMass       equal masses factor out only if the warp's and the
 //                   chunk's are the same
+//   kHeavyReach     |coordinate| (with a second record) and eps2 up to which
+//   kHeavySoft      masses above 1 factor out: unscaled sums there are well
+//                   above underflow
 //   kOwnSign        sign of the warp's own masses handed to `pair`
 //   weight          factor of i-side sum c when it is folded (mass: the
 //                   chunk's mass where the masses are factored out, else 1)
@@ -103,17 +115,20 @@ struct SymForcePolicy {
   static constexpr int kMinBlocks = 2;
   static constexpr bool kWide = true;
   static constexpr bool kSameMass = false;
+  // r^-3 d is at least 1e-23 where d is the longer one, r^-3 at least 1e-18 where eps is
+  static constexpr float kHeavySoft = 1e12f;
   static constexpr float kOwnSign = -1.f;
   float2 nx[P][3], acc[P][kSumsI];
 
-  __device__ __forceinline__ void load(const SymArgs& a, int64_t p, bool valid, int k, float& mass, float& reach) {
+  __device__ __forceinline__ void load(const SymArgs& a, int64_t p, bool valid, int k, float& mass, float& reach,
+                                       float& /*speed*/) {
     float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
     if (valid) v = __ldg(a.pos + p);
     sym_half(nx[k >> 1][0], k) = -v.x;
     sym_half(nx[k >> 1][1], k) = -v.y;
     sym_half(nx[k >> 1][2], k) = -v.z;
     mass = v.w;
-    reach = fmaxf(fabsf(v.x), fmaxf(fabsf(v.y), fabsf(v.z)));
+    reach = sym_reach(v);
   }
 
   template <int MODE, bool BOTH>
@@ -369,7 +384,12 @@ __global__ void __launch_bounds__(256, Pol::kMinBlocks) sym_kernel(const __grid_
   int32_t cur_I = -1;
   float scale = 1.f;   // of the sums in registers
   int held = 0;        // j blocks in them
-  bool own_uniform = false, own_near = false;  // the warp's masses are equal; its positions are in range
+
+  // the warp's own particles: equal masses that may factor out; r^-3 in range; (with a second
+  // record) within kHeavyReach and kHeavySoft; second records within a.fast
+  bool own_uniform = false, own_near = false, own_close = false, own_slow = false;
+  // the largest mass that may factor out, by the softening alone
+  auto heaviest = [&]() { return e2.x <= Pol::kHeavySoft ? kSymHuge : 1.f; };
 
   // adds the register sums to the row's (hi, lo) sums (each thread its own
   // particles') and clears them
@@ -454,7 +474,7 @@ __global__ void __launch_bounds__(256, Pol::kMinBlocks) sym_kernel(const __grid_
     if (ch.row != cur_I) {
       if (cur_I >= 0) flush(cur_I);
       cur_I = ch.row;
-      bool same = true, near = true;
+      bool same = true, near = true, close = true, slow = true;
       float m0 = 0.f;
       int64_t p0 = static_cast<int64_t>(cur_I) * B, pn = a.g.n;
       if constexpr (BATCHED) {
@@ -466,15 +486,23 @@ __global__ void __launch_bounds__(256, Pol::kMinBlocks) sym_kernel(const __grid_
 #pragma unroll
       for (int k = 0; k < K; ++k) {
         const int64_t p = p0 + k * NT + tid;
-        float m, reach;
-        acc.load(a, p, p < pn, k, m, reach);
+        float m, reach, speed = 0.f;
+        acc.load(a, p, p < pn, k, m, reach, speed);
         mass[k * NT + tid] = m;
         if (k == 0) m0 = __shfl_sync(0xffffffffu, m, 0);
         same = same && m == m0;
         near = near && reach <= kSymFar;
+        if constexpr (JR == 2) {
+          close = close && reach <= Pol::kHeavyReach;
+          slow = slow && speed <= a.fast;
+        }
       }
-      own_uniform = __all_sync(0xffffffffu, same && fabsf(m0) <= 3.4e38f);
-      own_near = __all_sync(0xffffffffu, near && e2.x >= kSymSoft);
+      own_uniform = __all_sync(0xffffffffu, same && fabsf(m0) <= (JR == 2 ? kSymHuge : heaviest()));
+      own_near = __all_sync(0xffffffffu, near && e2.x >= kSymSoft && e2.x <= kSymStiff);
+      if constexpr (JR == 2) {
+        own_close = __all_sync(0xffffffffu, close && e2.x <= Pol::kHeavySoft);
+        own_slow = __all_sync(0xffffffffu, slow);
+      }
 #pragma unroll
       for (int p = 0; p < P; ++p)
 #pragma unroll
@@ -493,11 +521,16 @@ __global__ void __launch_bounds__(256, Pol::kMinBlocks) sym_kernel(const __grid_
     float factor = 1.f;
     if constexpr (!Pol::kGuard) {
       const float mj = js[0].w;
-      bool same = fabsf(mj) <= 3.4e38f, near = own_near;
+      // with a second record the positions count too where either mass is above 1
+      const bool heavy = JR == 2 && (fabsf(mj) > 1.f || (own_uniform && fabsf(mass[tid]) > 1.f));
+      bool same = fabsf(mj) <= (JR == 2 ? kSymHuge : heaviest()), near = own_near;
+      if constexpr (JR == 2) same = same && own_slow && (!heavy || own_close);
       for (int t = lane; t < count; t += 32) {
         const float4 v = js[t];
+        const float reach = sym_reach(v);
         same = same && v.w == mj;
-        near = near && fmaxf(fabsf(v.x), fmaxf(fabsf(v.y), fabsf(v.z))) <= kSymFar;
+        near = near && reach <= kSymFar;
+        if constexpr (JR == 2) same = same && (!heavy || reach <= Pol::kHeavyReach) && sym_reach(js[CH + t]) <= a.fast;
       }
       if (Pol::kSameMass)
         same = same && own_uniform && mass[tid] == mj;

@@ -199,6 +199,7 @@ struct SymArgs {
   int32_t chunk;       // j records per ring stage (multiple of 32)
   int32_t stages;
   float eps2;
+  float fast;          // forms with a second record: its largest component for the mass-free terms
   uint64_t wait_ns;
   const SymRow* rows;  // ensembles: the rows (g then holds only the cost line and the CTAs)
   int32_t n_rows;

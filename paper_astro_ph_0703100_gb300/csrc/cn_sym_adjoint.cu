@@ -31,11 +31,15 @@ struct SymAdjointPolicy {
   static constexpr int kMinBlocks = 2;
   static constexpr bool kWide = false;
   static constexpr bool kSameMass = true;
+  // as in the jerk form, for the weights
+  static constexpr float kHeavyReach = 1e5f;
+  static constexpr float kHeavySoft = 1e10f;
   static constexpr float kOwnSign = 1.f;
   float2 nx[P][3], nw[P][3], acc[P][kSumsI];
   float2 mi[P];
 
-  __device__ __forceinline__ void load(const SymArgs& a, int64_t p, bool valid, int k, float& mass, float& reach) {
+  __device__ __forceinline__ void load(const SymArgs& a, int64_t p, bool valid, int k, float& mass, float& reach,
+                                       float& speed) {
     float4 v = make_float4(0.f, 0.f, 0.f, 0.f), u = v;
     if (valid) {
       v = __ldg(a.pos + p);
@@ -49,7 +53,8 @@ struct SymAdjointPolicy {
     sym_half(nw[k >> 1][2], k) = -u.z;
     sym_half(mi[k >> 1], k) = v.w;
     mass = v.w;
-    reach = 0.f;  // g = r^3 is formed in either mode, as in the one-sided kernel
+    reach = sym_reach(v);
+    speed = sym_reach(u);
   }
 
   template <int MODE, bool BOTH>

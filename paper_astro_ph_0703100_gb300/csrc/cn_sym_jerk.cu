@@ -29,10 +29,14 @@ struct SymJerkPolicy {
   static constexpr int kMinBlocks = 1;
   static constexpr bool kWide = true;
   static constexpr bool kSameMass = false;
+  // r^-3 is at least 2e-17 there, and r^-3 w a normal number for |w| > 1e-21
+  static constexpr float kHeavyReach = 1e5f;
+  static constexpr float kHeavySoft = 1e10f;
   static constexpr float kOwnSign = -1.f;
   float2 nx[P][3], nv[P][3], acc[P][kSumsI];
 
-  __device__ __forceinline__ void load(const SymArgs& a, int64_t p, bool valid, int k, float& mass, float& reach) {
+  __device__ __forceinline__ void load(const SymArgs& a, int64_t p, bool valid, int k, float& mass, float& reach,
+                                       float& speed) {
     float4 v = make_float4(0.f, 0.f, 0.f, 0.f), u = v;
     if (valid) {
       v = __ldg(a.pos + p);
@@ -45,7 +49,8 @@ struct SymJerkPolicy {
     sym_half(nv[k >> 1][1], k) = -u.y;
     sym_half(nv[k >> 1][2], k) = -u.z;
     mass = v.w;
-    reach = fmaxf(fabsf(v.x), fmaxf(fabsf(v.y), fabsf(v.z)));
+    reach = sym_reach(v);
+    speed = sym_reach(u);
   }
 
   template <int MODE, bool BOTH>
