@@ -99,6 +99,12 @@ __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
   e = __fadd_rn(__fadd_rn(a, -ap), __fadd_rn(b, -bp));
 }
 
+// The sum of a (hi, lo) pair kept by two_sum. Once hi has overflowed, lo is
+// NaN (infinity minus infinity) and hi the sum.
+__device__ __forceinline__ float pair_total(float hi, float lo) {
+  return fabsf(hi) <= 3.402823466e38f ? __fadd_rn(hi, lo) : hi;
+}
+
 // Adds the FP32 value x into the double-single pair (hi, lo).
 __device__ __forceinline__ void ds_accumulate(float& hi, float& lo, float x) {
   float s, e;

@@ -247,7 +247,7 @@ __global__ void __launch_bounds__(kRowThreads, 2) rows_kernel(const __grid_const
         two_sum(s, h[w * a.tile], s, t);
         l = __fadd_rn(l, __fadd_rn(t, h[NS * kAll + w * a.tile]));
       }
-      const float v = __fadd_rn(s, l);
+      const float v = pair_total(s, l);
       if (!whole)
         seg[e] = v;
       else if (p < ni) {
@@ -378,7 +378,7 @@ __global__ void __launch_bounds__(256) rows_merge_kernel(const __grid_constant__
         l = __fadd_rn(l, t);
       }
   }
-  const float v = __fadd_rn(h, l);
+  const float v = pair_total(h, l);
   if (c < 3)
     a.acc_out[3 * (i0 + p) + c] = v;
   else

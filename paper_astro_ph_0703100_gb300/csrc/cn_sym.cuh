@@ -420,7 +420,7 @@ __global__ void __launch_bounds__(256, Pol::kMinBlocks) sym_kernel(const __grid_
 #pragma unroll
       for (int k = 0; k < K; ++k) {
         const int e = c * B + k * NT + tid;
-        seg[e] = __fadd_rn(sums[e], sums[e + NI * B]);
+        seg[e] = pair_total(sums[e], sums[e + NI * B]);
       }
   };
   // once every warp has swept chunk q: refills its stage (thread 0) and adds
@@ -710,7 +710,7 @@ __global__ void __launch_bounds__(32 * kSymMergeWarps<BATCHED>) sym_merge_kernel
       l = __fadd_rn(l, __fadd_rn(e, part[w][c][lane].y));
     }
     if (m.last)
-      Pol::output(m, p, c, __fadd_rn(h, l));
+      Pol::output(m, p, c, pair_total(h, l));
     else
       m.carry[static_cast<size_t>(c) * m.n_pad + p] = make_float2(h, l);
   }
