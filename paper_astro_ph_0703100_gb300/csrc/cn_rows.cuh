@@ -206,7 +206,7 @@ __global__ void __launch_bounds__(kRowThreads, 2) rows_kernel(const __grid_const
   const float2 e2 = row_dup(a.eps2);
   float scale = 1.f;  // of the sums in registers
   int held = 0;       // j records in them, about
-  bool near_i = false, heavy_i = false;  // positions and softenings in range; for masses above 1 too
+  float cap = -1.f;   // masses that may factor out with the warp's particles, up to (none: -1)
   float* const mine = sums + warp * kPer + lane;  // the thread's sums: mine[c * kAll + 32 k]
 
   auto fold = [&]() {
@@ -284,8 +284,8 @@ __global__ void __launch_bounds__(kRowThreads, 2) rows_kernel(const __grid_const
         }
         near = near && fmaxf(fabsf(v.x), fmaxf(fabsf(v.y), fabsf(v.z))) <= kRowFar;
       }
-      near_i = __all_sync(0xffffffffu, near);
-      heavy_i = __all_sync(0xffffffffu, heavy);
+      heavy = __all_sync(0xffffffffu, heavy);
+      cap = __all_sync(0xffffffffu, near) ? (heavy ? 3.4e38f : 1.f) : -1.f;
 #pragma unroll
       for (int p = 0; p < P; ++p)
 #pragma unroll
@@ -310,7 +310,7 @@ __global__ void __launch_bounds__(kRowThreads, 2) rows_kernel(const __grid_const
       // this warp's records of the stage: the units wj, wj + nwj, ...
       const float4* js = ring + slot * static_cast<uint32_t>(CH);
       const int count = ((units - wj + nwj - 1) / nwj) * kRowUnit;
-      bool same = true, near = near_i;
+      bool same = true, near = cap >= 0.f;
       const float mj = js[wj * kRowUnit].w;
       for (int t = lane; t < count; t += 32) {
         const float4 v = js[(wj + t / kRowUnit * nwj) * kRowUnit + t % kRowUnit];
@@ -318,7 +318,7 @@ __global__ void __launch_bounds__(kRowThreads, 2) rows_kernel(const __grid_const
         near = near && fmaxf(fabsf(v.x), fmaxf(fabsf(v.y), fabsf(v.z))) <= kRowFar;
       }
       near = __all_sync(0xffffffffu, near);
-      same = __all_sync(0xffffffffu, same && near && fabsf(mj) <= (heavy_i ? 3.4e38f : 1.f));
+      same = __all_sync(0xffffffffu, same && near && fabsf(mj) <= cap);
       const float factor = same ? mj : 1.f;
       if (held > 0 && (factor != scale || held + count > kRowFold)) fold();
       scale = factor;
