@@ -1076,13 +1076,14 @@ struct RowPlan {
 // Shape of the row kernel. Small tiles (four particles per thread, all warps
 // on the same 128) waste the least on small sets: 4000 x 16384 31.6 us against
 // 32.6 for 8 x 32 and 56 for eight warps along i. Large plain sets take eight
-// per thread (2048 x 262144 209 against 213 us); with the potential or
+// per thread (2048 x 262144 209 against 213 us) where they fill those tiles as
+// well (1145 x 146556 86.2 us in the pair kernel, 87.2 with eight, 75.8 with four); with the potential or
 // per-particle softening the registers of four suit better, and the latter's
 // large sets take the warps along i (32768 x 32768 with the potential 461 us,
 // 466 with all warps on the same, 482 with eight per thread).
 cn_status rows_fit(int dev, const DeviceInfo& d, cn::RowForm form, int64_t n_i, int64_t n_j, RowPlan* rp) {
   const double pairs = static_cast<double>(n_i) * static_cast<double>(n_j);
-  rp->k = form == cn::kRowForce && pairs >= 1.5e8 ? 8 : 4;
+  rp->k = form == cn::kRowForce && pairs >= 1.5e8 && 20 * round_up(n_i, 256) <= 21 * round_up(n_i, 128) ? 8 : 4;
   rp->wi = form != cn::kRowForce && pairs >= 5e8 && n_i >= 16384 ? 8 : 1;
   rp->stages = 3;
   rp->chunk = rp->wi == 8 ? 256 : 1024;
@@ -1144,23 +1145,40 @@ cn_status rows_launch(const std::string& what, const DeviceInfo& d, cn::RowForm 
 }
 
 // Whether the row kernel is the faster one for any masses, on a device with
-// `sms` multiprocessors (pairs and particles counted per SM). Below 2.4e7 pairs
-// the pair kernel's small shapes are (4500 x 4500 15.6 us against 17.6, 8192 x
-// 2500 15.7 / 17.8), and fewer than 128 i-particles leave lanes idle (40 x
-// 600000 38.2 / 60.8). Above, with per-particle softening always (5000 x 5000
-// 22.5 / 19.3 us, 65536 x 65536 1713 / 1634). Plain sets and those with the
-// potential: the middle is the row kernel's (300 x 70000 31.7 / 27.4, 4000 x
-// 16384 39.8 / 33.6, 2048 x 262144 241 / 211, 8192 x 8192 36.3 / 34.9, 7000 x
-// 20000 66.6 / 63.3), and large sets keep the pair kernel (8192 x 100003 309 /
-// 320, 10007 x 100003 376 / 388, 16384 x 16384 108.1 / 109.5): unequal masses
-// throughout.
-bool rows_pays(cn::RowForm form, int64_t n_i, int64_t n_j, int sms) {
+// `sms` multiprocessors (pairs and particles counted per SM); p and g: the
+// pair kernel's shape and schedule of the call. Below 2.4e7 pairs the pair
+// kernel's small shapes are (4500 x 4500 15.6 us against 17.6, 8192 x 2500 15.7
+// / 17.8), and fewer than 128 i-particles leave lanes idle (40 x 600000 38.2 /
+// 60.8). Above, by 253 random shapes and 150 on a grid, unequal masses:
+// - i-particles that fill their tiles badly (more than 1.28 times their number
+//   in whole tiles, none from 401 on) keep the pair kernel: 135 x 180000 33.0 /
+//   46.9, 145 x 450445 48.8 / 62.9, but 202 x 239087 48.8 / 42.5.
+// - Up to 4096 of them the pair kernel's small shapes have large j-tiles: 300 x
+//   70000 31.7 / 27.4, 4000 x 16384 39.8 / 33.6, 2048 x 262144 241 / 211.
+// - More of them run at most 6% slower with the row kernel where the pair
+//   kernel's schedule wastes nothing (5990 x 6938 24.1 / 25.5, 6136 x 7916 26.4 /
+//   27.9) and up to 8% faster where it wastes a tenth: from 5% on it is taken
+//   (6750 x 3592 20.2 / 18.8, 7009 x 11997 45.0 / 41.8).
+// - Plain sets and those with the potential: large ones keep the pair kernel
+//   (8192 x 100003 309 / 320, 10007 x 100003 376 / 388, 16384 x 16384 108.1 /
+//   109.5).
+// - Per-particle softening, whose pair kernel holds two particles per lane
+//   group and a guard in every pair: always from 4.2e7 pairs (65536 x 65536 1713
+//   / 1634, 2065368 x 22 756 / 369); below, more than 4096 i-particles as above,
+//   and not on fewer than 1000 j records, which leave most of a row's warps idle
+//   (95845 x 275 22.4 / 28.3, 17999 x 1343 15.9 / 20.7).
+bool rows_pays(cn::RowForm form, int64_t n_i, int64_t n_j, int sms, const Plan& p, const Geometry& g) {
   const double share = 152.0 / std::max(sms, 1);
-  const double pairs = static_cast<double>(n_i) * static_cast<double>(n_j) * share;
-  if (n_i < 128 || pairs < 2.4e7) return false;
-  if (form == cn::kRowEpsI || form == cn::kRowEpsIPot) return true;
+  const double real = static_cast<double>(n_i) * static_cast<double>(n_j), pairs = real * share;
+  if (n_i < 128 || pairs < 2.4e7 || static_cast<double>(round_up(n_i, 128)) > 1.28 * static_cast<double>(n_i)) return false;
+  const bool eps_i = form == cn::kRowEpsI || form == cn::kRowEpsIPot;
   const double rows = static_cast<double>(n_i) * share;
-  return (rows <= 4096.0 && pairs <= 5.5e8) || (rows <= 8192.0 && pairs <= 1.5e8);
+  if (eps_i ? pairs >= 4.2e7 : rows <= 4096.0 && pairs <= 5.5e8) return true;
+  if (eps_i ? n_j < 1000 : rows > 8192.0 || pairs > 1.5e8) return false;
+  if (rows <= 4096.0) return true;
+  // the useful part of what the pair kernel's busiest CTA would do, were they all that busy
+  const double busiest = static_cast<double>(ceil_div(g.units, g.n_chunks)) * static_cast<double>(g.n_chunks);
+  return real < 0.95 * busiest * static_cast<double>(p.i_tile()) * static_cast<double>(p.j_tile);
 }
 
 // ------------------------------------------------------------------ single-system force
@@ -1204,7 +1222,6 @@ cn_status force_common(bool dd, int64_t n_i, const float* pos_i, int64_t n_j, co
   const bool self = !dd && !eps_i && !guard && pos_i == pos_mass_j && n_i == n_j && sym_pays(cn::kSymForce, n_i, d->sms);
   const cn::RowForm row_form =
       eps_i ? (pot ? cn::kRowEpsIPot : cn::kRowEpsI) : (pot ? cn::kRowForcePot : cn::kRowForce);
-  const bool apart = !dd && (eps_i || !guard) && !self && rows_pays(row_form, n_i, n_j, d->sms);
   struct Cached {
     PlanCache key;
     bool sym = false;
@@ -1240,7 +1257,8 @@ cn_status force_common(bool dd, int64_t n_i, const float* pos_i, int64_t n_j, co
       now.sym = true;
       now.sp.data = static_cast<char*>(ws);
     }
-    bool wanted_rows = apart && !registered_tune(dev, variant, n_i, n_j);
+    bool wanted_rows = !dd && (eps_i || !guard) && !self && rows_pays(row_form, n_i, n_j, d->sms, now.p, now.g) &&
+                       !registered_tune(dev, variant, n_i, n_j);
     if (wanted_rows) wanted_rows = rows_fit(dev, *d, row_form, n_i, n_j, &now.rp) == CN_OK;
     if (wanted_rows && lib_ws) {
       now.rows = sym_workspace(s, now.rp.need, &now.data) == CN_OK;
@@ -2249,8 +2267,12 @@ size_t cn_workspace_bytes(int variant, int64_t n_i, int64_t n_j) {
     if (n_i == n_j && sym_pays(form, n_i, d->sms) &&
         sym_fit(dev, *d, form, n_i, false, sym_default_plan(form, n_i, d->sms), &sp) == CN_OK)
       need = std::max(need, sp.need);
+    Plan p;
+    Geometry g;
     RowPlan rp;
-    if (rows_pays(rows, n_i, n_j, d->sms) && rows_fit(dev, *d, rows, n_i, n_j, &rp) == CN_OK)
+    if (resolve_plan(dev, variant, n_i, n_j, false, nullptr, &p) == CN_OK &&
+        single_geometry(dev, *d, variant, false, p, n_i, n_j, &g) == CN_OK &&
+        rows_pays(rows, n_i, n_j, d->sms, p, g) && rows_fit(dev, *d, rows, n_i, n_j, &rp) == CN_OK)
       need = std::max(need, rp.need);
     return need;
   });
