@@ -207,6 +207,15 @@ cn_status current_device(int* dev_out, DeviceInfo** info) {
   return CN_OK;
 }
 
+// Launches that hand data from one to the next through a workspace of their
+// stream are issued under this lock: calls of several threads on one stream
+// follow one another there, and do not mix their launches (as calls of one
+// launch cannot). Streams share the locks by hash.
+std::recursive_mutex& launch_order(cudaStream_t s) {
+  static std::recursive_mutex locks[64];
+  return locks[(reinterpret_cast<uintptr_t>(s) / 64) % 64];
+}
+
 // ------------------------------------------------------------------ library workspaces
 // Per (device, stream): `ctrl` holds the queue words and the split-tile
 // arrival counters (zeroed when allocated, left zero by every kernel); `data`
@@ -995,6 +1004,7 @@ cn_status sym_launch(const std::string& what, const DeviceInfo& d, cn::SymForm f
   m.n_pad = sp.n_pad;
   m.tile = static_cast<int32_t>(sp.tile);
   m.n_merge = static_cast<int32_t>(sp.n_blocks);
+  std::lock_guard<std::recursive_mutex> order(launch_order(s));
   for (int64_t r0 = 0; r0 < sp.tiles; r0 += sp.band) {
     const int64_t r1 = std::min(sp.tiles, r0 + sp.band);
     a.g.row0 = static_cast<int32_t>(r0);
@@ -1140,6 +1150,7 @@ cn_status rows_launch(const std::string& what, const DeviceInfo& d, cn::RowForm 
                  what.c_str(), rp.k, static_cast<long long>(rp.tile), static_cast<long long>(rp.rows), rp.chunk, rp.stages,
                  static_cast<long long>(rp.units), rp.grid, rp.smem, rp.need);
   if (inject("launch")) return fail(CN_ERR_CUDA, "kernel launch: injected launch failure");
+  std::lock_guard<std::recursive_mutex> order(launch_order(s));
   const cudaError_t e = cn::launch_rows(form, rp.k, a, rp.smem, s);
   return e == cudaSuccess ? CN_OK : fail_cuda(e, "row kernel launch");
 }
@@ -1495,6 +1506,7 @@ cn_status launch_ensemble(const DeviceInfo& d, const cn_batch_plan* plan, const 
                  plan->n_clusters, plan->sym_k, plan->sym_threads, plan->sym_chunk, plan->sym_stages, plan->sym_rows,
                  static_cast<long long>(a.g.cost), a.g.grid, plan->sym_smem, plan->sym_bytes);
   if (inject("launch")) return fail(CN_ERR_CUDA, "kernel launch: injected launch failure");
+  std::lock_guard<std::recursive_mutex> order(launch_order(s));
   const cudaError_t e = cn::sym_ops(form).launch(a, m, plan->sym_k, false, plan->sym_threads, plan->sym_smem, s);
   return e == cudaSuccess ? CN_OK : fail_cuda(e, "symmetric ensemble launch");
 }
@@ -2438,6 +2450,7 @@ cn_status cn_force_adjoint(int64_t n, const float* pos_mass, float eps2, const f
       if (const SymPlan* sp = sym_self_plan(dev, *d, cn::kSymAdjoint, cn::kAdjoint, n, un * 16 + 256, s)) {
         float* wrec = reinterpret_cast<float*>(sp->data + align_up(sp->need, 256));
         if (inject("launch")) return fail(CN_ERR_CUDA, "kernel launch: injected launch failure");
+        std::lock_guard<std::recursive_mutex> order(launch_order(s));
         const cudaError_t e = cn::launch_pack_w(w, reinterpret_cast<float4*>(wrec), n, s);
         if (e != cudaSuccess) return fail_cuda(e, "weight packing launch");
         float* const out[3] = {grad_pos, grad_mass, nullptr};
@@ -2453,6 +2466,7 @@ cn_status cn_force_adjoint(int64_t n, const float* pos_mass, float eps2, const f
     if ((st = library_workspace(s, g.ctrl_bytes, g.data_bytes, &ctrl, &data)) != CN_OK) return st;
     float4* wrec = reinterpret_cast<float4*>(data + g.off_wrec);
     if (inject("launch")) return fail(CN_ERR_CUDA, "kernel launch: injected launch failure");
+    std::lock_guard<std::recursive_mutex> order(launch_order(s));
     cudaError_t e = cn::launch_pack_w(w, wrec, n, s);
     if (e != cudaSuccess) return fail_cuda(e, "weight packing launch");
     PairArgs a = base_args(ctrl, data, g, p, d->status);
