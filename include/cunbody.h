@@ -463,11 +463,14 @@ CN_API cn_status cn_force_host_f64(const double *xj, const double *mj, const dou
 
 /* ------------------------------------------------------------------ tuning */
 
-/* Launch shape that calls of `variant` with these sizes will use on the
+/* Launch shape that the pair kernel of `variant` uses for these sizes on the
  * current device: an entry set by cn_tune_set / cn_autotune for the size
- * class (ceil(log2 n_i), ceil(log2 n_j)), else the built-in heuristic. */
+ * class (ceil(log2 n_i), ceil(log2 n_j)), else the built-in heuristic. Calls
+ * that take the symmetric or the row kernel instead (see cn_force) have shapes
+ * of their own. */
 CN_API cn_status cn_tune_get(int variant, int64_t n_i, int64_t n_j, cn_tune *out);
-/* Stores (tune != NULL) or clears (tune == NULL) the shape for the size class. */
+/* Stores (tune != NULL) or clears (tune == NULL) the shape for the size class.
+ * A stored shape keeps every call of the class in the pair kernel. */
 CN_API cn_status cn_tune_set(int variant, int64_t n_i, int64_t n_j, const cn_tune *tune);
 
 /*
@@ -477,7 +480,8 @@ CN_API cn_status cn_tune_set(int variant, int64_t n_i, int64_t n_j, const cn_tun
  *   {"format": "cunbody-tune-1", "device": "<name>", "arch": "sm_103",
  *    "sms": <multiprocessors>, "entries": [{"variant": "f32", "n_i_class": 17,
  *    "n_j_class": 17, "i_per_thread": 8, ...}, ...]}
- * where a size class is ceil(log2 n). Overwrites the file; CN_ERR_INVALID_ARG
+ * where a size class is ceil(log2 n), and an entry of cn_autotune also says
+ * "sets": "one" or "two" (the calls it was timed on). Overwrites the file; CN_ERR_INVALID_ARG
  * if it cannot be written.
  * cn_tune_load reads such a file and stores its entries for the current
  * device, replacing entries of the same variant and size classes. The whole
@@ -492,8 +496,14 @@ CN_API cn_status cn_tune_load(const char *path, int32_t *n_loaded);
 
 /*
  * Times every candidate launch shape for `variant` on these inputs (CUDA
- * events on `stream`, best of `reps`), stores the fastest with cn_tune_set
- * and returns it in best_out. Outputs are overwritten; synchronises
+ * events on `stream`, best of `reps`), stores the fastest for the size class
+ * and returns it in best_out. Where the call takes the symmetric or the row
+ * kernel by default, that is timed too; when it is the fastest, nothing is
+ * stored, so that calls go on taking it, and best_out is the pair kernel's
+ * default shape (storing that would keep them in the pair kernel). A shape
+ * found for one set against itself (pos_i == pos_mass_j, n_i == n_j) leaves
+ * the row kernel to calls of two sets in its class, one found for two sets
+ * leaves the symmetric kernel to calls of one. Outputs are overwritten; synchronises
  * `stream`. For the DD variants acc_out/pot_out point to double arrays,
  * for the F32 variants to float arrays. Not for CN_VARIANT_ADJOINT or the
  * batched variants (see cn_autotune_batched).
@@ -503,7 +513,9 @@ CN_API cn_status cn_autotune(int variant, int64_t n_i, const float *pos_i, int64
 
 /* Times candidate shapes for a batched ensemble (building a plan for each),
  * returns the fastest in best_out and stores it for CN_VARIANT_BATCHED /
- * CN_VARIANT_BATCHED_POT keyed by (number of clusters, total particles). */
+ * CN_VARIANT_BATCHED_POT keyed by (number of clusters, total particles). The
+ * default plan is timed too, which may take the symmetric form; when it is the
+ * fastest, nothing is stored and best_out is its one-sided shape. */
 CN_API cn_status cn_autotune_batched(int32_t n_clusters, const int64_t *offsets_host, const float *eps2_host,
                               const float *pos_mass, float *acc_out, float *pot_out, int reps, cn_stream stream,
                               cn_tune *best_out);

@@ -352,7 +352,15 @@ cn_status library_aux(cudaStream_t s, double** out) {
 }
 
 // ------------------------------------------------------------------ tuning
-std::map<std::tuple<int, int, int, int>, cn_tune> g_tune;
+// Which calls a stored shape was timed on. It keeps those, or the calls of any
+// sets (cn_tune_set), in the pair kernel where they would take another one;
+// a size class holds one set against itself and two sets alike.
+enum TunedOn : int { kTunedAny = 0, kTunedOneSet = 1, kTunedTwoSets = 2 };
+struct Tuned {
+  cn_tune t;
+  TunedOn on;
+};
+std::map<std::tuple<int, int, int, int>, Tuned> g_tune;
 
 int bucket(int64_t n) {
   int b = 0;
@@ -665,9 +673,25 @@ bool two_records(int variant) {
   return variant == cn::kAdjoint || variant == cn::kJerk || variant == cn::kJerkPot;
 }
 
-bool registered_tune(int dev, int variant, int64_t n_i, int64_t n_j) {
+// Whether a stored shape keeps calls of these sets in the pair kernel.
+bool registered_tune(int dev, int variant, int64_t n_i, int64_t n_j, TunedOn sets) {
   std::lock_guard<std::mutex> lock(g_mu);
-  return g_tune.count({dev, variant, bucket(n_i), bucket(n_j)}) > 0;
+  const auto it = g_tune.find({dev, variant, bucket(n_i), bucket(n_j)});
+  return it != g_tune.end() && (it->second.on == kTunedAny || it->second.on == sets);
+}
+
+cn_status store_tune(int variant, int64_t n_i, int64_t n_j, const cn_tune* tune, TunedOn on) {
+  int dev = 0;
+  const cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return fail_cuda(e, "cudaGetDevice");
+  std::lock_guard<std::mutex> lock(g_mu);
+  const auto key = std::make_tuple(dev, variant, bucket(n_i), bucket(n_j));
+  if (tune)
+    g_tune[key] = Tuned{*tune, on};
+  else
+    g_tune.erase(key);
+  g_plan_gen.fetch_add(1, std::memory_order_acq_rel);
+  return CN_OK;
 }
 
 cn_status resolve_plan(int dev, int variant, int64_t n_i, int64_t n_j, bool guard, const cn_tune* explicit_tune,
@@ -686,7 +710,7 @@ cn_status resolve_plan(int dev, int variant, int64_t n_i, int64_t n_j, bool guar
     std::lock_guard<std::mutex> lock(g_mu);
     auto it = g_tune.find({dev, variant, bucket(n_i), bucket(n_j)});
     if (it != g_tune.end()) {
-      chosen = it->second;
+      chosen = it->second.t;
       have = true;
     }
   }
@@ -1258,7 +1282,7 @@ cn_status force_common(bool dd, int64_t n_i, const float* pos_i, int64_t n_j, co
     // loaded with it.
     if ((st = resolve_plan(dev, variant, n_i, n_j, guard && !eps_i, nullptr, &now.p)) != CN_OK) return st;
     if ((st = single_geometry(dev, *d, variant, guard, now.p, n_i, n_j, &now.g)) != CN_OK) return st;
-    bool wanted = self && !registered_tune(dev, variant, n_i, n_j);
+    bool wanted = self && !registered_tune(dev, variant, n_i, n_j, kTunedOneSet);
     const cn::SymForm form = pot ? cn::kSymForcePot : cn::kSymForce;
     if (wanted) wanted = sym_fit(dev, *d, form, n_i, false, sym_default_plan(form, n_i, d->sms), &now.sp) == CN_OK;
     if (wanted && lib_ws) {
@@ -1269,7 +1293,7 @@ cn_status force_common(bool dd, int64_t n_i, const float* pos_i, int64_t n_j, co
       now.sp.data = static_cast<char*>(ws);
     }
     bool wanted_rows = !dd && (eps_i || !guard) && !self && rows_pays(row_form, n_i, n_j, d->sms, now.p, now.g) &&
-                       !registered_tune(dev, variant, n_i, n_j);
+                       !registered_tune(dev, variant, n_i, n_j, kTunedTwoSets);
     if (wanted_rows) wanted_rows = rows_fit(dev, *d, row_form, n_i, n_j, &now.rp) == CN_OK;
     if (wanted_rows && lib_ws) {
       now.rows = sym_workspace(s, now.rp.need, &now.data) == CN_OK;
@@ -1338,7 +1362,7 @@ const SymPlan* sym_self_plan(int dev, const DeviceInfo& d, cn::SymForm form, int
   thread_local SymPlan t_last;
   const uint64_t gen0 = g_plan_gen.load(std::memory_order_acquire);
   if (t_last.key.hit(gen0, dev, form, n, n, false, s)) return &t_last;
-  if (registered_tune(dev, variant, n, n)) return nullptr;
+  if (registered_tune(dev, variant, n, n, kTunedOneSet)) return nullptr;
   const uint64_t bumps0 = t_own_bumps;
   t_last.key.valid = false;
   if (sym_fit(dev, d, form, n, false, sym_default_plan(form, n, d.sms), &t_last) != CN_OK) return nullptr;
@@ -1452,7 +1476,7 @@ cn_status symmetric_common(int64_t n, const float* pos_mass, float eps2, float* 
     const uint64_t bumps0 = t_own_bumps;
     cn_tune pot_tune{};
     const cn_tune* shape = nullptr;
-    if (pot && !registered_tune(dev, cn::kSym, n, n)) {
+    if (pot && !registered_tune(dev, cn::kSym, n, n, kTunedOneSet)) {
       pot_tune = sym_default_tune(n, d->sms, true);
       shape = &pot_tune;
     }
@@ -1732,7 +1756,7 @@ cn_status build_group_plan(const std::vector<Group>& groups, bool lists, int64_t
   const int64_t key_i = static_cast<int64_t>(groups.size());
   cn_tune fitted{};
   double one_sided_s = 0.0;
-  if (!tune && !registered_tune(dev, variant, key_i, n_i_total)) {
+  if (!tune && !registered_tune(dev, variant, key_i, n_i_total, kTunedAny)) {
     // i-tile fitted to the group sizes: every group is cut into whole i-tiles,
     // so a tile larger than the typical group leaves lanes idle, and every
     // j range into whole j-tiles (padded with zero masses). Among the
@@ -2271,18 +2295,19 @@ size_t cn_workspace_bytes(int variant, int64_t n_i, int64_t n_j) {
     // accepted, and takes the pair kernel
     int dev = 0;
     DeviceInfo* d = nullptr;
-    if (current_device(&dev, &d) != CN_OK || registered_tune(dev, variant, n_i, n_j)) return need;
+    if (current_device(&dev, &d) != CN_OK) return need;
     const bool pot = variant == cn::kF32Pot;
     const cn::SymForm form = pot ? cn::kSymForcePot : cn::kSymForce;
     const cn::RowForm rows = pot ? cn::kRowForcePot : cn::kRowForce;
     SymPlan sp;
-    if (n_i == n_j && sym_pays(form, n_i, d->sms) &&
+    if (n_i == n_j && sym_pays(form, n_i, d->sms) && !registered_tune(dev, variant, n_i, n_j, kTunedOneSet) &&
         sym_fit(dev, *d, form, n_i, false, sym_default_plan(form, n_i, d->sms), &sp) == CN_OK)
       need = std::max(need, sp.need);
     Plan p;
     Geometry g;
     RowPlan rp;
-    if (resolve_plan(dev, variant, n_i, n_j, false, nullptr, &p) == CN_OK &&
+    if (!registered_tune(dev, variant, n_i, n_j, kTunedTwoSets) &&
+        resolve_plan(dev, variant, n_i, n_j, false, nullptr, &p) == CN_OK &&
         single_geometry(dev, *d, variant, false, p, n_i, n_j, &g) == CN_OK &&
         rows_pays(rows, n_i, n_j, d->sms, p, g) && rows_fit(dev, *d, rows, n_i, n_j, &rp) == CN_OK)
       need = std::max(need, rp.need);
@@ -2613,17 +2638,7 @@ cn_status cn_tune_set(int variant, int64_t n_i, int64_t n_j, const cn_tune* tune
       cn_status st = check_tune(variant, *tune);
       if (st != CN_OK) return st;
     }
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return fail_cuda(e, "cudaGetDevice");
-    std::lock_guard<std::mutex> lock(g_mu);
-    const auto key = std::make_tuple(dev, variant, bucket(n_i), bucket(n_j));
-    if (tune)
-      g_tune[key] = *tune;
-    else
-      g_tune.erase(key);
-    g_plan_gen.fetch_add(1, std::memory_order_acq_rel);
-    return CN_OK;
+    return store_tune(variant, n_i, n_j, tune, kTunedAny);
   });
 }
 
@@ -2648,14 +2663,15 @@ cn_status cn_tune_save(const char* path) {
       bool first = true;
       for (const auto& kv : g_tune) {
         if (std::get<0>(kv.first) != dev) continue;
-        const cn_tune& t = kv.second;
+        const cn_tune& t = kv.second.t;
+        const char* const on[] = {"", ", \"sets\": \"one\"", ", \"sets\": \"two\""};
         char line[512];
         std::snprintf(line, sizeof(line),
                       "%s\n  {\"variant\": \"%s\", \"n_i_class\": %d, \"n_j_class\": %d, \"i_per_thread\": %d, "
                       "\"threads\": %d, \"j_tile\": %d, \"stages\": %d, \"ctas_per_sm\": %d, \"chunk_units\": %d, "
-                      "\"j_lanes\": %d}",
+                      "\"j_lanes\": %d%s}",
                       first ? "" : ",", variant_name(std::get<1>(kv.first)), std::get<2>(kv.first), std::get<3>(kv.first),
-                      t.i_per_thread, t.threads, t.j_tile, t.stages, t.ctas_per_sm, t.chunk_units, t.j_lanes);
+                      t.i_per_thread, t.threads, t.j_tile, t.stages, t.ctas_per_sm, t.chunk_units, t.j_lanes, on[kv.second.on]);
         out += line;
         first = false;
       }
@@ -2699,6 +2715,7 @@ cn_status cn_tune_load(const char* path, int32_t* n_loaded) {
     struct Entry {
       int variant, ci, cj;
       cn_tune t;
+      TunedOn on;
     };
     std::vector<Entry> parsed;
     for (const JsonValue& e : entries->items) {
@@ -2715,7 +2732,12 @@ cn_status cn_tune_load(const char* path, int32_t* n_loaded) {
       Entry en{variant, static_cast<int>(ci), static_cast<int>(cj),
                cn_tune{static_cast<int32_t>(k), static_cast<int32_t>(th), static_cast<int32_t>(jt),
                        static_cast<int32_t>(stg), static_cast<int32_t>(cps), static_cast<int32_t>(ch),
-                       static_cast<int32_t>(jl)}};
+                       static_cast<int32_t>(jl)}, kTunedAny};
+      if (const JsonValue* on = e.get("sets")) {
+        if (on->kind != JsonValue::kString || (on->text != "one" && on->text != "two"))
+          return fail(CN_ERR_INVALID_ARG, "tuning file: an entry has a missing or out-of-range field");
+        en.on = on->text == "one" ? kTunedOneSet : kTunedTwoSets;
+      }
       const cn_status st = check_tune(variant, en.t);
       if (st != CN_OK) return st;
       parsed.push_back(en);
@@ -2733,7 +2755,7 @@ cn_status cn_tune_load(const char* path, int32_t* n_loaded) {
                                                  arch + ", " + std::to_string(sms) + " SMs)");
     {
       std::lock_guard<std::mutex> lock(g_mu);
-      for (const Entry& en : parsed) g_tune[std::make_tuple(dev, en.variant, en.ci, en.cj)] = en.t;
+      for (const Entry& en : parsed) g_tune[std::make_tuple(dev, en.variant, en.ci, en.cj)] = Tuned{en.t, en.on};
       g_plan_gen.fetch_add(1, std::memory_order_acq_rel);
     }
     if (n_loaded) *n_loaded = static_cast<int32_t>(parsed.size());
@@ -2762,7 +2784,8 @@ cn_status cn_autotune(int variant, int64_t n_i, const float* pos_i, int64_t n_j,
     cn_tune best{};
     cn_status result = CN_OK;
     std::vector<cn_tune> cands;
-    bool self = false;
+    const TunedOn on = pos_i == pos_mass_j && n_i == n_j ? kTunedOneSet : kTunedTwoSets;
+    bool other = false;  // the call without an entry takes another kernel than the pair kernel
     {
       // the default shape of these sizes first (its j-tile fitted to the
       // schedule, which the grid below does not contain), so that the result
@@ -2772,7 +2795,16 @@ cn_status cn_autotune(int variant, int64_t n_i, const float* pos_i, int64_t n_j,
       cn_status st = current_device(&dev, &d);
       if (st != CN_OK) return st;
       cands.push_back(default_tune(variant, n_i, n_j, d->sms));
-      self = !dd && pos_i == pos_mass_j && n_i == n_j && sym_pays(cn::kSymForce, n_i, d->sms);
+      if (!dd && !needs_guard(eps2)) {
+        Plan p;
+        Geometry g;
+        if (on == kTunedOneSet && sym_pays(cn::kSymForce, n_i, d->sms))
+          other = true;
+        else
+          other = resolve_plan(dev, variant, n_i, n_j, false, &cands.front(), &p) == CN_OK &&
+                  single_geometry(dev, *d, variant, false, p, n_i, n_j, &g) == CN_OK &&
+                  rows_pays(pot ? cn::kRowForcePot : cn::kRowForce, n_i, n_j, d->sms, p, g);
+      }
     }
     for (int k : ks) {
       if (!valid_k(variant, k)) continue;
@@ -2812,16 +2844,15 @@ cn_status cn_autotune(int variant, int64_t n_i, const float* pos_i, int64_t n_j,
       return force_common(dd, n_i, pos_i, n_j, pos_mass_j, eps2, acc_out, pot ? pot_out : nullptr, nullptr, 0, true,
                           ts);
     };
-    // A set against itself takes the symmetric form (from sym_pays) unless a
-    // tune is registered: that default is timed first, as the candidate
-    // without an entry.
-    if (self) cands.insert(cands.begin(), cands.front());
-    bool untuned = self, best_untuned = false;
+    // Without an entry the symmetric or the row kernel may take the call: that
+    // default is timed first, as the candidate without an entry.
+    if (other) cands.insert(cands.begin(), cands.front());
+    bool untuned = other, best_untuned = false;
     for (const cn_tune& t : cands) {
       if (check_tune(variant, t) != CN_OK) continue;
       const bool bare = untuned;
       untuned = false;
-      cn_tune_set(variant, n_i, n_j, bare ? nullptr : &t);
+      store_tune(variant, n_i, n_j, bare ? nullptr : &t, on);
       cn_status st = call();  // warm-up (and workspace growth)
       if (st == CN_ERR_INVALID_ARG) continue;  // shape does not fit
       if (st != CN_OK) {
@@ -2875,7 +2906,7 @@ cn_status cn_autotune(int variant, int64_t n_i, const float* pos_i, int64_t n_j,
       cn_tune_set(variant, n_i, n_j, nullptr);
       return fail(CN_ERR_INVALID_ARG, "no candidate launch shape fits");
     }
-    cn_tune_set(variant, n_i, n_j, best_untuned ? nullptr : &best);
+    store_tune(variant, n_i, n_j, best_untuned ? nullptr : &best, on);
     if (best_out) *best_out = best;
     return CN_OK;
   });
@@ -2907,7 +2938,7 @@ cn_status cn_autotune_batched(int32_t n_clusters, const int64_t* offsets_host, c
     int dev = 0;
     cudaGetDevice(&dev);
     cn_tune before{}, bare_shape{};
-    const bool had = registered_tune(dev, variant, n_clusters, n_total);
+    const bool had = registered_tune(dev, variant, n_clusters, n_total, kTunedAny);
     if (had) cn_tune_get(variant, n_clusters, n_total, &before);
     cn_tune_set(variant, n_clusters, n_total, nullptr);
     bool best_bare = false;
