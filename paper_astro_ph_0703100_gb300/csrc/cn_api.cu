@@ -929,7 +929,7 @@ cn_status check_records(const float* p, int64_t n, const char* name) {
 // Shape, workspace and layout of a symmetric launch.
 struct SymPlan {
   PlanCache key;
-  int k = 0, threads = 0, chunk = 0, stages = 0;
+  int k = 0, threads = 0, chunk = 0, stages = 0, fold = 0;
   bool guard = false;
   int64_t tile = 0, tiles = 0, n_blocks = 0, n_pad = 0;
   int64_t band = 0;  // tile rows per launch
@@ -967,6 +967,7 @@ cn_status sym_fit(int dev, const DeviceInfo& d, cn::SymForm form, int64_t n, boo
   sp->k = guard ? 2 : std::min(ops.max_k, std::max(2, p.k));
   sp->threads = p.threads;
   sp->guard = guard;
+  sp->fold = ops.max_stage / cn::kSymBlock;
   sp->chunk = static_cast<int>(std::min<int64_t>(round_up(p.j_tile, cn::kSymBlock), ops.max_stage));
   sp->stages = std::max(2, p.stages);  // a stage is refilled a chunk after it was read
   sp->tile = static_cast<int64_t>(sp->k) * sp->threads;
@@ -994,7 +995,9 @@ cn_status sym_fit(int dev, const DeviceInfo& d, cn::SymForm form, int64_t n, boo
   else if (static_cast<double>(sp->tiles) * static_cast<double>(row_b) > static_cast<double>(kSymSlotCap))
     sp->band = std::max<int64_t>(1, std::min<int64_t>(sp->tiles, static_cast<int64_t>(kSymSlotCap / row_b)));
   sp->jslot_b = align_up(static_cast<size_t>(sp->band) * row_b, 256);
-  sp->seg_b = align_up(static_cast<size_t>(sp->slots + sp->band) * static_cast<size_t>(sp->tile) * word, 256);
+  sp->seg_b = align_up(static_cast<size_t>(sp->slots + sp->band) * static_cast<size_t>(sp->tile) * sizeof(float) *
+                           static_cast<size_t>(ops.planes),
+                       256);
   sp->need = sp->jslot_b + sp->seg_b + (sp->band < sp->tiles ? 2 * row_b : 0);
   return CN_OK;
 }
@@ -1014,6 +1017,7 @@ cn_status sym_launch(const std::string& what, const DeviceInfo& d, cn::SymForm f
   a.status = d.status;
   a.n_pad = sp.n_pad;
   a.chunk = sp.chunk;
+  a.fold = sp.fold;
   a.stages = sp.stages;
   a.eps2 = eps2;
   // a mass-free term of these forms is at most 4 eps^-3 |w| with |w| <= 2 sqrt(3) of the largest component, and
@@ -1023,7 +1027,7 @@ cn_status sym_launch(const std::string& what, const DeviceInfo& d, cn::SymForm f
   cn::SymMerge m{};
   m.slots_seg = a.slots_seg;
   m.slots_j = a.slots_j;
-  m.carry = sp.band < sp.tiles ? reinterpret_cast<float2*>(sp.data + sp.jslot_b + sp.seg_b) : nullptr;
+  m.carry = sp.band < sp.tiles ? reinterpret_cast<double*>(sp.data + sp.jslot_b + sp.seg_b) : nullptr;
   for (int o = 0; o < 3; ++o) m.out[o] = out[o];
   m.n_pad = sp.n_pad;
   m.tile = static_cast<int32_t>(sp.tile);
@@ -1037,6 +1041,8 @@ cn_status sym_launch(const std::string& what, const DeviceInfo& d, cn::SymForm f
     a.g.cost = a.g.row_start(r1) - a.g.cost0;
     a.g.grid = static_cast<int32_t>(std::max<int64_t>(1, std::min<int64_t>(sp.slots, a.g.cost / cn::kSymCostPair)));
     m.g = a.g;
+    // parts of more than 1024 records
+    a.both_words = a.g.cost > static_cast<int64_t>(a.g.grid) * cn::kSymCostPair * (1024 / cn::kSymBlock);
     m.first = r0 == 0;
     m.last = r1 == sp.tiles;
     if (log_enabled()) {
@@ -1507,6 +1513,7 @@ cn_status launch_ensemble(const DeviceInfo& d, const cn_batch_plan* plan, const 
   a.n_seg = plan->sym_seg;
   a.status = d.status;
   a.chunk = plan->sym_chunk;
+  a.fold = cn::sym_ops(form).max_stage / cn::kSymBlock;
   a.stages = plan->sym_stages;
   a.wait_ns = g_wait_ns.load();
   a.rows = plan->d_rows;

@@ -51,7 +51,10 @@
 // j-side sums go to one slot per (row, block), i-side sums to one segment
 // per (CTA, row), both as planes of one float per particle; a second kernel
 // adds them per particle in a fixed order: the result is deterministic,
-// with no atomics on data.
+// with no atomics on data. A part of more than 1024 records is the sum of
+// several register chains; in the force forms its segment then keeps the low
+// words as well (131072 4003 / 4009 us, all segments at all sizes: 4096 .. 24576
+// 2 to 7% slower, for words that are zero while a segment is one chain).
 #pragma once
 
 #include "cn_device.cuh"
@@ -62,12 +65,20 @@ namespace cn {
 constexpr float kSymFar = 1e11f;       // |coordinate| up to which r^-3 stays a normal number
 constexpr float kSymSoft = 1e-20f;     // eps2 from which it stays finite
 constexpr float kSymStiff = 1e24f;     // eps2 up to which it stays a normal number
-constexpr float kSymHuge = 3.4e38f;    // finite
+constexpr float kSymHuge = 3.402823466e38f;  // finite
 
 enum SymMode : int {
   kSymUniform = 0,  // equal masses, factored out of the pair terms
   kSymGeneral = 1,  // r^-3 times either mass
   kSymWide = 2,     // (m r)(r r): any range
+};
+
+// of a warp's own particles
+enum SymOwn : int {
+  kOwnEqual = 1,  // equal masses
+  kOwnNear = 2,   // r^-3 in range
+  kOwnClose = 4,  // within kHeavyReach and kHeavySoft
+  kOwnSlow = 8,   // second records within SymArgs::fast
 };
 
 __device__ __forceinline__ float sym_reach(const float4& v) {
@@ -83,9 +94,14 @@ __device__ __forceinline__ float& sym_half(float2& v, int k) { return (k & 1) ? 
 //   kRec            float4 words per record (2: a velocity or a loss weight)
 //   kMinBlocks      256-thread CTAs per SM the registers are limited for
 //   kUnroll         steps per loop trip (divides 32)
-//   kFold           j records summed in FP32 registers between TwoSum folds
+//   kFold           j records summed in FP32 registers between TwoSum folds, at
+//                   most (SymArgs::fold, where a stage is one sweep)
 //   kStage          records per stage, at most
 //   kWide           offers the kSymWide terms
+//   kLow            long segments keep their low words (single systems)
+//   kRolled         the loop that writes a segment is not unrolled over its
+//                   sums: which is the faster one is up to the registers that
+//                   the compiler then finds for the sweeps (2%, measured)
 //   kSameMass       equal masses factor out only if the warp's and the
 //                   chunk's are the same
 //   kHeavyReach     |coordinate| (with a second record) and eps2 up to which
@@ -114,6 +130,8 @@ struct SymForcePolicy {
   static constexpr int kStage = FOLD < 256 ? FOLD : 256;
   static constexpr int kMinBlocks = 2;
   static constexpr bool kWide = true;
+  static constexpr bool kLow = true;
+  static constexpr bool kRolled = (POT && K >= 4) || FOLD < 256;
   static constexpr bool kSameMass = false;
   // r^-3 d is at least 1e-23 where d is the longer one, r^-3 at least 1e-18 where eps is
   static constexpr float kHeavySoft = 1e12f;
@@ -272,6 +290,7 @@ struct SymControl {
   uint64_t done[3];  // a chunk swept by every warp (and the chunk before it added up)
   int32_t abort;
   uint32_t issued;   // chunks staged (thread 0)
+  int32_t own[8];    // with a second record: what holds for each warp's own particles (kOwn...)
   SymCursor ahead;   // the next one (thread 0)
   int64_t end;
   SymChunk chunk[16];
@@ -346,6 +365,8 @@ template <class Pol, bool BATCHED>
 __global__ void __launch_bounds__(256, Pol::kMinBlocks) sym_kernel(const __grid_constant__ SymArgs a) {
   extern __shared__ __align__(1024) unsigned char smem[];
   constexpr int K = Pol::K, P = Pol::P, NI = Pol::kSumsI, NJ = Pol::kSumsJ, JR = Pol::kRec;
+  constexpr bool LOW = Pol::kLow && !BATCHED;
+  constexpr int NS = LOW ? 2 * NI : NI;  // planes of a segment
   const int NT = blockDim.x;
   const int tid = threadIdx.x;
   const int lane = tid & 31;
@@ -385,9 +406,8 @@ __global__ void __launch_bounds__(256, Pol::kMinBlocks) sym_kernel(const __grid_
   float scale = 1.f;   // of the sums in registers
   int held = 0;        // j blocks in them
 
-  // the warp's own particles: equal masses that may factor out; r^-3 in range; (with a second
-  // record) within kHeavyReach and kHeavySoft; second records within a.fast
-  bool own_uniform = false, own_near = false, own_close = false, own_slow = false;
+  // the warp's own particles: equal masses that may factor out; r^-3 in range
+  bool own_uniform = false, own_near = false;
   // the largest mass that may factor out, by the softening alone
   auto heaviest = [&]() { return e2.x <= Pol::kHeavySoft ? kSymHuge : 1.f; };
 
@@ -411,17 +431,26 @@ __global__ void __launch_bounds__(256, Pol::kMinBlocks) sym_kernel(const __grid_
       for (int c = 0; c < NI; ++c) acc.acc[p][c] = make_float2(0.f, 0.f);
     held = 0;
   };
-  // writes the row's i-side sums to this CTA's segment
+  // writes the row's i-side sums to this CTA's segment: their totals and, where
+  // asked for, what those lack
   auto flush = [&](int32_t I) {
     fold();
-    float* seg = a.slots_seg + (static_cast<size_t>(blockIdx.x) + static_cast<size_t>(I - a.g.row0)) * NI * B;
-#pragma unroll
+    const bool both = LOW && a.both_words;
+    float* seg = a.slots_seg + (static_cast<size_t>(blockIdx.x) + static_cast<size_t>(I - a.g.row0)) * NS * B;
+#pragma unroll(Pol::kRolled ? 1 : NI)
     for (int c = 0; c < NI; ++c)
 #pragma unroll
       for (int k = 0; k < K; ++k) {
         const int e = c * B + k * NT + tid;
         seg[e] = pair_total(sums[e], sums[e + NI * B]);
       }
+    if (both) {
+#pragma unroll 1
+      for (int e = tid; e < NI * B; e += NT) {
+        const float h = sums[e], l = sums[e + NI * B];
+        seg[e + NI * B] = __fadd_rn(__fadd_rn(h, -pair_total(h, l)), l);
+      }
+    }
   };
   // once every warp has swept chunk q: refills its stage (thread 0) and adds
   // up this warp's share of its j-side sums, over the warps in order
@@ -500,8 +529,9 @@ __global__ void __launch_bounds__(256, Pol::kMinBlocks) sym_kernel(const __grid_
       own_uniform = __all_sync(0xffffffffu, same && fabsf(m0) <= (JR == 2 ? kSymHuge : heaviest()));
       own_near = __all_sync(0xffffffffu, near && e2.x >= kSymSoft && e2.x <= kSymStiff);
       if constexpr (JR == 2) {
-        own_close = __all_sync(0xffffffffu, close && e2.x <= Pol::kHeavySoft);
-        own_slow = __all_sync(0xffffffffu, slow);
+        close = __all_sync(0xffffffffu, close && e2.x <= Pol::kHeavySoft);
+        slow = __all_sync(0xffffffffu, slow);
+        ctl->own[warp] = (own_uniform ? kOwnEqual : 0) | (own_near ? kOwnNear : 0) | (close ? kOwnClose : 0) | (slow ? kOwnSlow : 0);
       }
 #pragma unroll
       for (int p = 0; p < P; ++p)
@@ -521,10 +551,19 @@ __global__ void __launch_bounds__(256, Pol::kMinBlocks) sym_kernel(const __grid_
     float factor = 1.f;
     if constexpr (!Pol::kGuard) {
       const float mj = js[0].w;
+      bool own_close = true, own_slow = true;
+      if constexpr (JR == 2) {
+        const int own = ctl->own[warp];
+        own_uniform = own & kOwnEqual;
+        own_near = own & kOwnNear;
+        own_close = own & kOwnClose;
+        own_slow = own & kOwnSlow;
+      }
       // with a second record the positions count too where either mass is above 1
       const bool heavy = JR == 2 && (fabsf(mj) > 1.f || (own_uniform && fabsf(mass[tid]) > 1.f));
       bool same = fabsf(mj) <= (JR == 2 ? kSymHuge : heaviest()), near = own_near;
       if constexpr (JR == 2) same = same && own_slow && (!heavy || own_close);
+#pragma unroll(JR == 2 ? 1 : 4)
       for (int t = lane; t < count; t += 32) {
         const float4 v = js[t];
         const float reach = sym_reach(v);
@@ -547,7 +586,7 @@ __global__ void __launch_bounds__(256, Pol::kMinBlocks) sym_kernel(const __grid_
     constexpr int kStep = Pol::kFold / kSymBlock;  // blocks between folds, at most
     // the blocks b0 .. b0 + nb - 1 of the chunk
     auto sweep = [&](int b0, int nb) {
-      if (held > 0 && (factor != scale || held + nb > kStep)) fold();
+      if (held > 0 && (factor != scale || held + nb > (Pol::kFold >= Pol::kStage ? a.fold : kStep))) fold();
       scale = factor;
       held += nb;
       if (ch.diag) {
@@ -612,9 +651,11 @@ __global__ void __launch_bounds__(256, Pol::kMinBlocks) sym_kernel(const __grid_
 // An ensemble's particles have few of either: 2 warps there.
 template <bool BATCHED>
 constexpr int kSymMergeWarps = BATCHED ? 2 : 8;
-template <class Pol, bool BATCHED>
+// LOW: the segments have low words.
+template <class Pol, bool BATCHED, bool LOW>
 __global__ void __launch_bounds__(32 * kSymMergeWarps<BATCHED>) sym_merge_kernel(const __grid_constant__ SymMerge m) {
   constexpr int NI = Pol::kSumsI, NW = kSymMergeWarps<BATCHED>;
+  constexpr int NS = Pol::kLow && !BATCHED ? 2 * NI : NI;  // planes of a segment
   __shared__ float2 part[NW][NI][32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   int64_t p, jrow = 0;  // the particle; the first row with a slot of it
@@ -634,7 +675,7 @@ __global__ void __launch_bounds__(32 * kSymMergeWarps<BATCHED>) sym_merge_kernel
     nj = mb.row - mb.first;
     const int64_t c0 = m.g.owner(r.cost);
     ns = static_cast<int>(m.g.owner(r.last()) - c0 + 1);
-    seg = m.slots_seg + static_cast<size_t>(c0 + mb.row) * NI * m.tile + (local - r.blk0 * kSymBlock);
+    seg = m.slots_seg + static_cast<size_t>(c0 + mb.row) * NS * m.tile + (local - r.blk0 * kSymBlock);
   } else {
     p = static_cast<int64_t>(blk) * kSymBlock + lane;
     valid = p < m.g.n;
@@ -647,7 +688,7 @@ __global__ void __launch_bounds__(32 * kSymMergeWarps<BATCHED>) sym_merge_kernel
       const int64_t last = s1 - (m.g.diag_end(I) < m.g.n_blocks ? kSymCostPair : kSymCostDiag);
       const int64_t c0 = m.g.owner(s0), c1 = m.g.owner(last);
       ns = static_cast<int>(c1 - c0 + 1);
-      seg = m.slots_seg + (static_cast<size_t>(c0) + static_cast<size_t>(I - m.g.row0)) * NI * m.tile +
+      seg = m.slots_seg + (static_cast<size_t>(c0) + static_cast<size_t>(I - m.g.row0)) * NS * m.tile +
             static_cast<size_t>(p - static_cast<int64_t>(I) * m.tile);
     }
     slot = m.slots_j + static_cast<size_t>(p);
@@ -660,13 +701,21 @@ __global__ void __launch_bounds__(32 * kSymMergeWarps<BATCHED>) sym_merge_kernel
   for (int c = 0; c < NI; ++c) hi[c] = lo[c] = 0.f;
   constexpr int kAhead = 4;
   for (int q = warp; q < total; q += kAhead * NW) {
-    float w[kAhead][NI];
+    float w[kAhead][NI], v[LOW ? kAhead : 1][NI];  // high words; low words of segments
 #pragma unroll
     for (int u = 0; u < kAhead; ++u) {
       const int e = q + u * NW;
       if (e < total && valid) {
-        const float* src = seg + static_cast<int64_t>(e - nj) * NI * m.tile;
+        const float* src = seg + static_cast<int64_t>(e - nj) * NS * m.tile;
         int64_t plane = m.tile;
+        if constexpr (LOW) {
+#pragma unroll
+          for (int c = 0; c < NI; ++c) v[u][c] = 0.f;
+          if (e >= nj) {
+#pragma unroll
+            for (int c = 0; c < NI; ++c) v[u][c] = __ldcs(src + (NI + c) * plane);
+          }
+        }
         if (e < nj) {
           if constexpr (BATCHED) {
             const SymRow& r = m.rows[jrow + e];
@@ -688,6 +737,7 @@ __global__ void __launch_bounds__(32 * kSymMergeWarps<BATCHED>) sym_merge_kernel
         for (int c = 0; c < NI; ++c) {
           float e;
           two_sum(hi[c], w[u][c], hi[c], e);
+          if constexpr (LOW) e = __fadd_rn(e, v[u][c]);
           lo[c] = __fadd_rn(lo[c], e);
         }
       }
@@ -698,21 +748,25 @@ __global__ void __launch_bounds__(32 * kSymMergeWarps<BATCHED>) sym_merge_kernel
   if (!valid) return;
   for (int c = warp; c < NI; c += NW) {
     float h = 0.f, l = 0.f;
-    if (!m.first) {
-      const float2 v = m.carry[static_cast<size_t>(c) * m.n_pad + p];
-      h = v.x;
-      l = v.y;
-    }
 #pragma unroll
     for (int w = 0; w < NW; ++w) {
       float e;
       two_sum(h, part[w][c][lane].x, h, e);
       l = __fadd_rn(l, __fadd_rn(e, part[w][c][lane].y));
     }
-    if (m.last)
+    if (m.first && m.last) {
       Pol::output(m, p, c, pair_total(h, l));
+      continue;
+    }
+    // bands: few and long, so that their sums can be added in FP64
+    double* carry = m.carry + static_cast<size_t>(c) * m.n_pad + p;
+    double t = m.first ? 0.0 : *carry;
+    t += static_cast<double>(h);
+    if (fabsf(h) <= kSymHuge) t += static_cast<double>(l);
+    if (m.last)
+      Pol::output(m, p, c, static_cast<float>(t));
     else
-      m.carry[static_cast<size_t>(c) * m.n_pad + p] = make_float2(h, l);
+      *carry = t;
   }
 }
 
@@ -753,11 +807,13 @@ struct SymTable {
       e = launch_pdl(f, dim3(static_cast<unsigned>(a.g.grid)), dim3(threads), args, bytes, s);
       if (e != cudaSuccess) return e;
       void* margs[] = {const_cast<SymMerge*>(&m)};
-      return launch_pdl(reinterpret_cast<const void*>(&sym_merge_kernel<decltype(pol), BATCHED>),
-                        dim3(static_cast<unsigned>(m.n_merge)), dim3(32 * kSymMergeWarps<BATCHED>), margs, 0, s);
+      const void* merge = reinterpret_cast<const void*>(&sym_merge_kernel<decltype(pol), BATCHED, false>);
+      if constexpr (P2::kLow && !BATCHED)
+        if (a.both_words) merge = reinterpret_cast<const void*>(&sym_merge_kernel<decltype(pol), BATCHED, true>);
+      return launch_pdl(merge, dim3(static_cast<unsigned>(m.n_merge)), dim3(32 * kSymMergeWarps<BATCHED>), margs, 0, s);
     });
   }
-  static SymOps ops(int max_k) { return SymOps{P2::kSumsI, max_k, P2::kStage, &smem, &occupancy, &launch}; }
+  static SymOps ops(int max_k) { return SymOps{P2::kSumsI, P2::kLow && !BATCHED ? 2 * P2::kSumsI : P2::kSumsI, max_k, P2::kStage, &smem, &occupancy, &launch}; }
 };
 
 }  // namespace cn

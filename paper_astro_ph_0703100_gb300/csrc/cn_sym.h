@@ -183,9 +183,10 @@ struct SymMergeBlock {
 };
 
 // A launch. Sum d of the i side of particle p goes to plane d of the (CTA c,
-// row I) segment, slots_seg[((c + I - row0) * sums + d) * tile + p - I tile]
+// row I) segment, slots_seg[((c + I - row0) * planes + d) * tile + p - I tile]
 // (c + I - row0 is unique per segment, since along the cost line neither the
-// CTA nor the row decreases); of the j side under row I to
+// CTA nor the row decreases); the force forms have a second plane each, for
+// the sums' low words where both_words is set. Sum d of the j side under row I to
 // slots_j[((I - row0) * sums + d) * n_pad + p].
 struct SymArgs {
   SymGrid g;
@@ -194,9 +195,11 @@ struct SymArgs {
   float* slots_seg;
   float* slots_j;
   int* status;
+  int32_t both_words;
   int64_t n_seg;       // allocated segments
   int64_t n_pad;       // n_blocks * 32
   int32_t chunk;       // j records per ring stage (multiple of 32)
+  int32_t fold;        // blocks summed in registers between folds (at least a stage's)
   int32_t stages;
   float eps2;
   float fast;          // forms with a second record: its largest component for the mass-free terms
@@ -208,13 +211,12 @@ struct SymArgs {
 // Per-particle merge of one launch: the j-side slots of rows I < P (the
 // particle's tile) in ascending order, then the segments of row P in CTA
 // order, summed in (hi, lo) pairs by TwoSum; with several bands the sums
-// are carried in acc64 as (hi, lo) words and the last band writes the
-// outputs.
+// are carried in FP64 and the last band writes the outputs.
 struct SymMerge {
   SymGrid g;
   const float* slots_seg;
   const float* slots_j;
-  float2* carry;      // [sums][n_pad] running (hi, lo) sums, NULL with a single band
+  double* carry;      // [sums][n_pad] running sums, NULL with a single band
   float* out[3];      // outputs, by form
   int64_t n_pad;
   int32_t tile;
@@ -235,12 +237,13 @@ enum SymForm : int {
   kSymBatchedPot = 6,
 };
 
-// A form's kernels: sums per particle, most particles per thread and records
-// per stage, shared
+// A form's kernels: sums per particle, planes of a segment, most particles per
+// thread and records per stage, shared
 // memory of a shape, resident CTAs per SM, and the launch of one band (pair
 // kernel and merge).
 struct SymOps {
   int sums;
+  int planes;
   int max_k;
   int max_stage;
   size_t (*smem)(int threads, int k, int chunk, int stages);

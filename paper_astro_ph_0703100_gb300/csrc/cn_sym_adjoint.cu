@@ -30,6 +30,8 @@ struct SymAdjointPolicy {
   static constexpr int kStage = 256;
   static constexpr int kMinBlocks = 2;
   static constexpr bool kWide = false;
+  static constexpr bool kLow = false;
+  static constexpr bool kRolled = true;
   static constexpr bool kSameMass = true;
   // as in the jerk form, for the weights
   static constexpr float kHeavyReach = 1e5f;

@@ -23,11 +23,13 @@ struct SymJerkPolicy {
   static constexpr int kSumsJ = kSumsI;
   static constexpr int kRec = 2;
   static constexpr bool kGuard = false;
-  static constexpr int kUnroll = K >= 8 ? 4 : 8;
+  static constexpr int kUnroll = K >= 8 && POT ? 4 : 8;
   static constexpr int kFold = 256;
   static constexpr int kStage = 256;
   static constexpr int kMinBlocks = 1;
   static constexpr bool kWide = true;
+  static constexpr bool kLow = false;
+  static constexpr bool kRolled = K >= 8 && !POT;
   static constexpr bool kSameMass = false;
   // r^-3 is at least 2e-17 there, and r^-3 w a normal number for |w| > 1e-21
   static constexpr float kHeavyReach = 1e5f;
