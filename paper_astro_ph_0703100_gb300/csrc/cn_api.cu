@@ -382,27 +382,34 @@ int64_t round_up(int64_t x, int64_t m) { return (x + m - 1) / m * m; }
 // (8 x 256 2.2e12 unordered pairs/s in the inner loop, 4 x 128 2.0e12, both
 // at 16 warps per SM); smaller ones cut the work finer over the CTAs and
 // waste less on the diagonal tiles, which are evaluated one-sided. Measured
-// (us, equal masses, 152 SMs, sums folded every 512 records, 8 steps per
-// trip: now 1 to 2% less at the large end; the lines lie where the order
-// changes, and another SM count moves them by the work per SM):
-//   n       2x128/128  4x128/256  8x128/128  8x256/128
-//   5000      16.7       16.8       19.3+      19.3+
-//   7000      25.3       23.6       25.0       25.2
-//   10000       -        37.5       39.7       39.7
-//   14000       -        65.2       63.6       64.8
-//   20000       -          -       113.7      111.8
-//   24576       -       167+       161.9      157.7
-//   50001       -          -       623        608
-//   131072      -          -      4159       4069
-// (threads x K / records per stage). With the potential the fourth sum takes
-// 64-record stages for two CTAs of 256 threads per SM: 50001 798 -> 790,
-// 131072 5343 -> 5250 against 8 x 128.
+// (us, equal masses, 152 SMs, folds as sym_fold has them; another SM count moves
+// the lines by the work per SM):
+//   n       2x128/128  4x128/256  4x256/128  8x128/128  8x256/128
+//   5000      16.7       16.8        -         19.3+      19.3+
+//   7000      25.3       22.9        -         25.0       25.2
+//   9001       -         31.3       33.3         -          -
+//   10007      -          -         37.7       39.7       39.7
+//   14000      -          -         62.6       64.9       64.8
+//   16384      -          -         80.8       79.7         -
+//   18000      -          -         95.4       99.1         -
+//   24000      -          -        159.6      157.8         -
+//   24576      -          -          -        161.9      156.5
+//   50001      -          -          -        623        605
+//   131072     -          -          -       4159       3985
+// (threads x K / records per stage). With the potential 4 x 256 stay ahead up to
+// 24576 (20000 142.4 us, 8 x 128 142.7, unequal masses 156.2 / 171.6), and
+// above the fourth sum takes 64-record stages for two CTAs of 256 threads per
+// SM: 50001 798 -> 790, 131072 5343 -> 5250 against 8 x 128.
+constexpr double kSymShort = 9700.0;   // where folds are short (sym_fold): from here ..
+constexpr double kSymLarge = 24576.0;  // .. to here
+
 cn_tune sym_default_tune(int64_t n, int sms, bool pot) {
   const double n_eff = static_cast<double>(n) * std::sqrt(152.0 / std::max(sms, 1));
+  const bool mid = n_eff >= kSymShort && n_eff < (pot ? kSymLarge : 16000.0);
   cn_tune t{};
-  t.i_per_thread = n_eff < 6000 ? 2 : n_eff < 12000 ? 4 : 8;
-  t.threads = n_eff < 24576 ? 128 : 256;
-  t.j_tile = n_eff >= 6000 && n_eff < 12000 ? 256 : pot && t.threads == 256 ? 64 : 128;
+  t.i_per_thread = n_eff < 6000 ? 2 : n_eff < kSymShort || mid ? 4 : 8;
+  t.threads = mid || n_eff >= kSymLarge ? 256 : 128;
+  t.j_tile = n_eff >= 6000 && n_eff < kSymShort ? 256 : pot && n_eff >= kSymLarge ? 64 : 128;
   t.stages = 3;
   t.j_lanes = 1;
   return t;
@@ -956,6 +963,20 @@ cn_status sym_occupancy(int dev, cn::SymForm form, const SymPlan& sp, int* ctas)
   return CN_OK;
 }
 
+// j blocks between the folds of register sums. Where the pair kernel's lane
+// groups split a j-tile into short chains, 256 records left a larger error than
+// it did (2-norm against 64 bits, geometric mean over 16 sets, cusps of unequal
+// masses: force 10007 1.20 of it, 13001 1.05, 18000 1.06, jerk 12000 1.07; now 0.99,
+// 0.96, 0.92, 0.88; Plummer spheres 0.58 .. 0.98). Below and above, 256 are at 0.5 ..
+// 0.99 of it and cost 1 to 2% less.
+int sym_fold(cn::SymForm form, int64_t n, int sms) {
+  const double n_eff = static_cast<double>(n) * std::sqrt(152.0 / std::max(sms, 1));
+  const bool force = form == cn::kSymForce || form == cn::kSymForcePot;
+  const bool jerk = form == cn::kSymJerk || form == cn::kSymJerkPot;
+  const bool few = force ? n_eff >= kSymShort && n_eff < kSymLarge : jerk && n_eff >= 7500.0 && n_eff < 16000.0;
+  return (few ? 128 : 256) / cn::kSymBlock;  // the adjoint's kernel folds within a stage
+}
+
 // Fits the plan of `form` for n particles (p: the shape); `need` bytes of
 // workspace go into data. The j-side slots of every off-diagonal unit take one
 // [rows][n_pad] array (half of it written) when that fits in kSymSlotCap,
@@ -967,8 +988,8 @@ cn_status sym_fit(int dev, const DeviceInfo& d, cn::SymForm form, int64_t n, boo
   sp->k = guard ? 2 : std::min(ops.max_k, std::max(2, p.k));
   sp->threads = p.threads;
   sp->guard = guard;
-  sp->fold = ops.max_stage / cn::kSymBlock;
-  sp->chunk = static_cast<int>(std::min<int64_t>(round_up(p.j_tile, cn::kSymBlock), ops.max_stage));
+  sp->fold = sym_fold(form, n, d.sms);
+  sp->chunk = static_cast<int>(std::min<int64_t>(round_up(p.j_tile, cn::kSymBlock), std::min(ops.max_stage, sp->fold * cn::kSymBlock)));
   sp->stages = std::max(2, p.stages);  // a stage is refilled a chunk after it was read
   sp->tile = static_cast<int64_t>(sp->k) * sp->threads;
   sp->tiles = ceil_div(n, sp->tile);
