@@ -400,8 +400,8 @@ int64_t round_up(int64_t x, int64_t m) { return (x + m - 1) / m * m; }
 // 24576 (20000 142.4 us, 8 x 128 142.7, unequal masses 156.2 / 171.6), and
 // above the fourth sum takes 64-record stages for two CTAs of 256 threads per
 // SM: 50001 798 -> 790, 131072 5343 -> 5250 against 8 x 128.
-constexpr double kSymShort = 9700.0;   // where folds are short (sym_fold): from here ..
-constexpr double kSymLarge = 24576.0;  // .. to here
+constexpr double kSymShort = 9700.0;   // where folds are short (sym_fold)
+constexpr double kSymLarge = 24576.0;  // from here 8 x 256
 
 cn_tune sym_default_tune(int64_t n, int sms, bool pot) {
   const double n_eff = static_cast<double>(n) * std::sqrt(152.0 / std::max(sms, 1));
@@ -968,12 +968,14 @@ cn_status sym_occupancy(int dev, cn::SymForm form, const SymPlan& sp, int* ctas)
 // it did (2-norm against 64 bits, geometric mean over 16 sets, cusps of unequal
 // masses: force 10007 1.20 of it, 13001 1.05, 18000 1.06, jerk 12000 1.07; now 0.99,
 // 0.96, 0.92, 0.88; Plummer spheres 0.58 .. 0.98). Below and above, 256 are at 0.5 ..
-// 0.99 of it and cost 1 to 2% less.
+// 0.99 of it and cost 1 to 2% less. Up to 26000 also against the reduce-scatter
+// kernel that cn_force_symmetric had, whose tiles are small until there (24577 1.13
+// of its error, now 1.01; 28000 0.66 with 256).
 int sym_fold(cn::SymForm form, int64_t n, int sms) {
   const double n_eff = static_cast<double>(n) * std::sqrt(152.0 / std::max(sms, 1));
   const bool force = form == cn::kSymForce || form == cn::kSymForcePot;
   const bool jerk = form == cn::kSymJerk || form == cn::kSymJerkPot;
-  const bool few = force ? n_eff >= kSymShort && n_eff < kSymLarge : jerk && n_eff >= 7500.0 && n_eff < 16000.0;
+  const bool few = force ? n_eff >= kSymShort && n_eff < 26000.0 : jerk && n_eff >= 7500.0 && n_eff < 16000.0;
   return (few ? 128 : 256) / cn::kSymBlock;  // the adjoint's kernel folds within a stage
 }
 

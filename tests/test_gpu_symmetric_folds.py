@@ -15,8 +15,8 @@ from gpu_common import dev_tensor, lib
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("form,n", [("force", 12000), ("force", 18000), ("pot", 12000), ("pot", 20000), ("jerk", 9000),
-                                    ("jerk", 15000)])
+@pytest.mark.parametrize("form,n", [("force", 12000), ("force", 18000), ("pot", 12000), ("pot", 20000),
+                                    ("symmetric", 25001), ("jerk", 9000), ("jerk", 15000)])
 def test_light_records_behind_a_heavy_one(form, n):
     cn = lib()
     # two masses in turn: those of a stage that were all equal would be summed apart
@@ -31,6 +31,8 @@ def test_light_records_behind_a_heavy_one(form, n):
         if form == "jerk":
             v = dev_tensor(np.zeros((n, 4), dtype=np.float32))
             out = cn.cn_force_jerk(d, v, d, v, 1.0)[0]
+        elif form == "symmetric":
+            out = cn.cn_force_symmetric(d, 1.0)[0]
         else:
             a, phi = cn.cn_force(d, d, 1.0, potential=form == "pot")
             out = a if phi is None else phi
