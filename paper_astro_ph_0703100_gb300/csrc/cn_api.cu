@@ -457,6 +457,8 @@ int32_t fit_j_tile(int64_t n_i, int64_t n_j, int64_t i_tile, int32_t lo, int32_t
   return best_t;
 }
 
+constexpr int64_t kDDSmall = 10500;  // particles from which the compensated form has fixed shapes
+
 // The j-tile of a small compensated call in tiles of 64 i-particles (one per
 // thread). Such a call is a chain of latencies, not work: a pair term takes
 // about 0.06 us of one warp, and one warp per scheduler (two CTAs of 64
@@ -603,7 +605,7 @@ cn_tune default_tune(int variant, int64_t n_i, int64_t n_j, int sms) {
     t.i_per_thread = 4;
     t.threads = 256;
     t.j_tile = fit_j_tile(n_i, n_j, 1024, 256, 1024, 16, sms, 9);
-  } else if (dd && n < 10500) {
+  } else if (dd && n < kDDSmall) {
     // compensated form, small systems: one i-particle per thread in CTAs of 64
     // threads fills the SMs and its CTAs are many enough to even out the last
     // round. Up to 1.894e7 pairs the j-tile is fitted (dd_small_j_tile); above,
@@ -2319,6 +2321,23 @@ cn_status cn_force_dd_ws(int64_t n_i, const float* pos_i, int64_t n_j, const flo
 size_t cn_workspace_bytes(int variant, int64_t n_i, int64_t n_j) {
   return cn::guard_value<size_t>(0, [&]() -> size_t {
     size_t need = cn::one_sided_workspace_bytes(variant, n_i, n_j);
+    if (need != 0 && (variant == cn::kDD || variant == cn::kDDPot)) {
+      // enough for any part of these sets too: the small shapes' j-tiles are
+      // fitted to the sizes, so a smaller call may be cut into more units. None
+      // has more than tiles of 64 by 32.
+      int dev = 0;
+      DeviceInfo* d = nullptr;
+      Plan p;
+      p.k = 1;
+      p.threads = 64;
+      p.j_tile = 32;
+      p.stages = 4;
+      Geometry g;
+      if (current_device(&dev, &d) == CN_OK &&
+          single_geometry(dev, *d, variant, false, p, std::min(n_i, kDDSmall), std::min(n_j, kDDSmall), &g) == CN_OK)
+        need = std::max(need, g.ws_bytes);
+      return need;
+    }
     if (need == 0 || (variant != cn::kF32 && variant != cn::kF32Pot)) return need;
     // the slots of the symmetric form (one set against itself) and the
     // segments of the row kernel; a smaller buffer that holds the above is
