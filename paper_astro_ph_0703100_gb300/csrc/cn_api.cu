@@ -468,13 +468,19 @@ constexpr int64_t kDDSmall = 10500;  // particles from which the compensated for
 // j-tile with the least of the sum; in a sweep of 13 j-tiles it was the
 // fastest one at every size tried up to 2600 (us, 2 x 64 threads with 128
 // records before / now: 256 22.3 / 11.5, 1100 31.8 / 19.6, 2048 41.6 / 27.6, 2600
-// 61.6 / 35.3, 100 x 4000 59.7 / 31.2). From 1.4e7 pairs on the units of a
-// round no longer wait for one another and tiles up to 256 are the better ones
-// (4095: 224 records 72 us, 512 91, 480 102).
+// 61.6 / 35.3, 100 x 4000 59.7 / 31.2). From 1.4e7 pairs on the eight CTAs of an
+// SM are all busy, and the smallest tile is taken that leaves each one unit: a
+// second unit for some of them costs a whole one (7982 x 2140, 1216 CTAs: 256
+// records, 1125 units 69.2 us, 192, 1500 units 94.7; 4095: 256 records 72 us,
+// 512 91, 480 102; 8947 x 1658 224 records 61.7, 128 70.0).
 int32_t dd_small_j_tile(int64_t n_i, int64_t n_j, int sms) {
   const int64_t rows = (n_i + 63) / 64;
-  const int64_t most = static_cast<double>(n_i) * static_cast<double>(n_j) <= 1.4e7 ? 768 : 256;
-  const int64_t hi = std::min<int64_t>(most, (std::max<int64_t>(n_j, 1) + 31) / 32 * 32);
+  const int64_t hi = std::min<int64_t>(768, (std::max<int64_t>(n_j, 1) + 31) / 32 * 32);
+  if (static_cast<double>(n_i) * static_cast<double>(n_j) > 1.4e7) {
+    int64_t t = 32;
+    while (t < hi && rows * ((n_j + t - 1) / t) > 8 * static_cast<int64_t>(sms)) t += 32;
+    return static_cast<int32_t>(t);
+  }
   int32_t best_t = 32;
   int64_t best = -1;
   for (int64_t t = 32; t <= hi; t += 32) {
