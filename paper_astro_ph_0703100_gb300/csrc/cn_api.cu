@@ -18,6 +18,7 @@
 #include <cstring>
 #include <map>
 #include <mutex>
+#include <optional>
 #include <string>
 #include <tuple>
 #include <vector>
@@ -88,6 +89,13 @@ cn_status fail_cuda(cudaError_t e, const char* what) {
   g_last_error = std::string(what) + ": " + cudaGetErrorString(e);
   return CN_ERR_CUDA;
 }
+
+// A step that a call can do without: what fails in it is no error of the call
+// and leaves the thread's message as it was.
+struct Attempt {
+  std::string kept = g_last_error;
+  ~Attempt() { g_last_error.swap(kept); }
+};
 
 // An NVTX range around each entry point (visible to Nsight tools; a few
 // nanoseconds when no tool is attached).
@@ -1319,6 +1327,7 @@ cn_status force_common(bool dd, int64_t n_i, const float* pos_i, int64_t n_j, co
     // loaded with it.
     if ((st = resolve_plan(dev, variant, n_i, n_j, guard && !eps_i, nullptr, &now.p)) != CN_OK) return st;
     if ((st = single_geometry(dev, *d, variant, guard, now.p, n_i, n_j, &now.g)) != CN_OK) return st;
+    std::optional<Attempt> attempt(std::in_place);
     bool wanted = self && !registered_tune(dev, variant, n_i, n_j, kTunedOneSet);
     const cn::SymForm form = pot ? cn::kSymForcePot : cn::kSymForce;
     if (wanted) wanted = sym_fit(dev, *d, form, n_i, false, sym_default_plan(form, n_i, d->sms), &now.sp) == CN_OK;
@@ -1342,6 +1351,7 @@ cn_status force_common(bool dd, int64_t n_i, const float* pos_i, int64_t n_j, co
     // of these sizes, also one that did without it: a capture may then make
     // a call that has to fall back on it.
     if (!now.sym && !now.rows) {
+      attempt.reset();
       if ((st = launch_workspace(s, now.g, ws, ws_bytes, lib_ws, &now.ctrl, &now.data)) != CN_OK) return st;
     } else if (lib_ws) {
       char *ctrl = nullptr, *data = nullptr;
@@ -1400,6 +1410,7 @@ const SymPlan* sym_self_plan(int dev, const DeviceInfo& d, cn::SymForm form, int
   const uint64_t gen0 = g_plan_gen.load(std::memory_order_acquire);
   if (t_last.key.hit(gen0, dev, form, n, n, false, s)) return &t_last;
   if (registered_tune(dev, variant, n, n, kTunedOneSet)) return nullptr;
+  const Attempt attempt;
   const uint64_t bumps0 = t_own_bumps;
   t_last.key.valid = false;
   if (sym_fit(dev, d, form, n, false, sym_default_plan(form, n, d.sms), &t_last) != CN_OK) return nullptr;
@@ -1602,6 +1613,7 @@ cn_status run_batched(const cn_batch_plan* plan, const float* pos_i, const float
   if (plan->sym_rows > 0) {
     char* slots = nullptr;
     if (!ws) {
+      const Attempt attempt;
       if (sym_workspace(s, plan->sym_bytes, &slots) != CN_OK) slots = nullptr;
     } else if (aligned(ws, 256) && ws_bytes >= std::max(plan->sym_bytes, plan->ws_bytes)) {
       slots = static_cast<char*>(ws);
@@ -1949,7 +1961,10 @@ cn_status build_group_plan(const std::vector<Group>& groups, bool lists, int64_t
   }
   // an ensemble in its default shape: the symmetric form too, where it is
   // expected to be the faster one (a plan without it when its table cannot be had)
-  if (!lists && !guard && tune == &fitted && !tiles.empty()) fit_ensemble(dev, *d, groups, one_sided_s, plan);
+  if (!lists && !guard && tune == &fitted && !tiles.empty()) {
+    const Attempt attempt;
+    fit_ensemble(dev, *d, groups, one_sided_s, plan);
+  }
   *out = plan;
   return CN_OK;
 }
