@@ -256,14 +256,17 @@ cn_status grow(cudaStream_t s, void** buf, size_t* bytes, size_t need, bool zero
     return fail(CN_ERR_WORKSPACE,
                 "the library workspace of this stream must grow, which allocates; not allowed during graph "
                 "capture (make one call before capturing, or pass a workspace)");
-  if (inject("alloc")) return fail(CN_ERR_CUDA, "cudaMalloc: injected allocation failure");
   cudaError_t e;
   if (*buf) {
     if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return fail_cuda(e, "cudaStreamSynchronize");
     cudaFree(*buf);
     *buf = nullptr;
     *bytes = 0;
+    // cached plans hold its address, also when no new one can be had
+    g_plan_gen.fetch_add(1, std::memory_order_acq_rel);
+    ++t_own_bumps;
   }
+  if (inject("alloc")) return fail(CN_ERR_CUDA, "cudaMalloc: injected allocation failure");
   const size_t nb = align_up(std::max(need, static_cast<size_t>(1) << 16), static_cast<size_t>(1) << 16);
   void* p = nullptr;
   if ((e = cudaMalloc(&p, nb)) != cudaSuccess) return fail_cuda(e, what);
@@ -273,7 +276,7 @@ cn_status grow(cudaStream_t s, void** buf, size_t* bytes, size_t need, bool zero
   }
   *buf = p;
   *bytes = nb;
-  g_plan_gen.fetch_add(1, std::memory_order_acq_rel);  // cached plans held the old address
+  g_plan_gen.fetch_add(1, std::memory_order_acq_rel);
   ++t_own_bumps;
   return CN_OK;
 }
