@@ -146,7 +146,18 @@ typedef struct cn_tune {
  * class) takes the kernel of cn_force_symmetric: every unordered pair once,
  * the same accuracy, and its slots in the library workspace. Where those
  * cannot be allocated (memory, or a capture before which no such call was
- * made on the stream) the call takes the one-sided kernel.
+ * made on the stream) the call takes the one-sided kernel. The slots of a
+ * stream take 12 N^2 / B bytes (16 with the potential; tiles of B = 256 .. 2048
+ * particles: 24 MB at N = 32768, 101 MB at 131072, at most 512 MiB) and some MB
+ * of segments; they, and outgrown ones of up to the same size again that a
+ * captured graph may still use, are held until the stream's workspaces are
+ * released. Other calls hold a few MB.
+ * One set on another takes the row kernel (every ordered pair; the
+ * i-particles over the lanes, the j records over the warps; (hi, lo) sums)
+ * where it is the faster one for any masses: on a GB300 from 2.4e7 pairs on up
+ * to 5.5e8 for 128 to 4096 i-particles and up to 1.5e8 for up to 8192, by how the
+ * sets fill the tiles; not with eps2 below normal size or a tune registered.
+ * Sums above the FP32 range come out as infinities.
  */
 CN_API cn_status cn_force(int64_t n_i, const float *pos_i, int64_t n_j, const float *pos_mass_j, float eps2,
                    float *acc_out, float *pot_out, cn_stream stream);
@@ -158,8 +169,9 @@ CN_API cn_status cn_force(int64_t n_i, const float *pos_i, int64_t n_j, const fl
  * cudaMemsetAsync on `stream` before the kernel. No allocation happens
  * inside this call. Calls sharing a workspace must not overlap in time on
  * the device. For one set against itself (see cn_force) the bytes asked for
- * hold the symmetric form's slots; a smaller workspace that is large enough
- * for the one-sided kernel is accepted and takes that kernel. */
+ * hold the symmetric form's slots (for two sets that take the row kernel, its
+ * segments); a smaller workspace that is large enough for the pair kernel is
+ * accepted and takes that kernel. */
 CN_API cn_status cn_force_ws(int64_t n_i, const float *pos_i, int64_t n_j, const float *pos_mass_j, float eps2,
                       float *acc_out, float *pot_out, void *workspace, size_t ws_bytes, cn_stream stream);
 
@@ -190,6 +202,9 @@ CN_API cn_status cn_force_dd_ws(int64_t n_i, const float *pos_i, int64_t n_j, co
 
 /* Workspace bytes that a call of `variant` with these sizes needs under the
  * launch shape currently selected for them (see cn_tune_get). For
+ * CN_VARIANT_F32 / _POT they hold the slots of the symmetric form and the
+ * segments of the row kernel too, where a call takes those; for CN_VARIANT_DD /
+ * _POT they are enough for every call of no more i- and j-particles. For
  * CN_VARIANT_ADJOINT pass n_i = n_j = n. Returns 0 for invalid input. */
 CN_API size_t cn_workspace_bytes(int variant, int64_t n_i, int64_t n_j);
 
@@ -203,9 +218,9 @@ CN_API size_t cn_workspace_bytes(int variant, int64_t n_i, int64_t n_j);
  * the caller.
  *   Arguments, results and errors as cn_force; nothing is allocated.
  *   Scratch: a fixed 32 MiB array in the library's device image. A problem
- *   whose launch shape needs more scratch than that (see
- *   cn_workspace_bytes) is rejected with CN_ERR_WORKSPACE before anything
- *   runs.
+ *   whose pair kernel needs more scratch than that in its launch shape is
+ *   rejected with CN_ERR_WORKSPACE before anything runs; the symmetric and the
+ *   row kernel are taken where the array holds their slots as well.
  *   Set-up: the library's first call of any entry point on a device (this
  *   one or another) sets that device up, which looks up the array's device
  *   address and, under CUDA's lazy module loading, loads the library's
@@ -231,10 +246,13 @@ CN_API cn_status cn_force_noalloc(int64_t n_i, const float *pos_i, int64_t n_j, 
  *                values are on the device). A pair with s = 0 (eps2_i = 0
  *                and coincident points) contributes nothing.
  *   pos_mass_j, acc_out, pot_out, stream: as cn_force.
- * Same kernels and launch shapes as cn_force (tuned under
- * CN_VARIANT_F32_EPS_I / _POT), always with the s = 0 guard; with every
- * eps2_i equal to one value the results are bitwise those of cn_force's
- * one-sided kernel.
+ * Below 2.4e7 pairs, with fewer than 128 i-particles or with a tune
+ * registered under CN_VARIANT_F32_EPS_I / _POT: the pair kernel of cn_force
+ * with the s = 0 guard in every pair; with every eps2_i equal to one value the
+ * results are then bitwise those of cn_force's pair kernel in the same launch
+ * shape. Other calls take the row kernel (see cn_force; up to 4.2e7 pairs only
+ * where it is the faster one), which needs the guard only beside softenings
+ * outside 1e-20 .. 1e24 and agrees with cn_force to FP32 rounding.
  * Errors as cn_force.
  */
 CN_API cn_status cn_force_eps_i(int64_t n_i, const float *pos_eps_i, int64_t n_j, const float *pos_mass_j,
@@ -247,10 +265,11 @@ CN_API cn_status cn_force_eps_i(int64_t n_i, const float *pos_eps_i, int64_t n_j
  * from the other). The paper's kernel evaluates every ordered pair; this one
  * does 14 FP32 lane operations per unordered pair where the masses of a
  * stage are equal and 16 otherwise, against 2 x 12 for the two ordered
- * pairs. The j-side sums of each (row of tiles, block) and the i-side sums of
- * each (CTA, row) segment are merged per particle in (hi, lo) FP32 pairs in a
- * fixed order (bitwise reproducible for a given launch shape); accuracy as
- * cn_force.
+ * pairs (two more where masses, softening and coordinates would take the
+ * mass-free terms out of the FP32 range). The j-side sums of each (row of
+ * tiles, block) and the i-side sums of each (CTA, row) segment are merged per
+ * particle in (hi, lo) FP32 pairs, bands in FP64, in a fixed order (bitwise
+ * reproducible for a given launch shape); accuracy as cn_force.
  * cn_force takes this form by itself for a set against itself above 4096
  * particles; below that the one-sided form is faster.
  *   pos_mass : float[n][4] device records (x, y, z, m), 16-byte aligned
@@ -264,8 +283,8 @@ CN_API cn_status cn_force_eps_i(int64_t n_i, const float *pos_eps_i, int64_t n_j
  * CN_ERR_MISALIGNED, CN_ERR_CUDA (launch), CN_ERR_WORKSPACE (below).
  * Uses a library workspace of j-side slots, 12 N^2 / B bytes (16 with the
  * potential) for tiles of B particles (101 MB at N = 131072 with the default
- * 2048-particle tiles, half of it written), plus the i-side segments (12 or
- * 16 B per particle of a tile per CTA and row), while the slots fit in 512
+ * 2048-particle tiles, half of it written), plus the i-side segments (24 or
+ * 32 B per particle of a tile per CTA and row), while the slots fit in 512
  * MiB; above, the tile rows
  * are processed in bands of w rows (about 12 w N + 24 N bytes, w chosen to
  * fit 512 MiB, or set by the tune's chunk_units), one kernel and one merge
@@ -399,11 +418,12 @@ CN_API cn_status cn_list_plan_capture(cn_batch_plan *plan, const float *pos_i, c
  * of Eq. 1.
  *   pos_mass  : float[n][4]; w : float[n][3] (any 4-byte alignment)
  *   grad_pos  : float[n][3]; grad_mass : float[n] (both written)
- * FP32 pair arithmetic, sums folded by TwoSum every 64 terms. Above 2048
- * particles (on a GB300, eps2 of normal size, no tune registered) each
- * unordered pair is evaluated once, as in cn_force_symmetric, with its slots
- * in the library workspace; where those cannot be allocated, and below, every
- * ordered pair is, with an FP64 merge of split tiles.
+ * FP32 pair arithmetic. Above 2048 particles (on a GB300, eps2 of normal
+ * size, no tune registered) each unordered pair is evaluated once, as in
+ * cn_force_symmetric, sums folded by TwoSum every 32 terms, with its slots in
+ * the library workspace; where those cannot be allocated, and below, every
+ * ordered pair is, sums folded every 64 terms, with an FP64 merge of split
+ * tiles.
  */
 CN_API cn_status cn_force_adjoint(int64_t n, const float *pos_mass, float eps2, const float *w, float *grad_pos,
                            float *grad_mass, cn_stream stream);

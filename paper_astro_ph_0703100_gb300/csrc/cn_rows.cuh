@@ -28,7 +28,10 @@
 // in CTA order. Register sums are folded into (hi, lo) sums by TwoSum every
 // kRowFold records: 128 cost 1% at 2048 x 262144 (208 / 211 us) and keep the
 // error below the pair kernel's (8192 x 8192 1.0e-7 of 1.1e-7, 1.3e-7 with 512;
-// 2048 x 262144 3.7e-8 of 5.1e-8). Deterministic, no atomics on data.
+// 2048 x 262144 3.7e-8 of 5.1e-8). Where each warp has particles of its own
+// (large sets with per-particle softening) it is every stage of 256: 0.71 of the
+// pair kernel's error (24000 to 65536, geometric mean over 36 sets), and 128 cost 4%
+// there (65536 x 65536 1499 / 1563 us). Deterministic, no atomics on data.
 #pragma once
 
 #include "cn_device.cuh"
@@ -36,7 +39,7 @@
 
 namespace cn {
 
-constexpr int kRowFold = 128;        // j records summed in FP32 registers between TwoSum folds (two of a stage)
+constexpr int kRowFold = 128;        // j records summed in FP32 registers between TwoSum folds; a warp's share of a stage, if more
 constexpr int kRowUnit = 16;         // records per loop trip (divides 32)
 constexpr int kRowWarps = 8;
 constexpr int kRowThreads = 32 * kRowWarps;
@@ -205,7 +208,7 @@ __global__ void __launch_bounds__(kRowThreads, 2) rows_kernel(const __grid_const
   int32_t row = -1;
   const float2 e2 = row_dup(a.eps2);
   float scale = 1.f;  // of the sums in registers
-  int held = 0;       // j records in them, about
+  int held = 0;       // j records in them
   float cap = -1.f;   // masses that may factor out with the warp's particles, up to (none: -1)
   float* const mine = sums + warp * kPer + lane;  // the thread's sums: mine[c * kAll + 32 k]
 

@@ -15,7 +15,7 @@
 // this takes 24 shuffles and 24 additions per 8 records to 48 shuffles and
 // none, which leaves the FP32 pipe to the pair terms (inner loop at K = 8 x
 // 256 threads, 2.07 GHz: 1.93e12 -> 2.03e12 unordered pairs/s; whole calls at
-// N = 131072 with equal masses: 4653 -> 4015 us).
+// N = 131072 with equal masses: 4653 -> 3985 us).
 //
 // What bounds the loop: the FP32 pipe, and with it the register file. A
 // packed multiply-add whose three operands are different registers issues
@@ -40,10 +40,10 @@
 // Shared memory per CTA: a ring of staged chunks (bulk copies), three buffers
 // of the j-side sums of a chunk, one row per warp, and the i-side (hi, lo)
 // sums of the current row of tiles, folded from registers every kFold
-// records by TwoSum (force: 512 are 0.4% faster at N = 131072 and 0.8% at 50001,
-// but leave a larger error than the reduce-scatter form did: with the potential
-// 4.8e-8 against 4.1e-8 at 9836, 256 4.0e-8). The warps are not held together by a barrier: a warp
-// that has swept chunk k waits for the "done" barrier of chunk k - 1 (long
+// records by TwoSum, mid-size sets sooner (force: 512 are 0.4% faster at N =
+// 131072 and 0.8% at 50001, but leave a larger error than the reduce-scatter form
+// did: with the potential 4.8e-8 against 4.1e-8 at 9836, 256 4.0e-8). The warps
+// are not held together by a barrier: a warp that has swept chunk k waits for the "done" barrier of chunk k - 1 (long
 // complete unless a warp is a whole chunk behind), adds up its share of
 // chunk k - 1's rows and arrives on chunk k's barrier. A __syncthreads per
 // chunk instead cost 1.4 us per chunk (N = 131072, 64-record chunks).
@@ -53,8 +53,8 @@
 // adds them per particle in a fixed order: the result is deterministic,
 // with no atomics on data. A part of more than 1024 records is the sum of
 // several register chains; in the force forms its segment then keeps the low
-// words as well (131072 4003 / 4009 us, all segments at all sizes: 4096 .. 24576
-// 2 to 7% slower, for words that are zero while a segment is one chain).
+// words as well (all segments at all sizes: 4096 .. 24576 2 to 7% slower, for words
+// that are zero while a segment is one chain).
 #pragma once
 
 #include "cn_device.cuh"

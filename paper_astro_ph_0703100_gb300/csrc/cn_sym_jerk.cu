@@ -13,8 +13,10 @@ namespace {
 // ordered pairs. What bounds it: as the force form, with 12 to 14 of the 31
 // to 34 packed operations reading three registers, and 14 shuffles per step;
 // all the registers of one CTA per SM (up to 255 per thread) go to four or
-// eight particles per thread. Sums folded every 256 records keep the error
-// below the one-sided kernel's (512: 6.8e-8 against 5.5e-8 at N = 8192).
+// eight particles per thread. Sums are folded every 256 records, 128 at sizes
+// where the one-sided kernel's chains are as short (512: 6.8e-8 against 5.5e-8
+// at N = 8192). Steps per trip and the flush's form as measured for K = 8 (65536,
+// 4 / 8 steps, rolled / not: 2267 .. 2330 us, with the potential 2543 .. 2609).
 template <int K_, bool POT>
 struct SymJerkPolicy {
   static constexpr int K = K_;
