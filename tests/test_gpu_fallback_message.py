@@ -1,6 +1,7 @@
 """A call that succeeds without a step it can do without (slots of the symmetric
 form, segments of the row kernel) leaves no error message behind."""
 
+import ctypes
 import threading
 
 import numpy as np
@@ -10,6 +11,13 @@ from gpu_common import dev_tensor, lib, torch_cuda
 from paper_astro_ph_0703100_gb300 import synth
 
 pytestmark = pytest.mark.gpu
+
+
+def _own_stream(torch):
+    """A stream of its own, which no other test has used: PyTorch's come from a small pool."""
+    handle = ctypes.c_uint64(0)
+    assert int(torch.cuda.cudart().cudaStreamCreate(ctypes.addressof(handle))) == 0
+    return torch.cuda.ExternalStream(handle.value)
 
 
 @pytest.mark.parametrize("fault", ["alloc", "capture"])
@@ -26,7 +34,7 @@ def test_no_message_after_a_fallback(monkeypatch, form, fault):
     got = []
 
     def work():  # a thread of its own has no earlier message
-        s = torch.cuda.Stream()
+        s = _own_stream(torch)
         with torch.cuda.stream(s):
             cn.cn_force_eps_i(j, j[:500].contiguous())  # the one-sided workspaces alone
             wide.run(d)
